@@ -354,8 +354,35 @@ __device__ __forceinline__ int add_acquire(int* p, int v)
     return old;
 }
 
+// One axis of a box as the traversal reads it: centre and half extent.  h
+// covers both sides exactly (rounded up), times 1 + 8 u (u = 2^-24): the slab
+// test (pt.cu) forms (c - o) inv -+ h |inv|, whose rounding is at most
+// 3 u |t| + 2 u h |inv| per side, so its interval holds the box's
+__device__ __forceinline__ void centre_half(float lo, float hi, float& c, float& h)
+{
+    c = 0.5f * lo + 0.5f * hi;
+    h = __fmul_ru(fmaxf(__fsub_ru(hi, c), __fsub_ru(c, lo)), 1.0000005f);
+}
+// the 64-byte traversal node: per axis the two children's centres, then per
+// axis their half extents, then the child ids
+__device__ __forceinline__ void write_node(float4* __restrict__ nodes, int id, const float* L,
+                                           const float* R, int l, int r)
+{
+    float c[6], h[6];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        centre_half(L[a], L[3 + a], c[2 * a], h[2 * a]);
+        centre_half(R[a], R[3 + a], c[2 * a + 1], h[2 * a + 1]);
+    }
+    float4* nd = nodes + 4 * (size_t)id;
+    nd[0] = make_float4(c[0], c[1], c[2], c[3]);
+    nd[1] = make_float4(c[4], c[5], h[0], h[1]);
+    nd[2] = make_float4(h[2], h[3], h[4], h[5]);
+    nd[3] = make_float4(__int_as_float(l), __int_as_float(r), 0.0f, 0.0f);
+}
+
 // bottom-up refit: the second child to arrive at a parent computes its box
-// and writes the 64-byte traversal node (both child boxes + child ids)
+// and writes the traversal node
 __global__ void k_refit(int n, const int* __restrict__ left, const int* __restrict__ right,
                         const int* __restrict__ parent, float* box, int* visit,
                         float4* __restrict__ nodes)
@@ -379,10 +406,7 @@ __global__ void k_refit(int n, const int* __restrict__ left, const int* __restri
             b[a] = fminf(L[a], R[a]);
             b[3 + a] = fmaxf(L[3 + a], R[3 + a]);
         }
-        nodes[4 * node + 0] = make_float4(L[0], L[1], L[2], L[3]);
-        nodes[4 * node + 1] = make_float4(L[4], L[5], R[0], R[1]);
-        nodes[4 * node + 2] = make_float4(R[2], R[3], R[4], R[5]);
-        nodes[4 * node + 3] = make_float4(__int_as_float(l), __int_as_float(r), 0.0f, 0.0f);
+        write_node(nodes, node, L, R, l, r);
         node = parent[node];
     }
 }
@@ -444,10 +468,8 @@ __device__ __forceinline__ void ploc_write_node(int id, int ca, float4 a0, float
                                                 float4 b0, float4 b1, float4* __restrict__ nodes,
                                                 float* __restrict__ box, float4& u0, float4& u1)
 {
-    nodes[4 * id + 0] = make_float4(a0.x, a0.y, a0.z, a0.w);
-    nodes[4 * id + 1] = make_float4(a1.x, a1.y, b0.x, b0.y);
-    nodes[4 * id + 2] = make_float4(b0.z, b0.w, b1.x, b1.y);
-    nodes[4 * id + 3] = make_float4(__int_as_float(ca), __int_as_float(cb), 0.0f, 0.0f);
+    const float L[6] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y}, R[6] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y};
+    write_node(nodes, id, L, R, ca, cb);
     u0 = make_float4(fminf(a0.x, b0.x), fminf(a0.y, b0.y), fminf(a0.z, b0.z), fmaxf(a0.w, b0.w));
     u1 = make_float4(fmaxf(a1.x, b1.x), fmaxf(a1.y, b1.y), 0.0f, 0.0f);
     float* bx = box + (size_t)id * 6;
@@ -1674,7 +1696,16 @@ extern "C" mrs_status mrs_scene_export_nodes(mrs_scene S, float* nodes, int64_t 
     MRS_CHECK(cudaDeviceSynchronize());
     if (nodes && ns > 1) {
         MRS_ARG(n_floats >= 16 * (int64_t)(ns - 1), "n_floats must be >= 16 (ns - 1)");
+        // child ids from the traversal nodes, the children's exact boxes from the box array
         MRS_CHECK(cudaMemcpy(nodes, S->nodes, sizeof(float4) * 4 * (size_t)(ns - 1), cudaMemcpyDeviceToHost));
+        std::vector<float> box((2 * (size_t)ns - 1) * 6);
+        MRS_CHECK(cudaMemcpy(box.data(), S->box, box.size() * sizeof(float), cudaMemcpyDeviceToHost));
+        for (int i = 0; i < ns - 1; ++i) {
+            float* nd = nodes + 16 * (size_t)i;
+            int32_t id[2];
+            memcpy(id, nd + 12, sizeof(id));
+            for (int c = 0; c < 2; ++c) memcpy(nd + 6 * c, box.data() + 6 * (size_t)id[c], 6 * sizeof(float));
+        }
     }
     if (order && ns > 0)
         MRS_CHECK(cudaMemcpy(order, S->order, sizeof(int) * (size_t)ns, cudaMemcpyDeviceToHost));
