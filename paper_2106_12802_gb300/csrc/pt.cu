@@ -103,6 +103,7 @@ struct SceneView {
     int n, ns, n_lights;   // triangles; of them in the LBVH (positions 0..ns-1); lights
     const float4* __restrict__ nodes;
     const float4* __restrict__ tris;
+    const float* __restrict__ leaf_box;   // [ns][6] lo, hi of the leaves' boxes
     const int2* __restrict__ tri_ml;
     const float* __restrict__ mats;
     const float* __restrict__ lights;
@@ -162,6 +163,26 @@ __device__ __noinline__ V3 reciprocal_zero(const float4* __restrict__ nodes, V3 
     if (d.y == 0.0f) inv.y = copysignf(1e36f / fmaxf(my, 1.0f), d.y);
     if (d.z == 0.0f) inv.z = copysignf(1e36f / fmaxf(mz, 1.0f), d.z);
     return inv;
+}
+
+// The plain slab test of leaf k's exact box.  The triangle test's rounding can
+// put a grazing hit just outside the triangle's box; such a hit does not count,
+// whatever the tree above the leaf lets through (the boxes tested there are
+// slightly larger).  Only a triangle that was hit gets here, about once per ray.
+// inv: the traversal's reciprocals (infinite here where d is zero).
+__device__ __forceinline__ bool in_leaf_box(const float* __restrict__ box, V3 o, V3 d, V3 inv, float tmax)
+{
+    const float2* p = (const float2*)box;
+    const float2 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);   // lo.xy | lo.z hi.x | hi.yz
+    if (d.x == 0.0f) inv.x = copysignf(INFINITY, d.x);
+    if (d.y == 0.0f) inv.y = copysignf(INFINITY, d.y);
+    if (d.z == 0.0f) inv.z = copysignf(INFINITY, d.z);
+    const float t0x = (a.x - o.x) * inv.x, t1x = (b.y - o.x) * inv.x;
+    const float t0y = (a.y - o.y) * inv.y, t1y = (c.x - o.y) * inv.y;
+    const float t0z = (b.x - o.z) * inv.z, t1z = (c.y - o.z) * inv.z;
+    const float tn = fmaxf(fmaxf(fminf(t0x, t1x), fminf(t0y, t1y)), fmaxf(fminf(t0z, t1z), 0.0f));
+    const float tf = fminf(fminf(fmaxf(t0x, t1x), fmaxf(t0y, t1y)), fminf(fmaxf(t0z, t1z), tmax));
+    return tn <= tf * 1.0000005f;
 }
 
 // closest hit (ties to the smaller triangle index) or any hit below tmax
@@ -225,9 +246,12 @@ __device__ int traverse(const SceneView& S, V3 o, V3 d, float tmax, float& t_out
             int k = node - (n - 1), prim;
             if (kCount) ++*ntest;
             float t = intersect(o, d, S.tris + 3 * k, kAny ? tmax : T_INF, prim);
-            if (t > 0.0f) {
+            if (t > 0.0f && (kAny || t < bt || (t == bt && prim < best_prim)) &&
+                in_leaf_box(S.leaf_box + 6 * (size_t)k, o, d, inv, kAny ? tmax : T_INF)) {
                 if (kAny) { t_out = t; return k; }
-                if (t < bt || (t == bt && prim < best_prim)) { bt = t; best = k; best_prim = prim; }
+                bt = t;
+                best = k;
+                best_prim = prim;
             }
         }
         if (sp == 0) break;
@@ -971,7 +995,8 @@ __global__ void k_philox(const uint32_t* triples, int n, uint2 key, float* out)
 
 SceneView view(const mrs_scene_s* S)
 {
-    return SceneView{S->n, S->ns, S->n_lights, S->nodes, S->tris, S->tri_ml, S->mats, S->lights};
+    return SceneView{S->n, S->ns, S->n_lights, S->nodes, S->tris,
+                     S->box + 6 * (size_t)(S->ns > 0 ? S->ns - 1 : 0), S->tri_ml, S->mats, S->lights};
 }
 
 // persistent grid of the tail kernel: as many blocks as fit on the GPU at once
