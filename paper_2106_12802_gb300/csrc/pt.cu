@@ -709,9 +709,14 @@ __device__ __forceinline__ void shadow_body(const WaveParams& w, const Jobs& job
 // wavefront kernels (trace, shade, shadow; a path's state lives in P), so
 // its radiance is bit-identical; the per-bounce counts are the same numbers,
 // gathered per block in shared memory.  cnt[kWorkSlot] hands out the paths.
-// 32 registers and 8 blocks per SM, as the traversal kernels: with 64
-// registers (4 blocks) the tail ran 2-7% slower despite no spills.
+// A warp takes `width` paths at a time: all 32 lanes when there are paths
+// enough for every warp of the persistent grid, else only its share (down to
+// one), because lanes on different paths wait for one another at every
+// divergent step and a small wave is bound by that latency, not by issue slots
+// (48 x 48 @ 1 spp: 0.230 -> 0.128 ms on the Cornell box, 0.323 -> 0.159 ms on
+// the 200k-triangle scene; 160 x 120 @ 1: 0.274 -> 0.197, 0.337 -> 0.206).
 constexpr int kWorkSlot = 63;
+constexpr int64_t kTailSmall = 640 * 1024, kTailMedium = 2 * 1024 * 1024;   // see tail_plan
 template <bool kCount, class Jobs>
 __device__ __forceinline__ void tail_body(const WaveParams& w, const Jobs& jobs, int b0,
                                           int max_depth)
@@ -724,11 +729,13 @@ __device__ __forceinline__ void tail_body(const WaveParams& w, const Jobs& jobs,
     const int count = (int)*(volatile uint32_t*)&w.cnt[b0];
     const int* q = (b0 & 1) ? P.q1 : P.q0;
     const int lane = threadIdx.x & 31;
+    const int warps = (int)(gridDim.x * (blockDim.x / 32));
+    const int width = min(32, (count + warps - 1) / warps);
     int p = -1, b = b0;
     bool drained = false;   // warp-uniform: the queue has been handed out
     for (;;) {
         // refill: lanes without a path take consecutive queue slots
-        const bool want = p < 0;
+        const bool want = p < 0 && lane < width;
         const unsigned m = __ballot_sync(0xffffffffu, want);
         if (m && !drained) {
             const int leader = __ffs(m) - 1;
@@ -816,12 +823,13 @@ __global__ void __launch_bounds__(kThreads, 8)
 {
     shadow_body<false>(w, ManyJobs{T}, b);
 }
-template <bool kCount>
-__global__ void __launch_bounds__(kThreads, 8) k_tail(const __grid_constant__ WaveParams w, int b0)
+template <bool kCount, int kBlocks>
+__global__ void __launch_bounds__(kThreads, kBlocks) k_tail(const __grid_constant__ WaveParams w, int b0)
 {
     tail_body<kCount>(w, OneJob{w.J}, b0, w.J.max_depth);
 }
-__global__ void __launch_bounds__(kThreads, 8)
+template <int kBlocks>
+__global__ void __launch_bounds__(kThreads, kBlocks)
     k_tail_b(const __grid_constant__ WaveParams w, const __grid_constant__ JobTable T, int b0,
              int max_depth)
 {
@@ -999,31 +1007,49 @@ SceneView view(const mrs_scene_s* S)
                      S->box + 6 * (size_t)(S->ns > 0 ? S->ns - 1 : 0), S->tri_ml, S->mats, S->lights};
 }
 
-// persistent grid of the tail kernel: as many blocks as fit on the GPU at once
-int tail_grid(bool counting)
+// How a wave of n paths runs its tail (results do not depend on it).  Up to
+// about 2M paths the render is bound by the latency of its paths' steps: fewer
+// blocks per SM with registers enough for no spills (64 at 4 blocks, 48 at 5)
+// beat more warps, and starting in the tail saves the wait for each wavefront
+// step's slowest ray.  Above that issue slots bound it: 8 blocks (32
+// registers), and bounce 0, whose rays are coherent, as wavefront steps (also
+// better for two renders side by side).  ms, 8 blocks from bounce 1 -> this
+// rule: Cornell box 333 x 217 @ 6 spp (434k paths) 0.75 -> 0.57, 512^2 @ 4
+// (1.0M) 1.29 -> 1.12, 700^2 @ 4 (2.0M) 2.07 -> 1.92; 200k-triangle scene 0.83
+// -> 0.55, 1.26 -> 0.97, 1.88 -> 1.60.  4 against 5 blocks: 434k paths 0.562 /
+// 0.600, 1.0M 1.003 / 0.991, 2.1M 1.791 / 1.716; 5 against 8: 2.1M 1.716 /
+// 1.690, 4.2M 3.22 / 3.10.  Bounce 0 against 1 at 4.2M: Cornell 3.92 / 3.81.
+struct TailPlan {
+    int bounce;   // first bounce in the tail kernel
+    int blocks;   // blocks per SM of the instantiation
+};
+TailPlan tail_plan(int64_t n, int32_t asked)
 {
-    static int g[2] = {0, 0};
-    int& v = g[counting ? 1 : 0];
-    if (!v) {
-        int per_sm = 0;
-        if (counting)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tail<true>, kThreads, 0);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tail<false>, kThreads, 0);
-        v = sm_count() * (per_sm < 1 ? 1 : per_sm);
-    }
-    return v;
+    TailPlan t;
+    t.blocks = n <= kTailSmall ? 4 : n <= kTailMedium ? 5 : 8;
+    t.bounce = asked >= 0 ? asked : n <= kTailMedium ? 0 : 1;
+    return t;
 }
 
-int tail_grid_batch()
+// the persistent grid: as many blocks as fit on the GPU at once
+template <class K> int persistent_grid(K kernel)
 {
-    static int v = 0;
-    if (!v) {
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tail_b, kThreads, 0);
-        v = sm_count() * (per_sm < 1 ? 1 : per_sm);
-    }
-    return v;
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0);
+    return sm_count() * (per_sm < 1 ? 1 : per_sm);
+}
+template <bool kCount, int kBlocks> void launch_tail(const WaveParams& w, int b0, cudaStream_t st)
+{
+    static const int g = persistent_grid(k_tail<kCount, kBlocks>);
+    MRS_TIMED(PK_TAIL, st, (k_tail<kCount, kBlocks><<<g, kThreads, 0, st>>>(w, b0)));
+    MRS_LAUNCHED(1);
+}
+template <int kBlocks>
+void launch_tail_b(const WaveParams& w, const JobTable& T, int b0, int max_depth, cudaStream_t st)
+{
+    static const int g = persistent_grid(k_tail_b<kBlocks>);
+    MRS_TIMED(PK_TAIL, st, (k_tail_b<kBlocks><<<g, kThreads, 0, st>>>(w, T, b0, max_depth)));
+    MRS_LAUNCHED(1);
 }
 
 inline int grid_for(int64_t n)
@@ -1131,11 +1157,8 @@ static mrs_status render_impl(mrs_scene S, Buf& arena, int64_t wave_paths, int32
         int g = grid_for(w.n_paths);
         MRS_TIMED(PK_RAYGEN, st, k_raygen<<<g, kThreads, 0, st>>>(w));
         MRS_LAUNCHED(1);
-        // first bounce of the tail kernel: by default bounce 1 (on the 200k-
-        // triangle scene at 1024^2, 4 and 16 spp, with and without roulette,
-        // and 256^2 at 64 spp, tails from bounce 0-3 beat the wavefront alone;
-        // from bounce 1 by 3-5% more than from bounce 2, the next best)
-        const int b_tail = tail >= 0 ? tail : 1;
+        const TailPlan plan = tail_plan(w.n_paths, tail);
+        const int b_tail = plan.bounce;
         for (int b = 0; b <= max_depth && b < b_tail; ++b) {
             if (stats) MRS_TIMED(PK_TRACE, st, k_trace<true><<<g, kThreads, 0, st>>>(w, b));
             else MRS_TIMED(PK_TRACE, st, k_trace<false><<<g, kThreads, 0, st>>>(w, b));
@@ -1147,10 +1170,10 @@ static mrs_status render_impl(mrs_scene S, Buf& arena, int64_t wave_paths, int32
             MRS_LAUNCHED(1);
         }
         if (b_tail <= max_depth) {
-            const int gt = tail_grid(stats != nullptr);
-            if (stats) MRS_TIMED(PK_TAIL, st, k_tail<true><<<gt, kThreads, 0, st>>>(w, b_tail));
-            else MRS_TIMED(PK_TAIL, st, k_tail<false><<<gt, kThreads, 0, st>>>(w, b_tail));
-            MRS_LAUNCHED(1);
+            if (stats) launch_tail<true, 8>(w, b_tail, st);
+            else if (plan.blocks == 8) launch_tail<false, 8>(w, b_tail, st);
+            else if (plan.blocks == 5) launch_tail<false, 5>(w, b_tail, st);
+            else launch_tail<false, 4>(w, b_tail, st);
         }
         // 16-byte sample loads when every pixel's run of kk samples starts on
         // a 16-byte boundary (the arrays are 256-byte aligned)
@@ -1375,8 +1398,6 @@ mrs_status render_batch_impl(mrs_ctx ctx, const mrs_render_job* jobs, int32_t n_
         v.key = make_uint2((uint32_t)J.seed, (uint32_t)(J.seed >> 32));
         return v;
     };
-    const int32_t tail = ctx->tail_bounce;
-    const int b_tail = tail >= 0 ? tail : 1;
     for (const auto& wv : waves) {
         JobTable T;
         memset(&T, 0, sizeof(T));
@@ -1398,6 +1419,8 @@ mrs_status render_batch_impl(mrs_ctx ctx, const mrs_render_job* jobs, int32_t n_
         w.scnt = scnt;
         w.stats = nullptr;
         MRS_CHECK(cudaMemsetAsync(cnt, 0, 4 * 2 * 64, st));
+        const TailPlan plan = tail_plan(off, ctx->tail_bounce);
+        const int b_tail = plan.bounce;
         const int g = grid_for(off);
         MRS_TIMED(PK_RAYGEN, st, k_raygen_b<<<g, kThreads, 0, st>>>(w, T));
         MRS_LAUNCHED(1);
@@ -1408,8 +1431,9 @@ mrs_status render_batch_impl(mrs_ctx ctx, const mrs_render_job* jobs, int32_t n_
             MRS_LAUNCHED(3);
         }
         if (b_tail <= maxd) {
-            MRS_TIMED(PK_TAIL, st, k_tail_b<<<tail_grid_batch(), kThreads, 0, st>>>(w, T, b_tail, maxd));
-            MRS_LAUNCHED(1);
+            if (plan.blocks == 8) launch_tail_b<8>(w, T, b_tail, maxd, st);
+            else if (plan.blocks == 5) launch_tail_b<5>(w, T, b_tail, maxd, st);
+            else launch_tail_b<4>(w, T, b_tail, maxd, st);
         }
         // each chunk's samples into its job's accumulator, in sample order
         for (size_t c = wv.first; c < wv.second; ++c) {

@@ -81,3 +81,18 @@ def test_zero_direction_components_and_flat_boxes(mrs, orc, kind, n, shift):
         assert np.array_equal(p.cpu().numpy()[clear], pb[clear])
         assert np.array_equal(t.cpu().numpy()[clear], tb[clear])
 
+
+# around the sizes where the tail kernel's launch changes: one path per warp,
+# less than a warp's lanes, 640k and 2M paths in the wave, and several waves
+@pytest.mark.parametrize("W,H,spp,wave", [(1, 1, 1, None), (7, 5, 3, None), (97, 61, 2, None), (331, 97, 5, None),
+                                          (512, 320, 4, None), (641, 256, 4, None), (1024, 512, 4, None),
+                                          (1025, 512, 4, None), (257, 129, 6, 40000)])
+def test_render_does_not_depend_on_the_tail_launch(mrs, W, H, spp, wave):
+    sc = mrs.Scene.seeded(3, n_spheres=12, n_large=3)
+    if wave:
+        sc.set_wave(wave)
+    a = mrs.render(sc, W, H, spp, 6, 2, seed=5, layers=True)
+    sc.set_tail(40)       # no tail kernel: one launch per step
+    b = mrs.render(sc, W, H, spp, 6, 2, seed=5, layers=True)
+    for k in b:
+        assert torch.equal(a[k], b[k]), k
