@@ -703,7 +703,7 @@ mrs_status mrs_rdn_check(mrs_rdn rdn);
  * MRS_ERR_TIMEOUT if a BF16 step's tensor-core wait gave up).  The first step
  * allocates the gradient and Adam moments (3 x n_params floats, moments
  * zero); the workspace (FP32: about 20 KB per LR pixel plus 1.3 KB per HR
- * pixel; BF16: about 11 KB per LR pixel plus 0.8 KB per HR pixel) lives in
+ * pixel; BF16: about 19 KB per LR pixel plus 1 KB per HR pixel) lives in
  * the handle.  A later MRS_PREC_BF16 mrs_rdn_fuse repacks its BF16 weights
  * from the updated FP32 ones.  A BF16 step copies the batch into the
  * handle's staging buffers; the first step of a shape (N, H, W, loss, beta)

@@ -29,7 +29,11 @@
 #include <cuda_fp8.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
+#include <queue>
+#include <utility>
+#include <vector>
 
 #include "conv_tc.cuh"
 
@@ -151,21 +155,22 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, int row_bytes)
     return d;
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc,
+// executed by the lane whose `leader` is set
+__device__ __forceinline__ void mma_f16(bool leader, uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc,
                                         uint32_t accum)
 {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accum));
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(accum), "r"((uint32_t)leader));
 }
-__device__ __forceinline__ void mma_f8(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc,
+__device__ __forceinline__ void mma_f8(bool leader, uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc,
                                        uint32_t accum)
 {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accum));
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(accum), "r"((uint32_t)leader));
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar)
 {
@@ -540,8 +545,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 for (int kk = 0; kk < KSTEPS; ++kk) {
                                     const uint64_t ad = arow + (uint64_t)((dx * ROWB + kk * 32) >> 4);
                                     const uint64_t bd = brow0 + (uint64_t)((dx * BROWS * ROWB + kk * 32) >> 4);
-                                    if (OPER == TC_BF16) mma_f16(tmem + dcol, ad, bd, idesc, 1u);
-                                    else mma_f8(tmem + dcol, ad, bd, idesc, 1u);
+                                    if (OPER == TC_BF16) mma_f16(true, tmem + dcol, ad, bd, idesc, 1u);
+                                    else mma_f8(true, tmem + dcol, ad, bd, idesc, 1u);
                                 }
                             }
                         }
@@ -790,7 +795,7 @@ mrs_status tc_make_act_map(CUtensorMap* m, const void* ptr, int N, int H, int W,
 
 mrs_status tc_make_view_map(CUtensorMap* m, const void* ptr, int N, int H, int W,
                             long long px_stride, long long row_stride, long long img_stride,
-                            int box_px)
+                            int box_px, int box_rows)
 {
     auto fn = encode_fn();
     if (!fn) { set_error("cuTensorMapEncodeTiled unavailable"); return MRS_ERR_CUDA; }
@@ -800,7 +805,7 @@ mrs_status tc_make_view_map(CUtensorMap* m, const void* ptr, int N, int H, int W
     }
     cuuint64_t dims[4] = {64, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
     cuuint64_t strides[3] = {(cuuint64_t)px_stride, (cuuint64_t)row_stride, (cuuint64_t)img_stride};
-    cuuint32_t box[4] = {64, (cuuint32_t)box_px, 1, 1};
+    cuuint32_t box[4] = {64, (cuuint32_t)box_px, (cuuint32_t)box_rows, 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides,
                     box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -885,24 +890,47 @@ mrs_status tc_conv3x3(const TcConvArgs& a, cudaStream_t st)
 // apart.  M = 128 is made of two 64-channel MN atoms LBO bytes apart, so one
 // MMA covers two taps:
 //   MMA dx     (dx = 0..2): rows 0-63 tap (ky 0, dx), rows 64-127 tap (ky 1, dx)
-//                           (input rows y-1 and y sit in slots RB bytes apart)
+//                           (input rows y-1 and y lie one box row apart)
 //   MMA 3 + dx            : rows 0-63 tap (ky 2, dx), rows 64-127 read a
 //                           region of ones, which makes those rows db[o]
 // A job is kWgKB output pixels of one image row.  Per job the producer loads
-// input rows y-1, y, y+1 (kWgKB + 2 pixels from x0 - 1, zero-filled outside
-// the image: the zero padding) and dy row y (kWgKB pixels); the kx shift is a
-// descriptor start offset of kx 128-byte rows.  Each CTA takes a contiguous
-// run of jobs, accumulates all 9 taps in TMEM (6 x 64 fp32 columns) and writes
-// one partial; the partials are summed by a separate reduction.
-// Warp 0 lane 0: TMA producer; warp 1: TMEM allocator, lane 0 MMA issuer;
-// warps 0-3: epilogue (warp w reads TMEM lanes 32w .. 32w + 31).
+// input rows y-1, y, y+1 (kWgKB + 2 pixels from x0 - 1, one TMA box, zero-filled
+// outside the image: the zero padding) and dy row y (kWgKB pixels); the kx shift
+// is a descriptor start offset of kx 128-byte rows.  MMAs into different D
+// regions do not pipeline, so a job issues one MMA's four K steps after the
+// other; K steps wholly outside the image are left out.
+// The accumulators of a run (6 x 64 FP32 columns) go to the epilogue's
+// registers, which add up the runs of one class: an earlier form wrote every
+// run's 147 KB as a partial sum, 178 launches and 10,400 partials for a step of
+// the two-encoder network, whose writing, re-reading and launch gaps cost
+// several times the MMAs.  A (tile, class) pair is the unit of work, or one
+// half of it (MMAs 0-2 or 3-5) where the whole would outlast an even share of
+// all work; the host deals the units to the CTAs, largest first.
+// Warps (16): 2 TMA producer, 3 MMA issuer (lane 0), 7 TMEM allocator, the
+// others epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31; lanes 0-63 have
+// 384 useful columns (4 warps x 96), lanes 64-127 192 (2 x 96) and the bias
+// row's 64 (warp 6).
 namespace {
 
-constexpr int kWgThreads = 128;
-constexpr int kWgRB = ((kWgKB + 2) * 128 + 1023) & ~1023;   // one input-row slot
-constexpr int kWgBB = kWgKB * 128;                           // dy slot
-constexpr int kWgStage = 3 * kWgRB + kWgBB;
-constexpr uint32_t kWgTx = 3 * (kWgKB + 2) * 128 + kWgKB * 128;   // bytes landed per job
+constexpr int kWgThreads = 512;
+constexpr int kWgXRow = (kWgKB + 2) * 128;                   // bytes of one input row of a job
+constexpr int kWgXBytes = 3 * kWgXRow;
+constexpr int kWgYBytes = kWgKB * 128;
+constexpr int kWgYOff = (kWgXBytes + 1023) & ~1023;
+constexpr int kWgStage = kWgYOff + kWgYBytes;
+constexpr int kWgStages = 6;
+constexpr int kWgOnes = (kWgXRow + 1023) & ~1023;
+constexpr size_t kWgSmem = 1024 + (size_t)kWgStages * kWgStage + kWgOnes + 8 * (2 * kWgStages + 2) + 16;
+static_assert(kWgSmem <= 227 * 1024, "wgrad shared memory");
+// kind::f16, D f32, A and B bf16, both MN-major, N = 64, M = 128
+constexpr uint32_t kWgIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                              ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+
+struct alignas(64) WgDesc {
+    CUtensorMap x, dy;
+    int njobs, runs, H, W, XS, cin, cout;
+};
+struct WgUnit { int tile, w, half; };   // half: 0 MMAs 0-5, 1 MMAs 0-2, 2 MMAs 3-5
 
 // MN-major SWIZZLE_128B descriptor: `lbo` = bytes to the next 64-element MN
 // atom, SBO = 1024 bytes to the next group of 8 K rows
@@ -925,37 +953,69 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity, long 
         if (clock64() - t0 > limit_cycles) return;
 }
 
-__global__ void __launch_bounds__(kWgThreads, 1)
-    k_wgrad_tc(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_dy,
-               TcWgradArgs a, int stages)
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
 {
-    // kind::f16, D f32, A and B bf16, both MN-major, N = 64, M = 128
-    constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                               ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
+// first job of run g
+__device__ __forceinline__ int wg_run(const WgDesc& d, int g) { return (int)((long long)d.njobs * g / d.runs); }
+
+// MMAs QA .. QB - 1 of a job: a01 / a2 are the A descriptors of MMAs 0 and 3
+// (one 128-byte row further per dx), bd the B descriptor; ks K steps of 16
+// pixels, each 2048 bytes (+ 128 in the start-address field, bits 0-13;
+// shared-memory addresses stay far below the field's 256 KB) into every operand
+template <int QA, int QB>
+__device__ __forceinline__ void wg_issue(uint32_t tmem, uint64_t a01, uint64_t a2, uint64_t bd, int ks, uint32_t more)
+{
+    if (ks == kWgKB / 16) {
+#pragma unroll
+        for (int q = QA; q < QB; ++q)
+#pragma unroll
+            for (int kk = 0; kk < kWgKB / 16; ++kk)
+                mma_f16(true, tmem + q * 64, (q < 3 ? a01 : a2) + (uint64_t)((q % 3) * 8 + kk * 128),
+                        bd + (uint64_t)(kk * 128), kWgIdesc, kk ? 1u : more);
+    } else {
+#pragma unroll
+        for (int q = QA; q < QB; ++q)
+#pragma unroll
+            for (int kk = 0; kk < kWgKB / 16 - 1; ++kk)
+                if (kk < ks)
+                    mma_f16(true, tmem + q * 64, (q < 3 ? a01 : a2) + (uint64_t)((q % 3) * 8 + kk * 128),
+                            bd + (uint64_t)(kk * 128), kWgIdesc, kk ? 1u : more);
+    }
+}
+
+__global__ void __launch_bounds__(kWgThreads, 1)
+    k_wgrad_tc(const WgDesc* __restrict__ tiles, const WgUnit* __restrict__ units, const int* __restrict__ first,
+               int classes, float* __restrict__ part, float* __restrict__ dbpart, int* err)
+{
     constexpr uint32_t kTmemCols = 512;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* sOnes = smem + (size_t)stages * kWgStage;
-    uint64_t* full = (uint64_t*)(sOnes + kWgRB);
-    uint64_t* empty = full + stages;
-    uint64_t* done = empty + stages;
-    uint32_t* tslot = (uint32_t*)(done + 1);
+    uint8_t* sOnes = smem + (size_t)kWgStages * kWgStage;
+    uint64_t* full = (uint64_t*)(sOnes + kWgOnes);
+    uint64_t* empty = full + kWgStages;
+    uint64_t* done = empty + kWgStages;      // a run's MMAs have completed
+    uint64_t* tfree = done + 1;              // its accumulators have been read
+    uint32_t* tslot = (uint32_t*)(tfree + 1);
+    constexpr int kWgEpiWarps = 13;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int XS = (a.W + kWgKB - 1) / kWgKB;
-    const long long njobs = (long long)a.N * a.H * XS;
-    const long long j0 = njobs * blockIdx.x / gridDim.x;
-    const long long j1 = njobs * (blockIdx.x + 1) / gridDim.x;
+    const int u0 = first[blockIdx.x], u1 = first[blockIdx.x + 1];
 
-    for (int i = threadIdx.x; i < kWgRB / 4; i += kWgThreads) ((uint32_t*)sOnes)[i] = 0x3F803F80u;  // bf16 1.0
+    for (int i = threadIdx.x; i < kWgOnes / 4; i += kWgThreads) ((uint32_t*)sOnes)[i] = 0x3F803F80u;  // bf16 1.0
     fence_async_smem();
     if (threadIdx.x == 0) {
-        for (int i = 0; i < stages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+        for (int i = 0; i < kWgStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
         mbar_init(done, 1);
+        mbar_init(tfree, kWgEpiWarps);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
     }
-    if (warp == 1) {
+    if (warp == 7) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(tslot)),
                      "r"(kTmemCols));
@@ -965,130 +1025,230 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     tc_fence_after();
     const uint32_t tmem = *(volatile uint32_t*)tslot;
 
-    if (warp == 0 && lane == 0) {
-        uint32_t it = 0, ph = 0;
-        int s = 0;
-        for (long long j = j0; j < j1; ++j, ++it, s = (s + 1 == stages ? 0 : s + 1),
-                       ph ^= (s == 0 ? 1u : 0u)) {
-            int xs = (int)(j % XS);
-            long long rest = j / XS;
-            int y = (int)(rest % a.H), n = (int)(rest / a.H);
-            if (!mbar_wait(&empty[s], ph ^ 1, a.err)) break;
-            mbar_expect_tx(&full[s], kWgTx);
-            uint8_t* sb = smem + (size_t)s * kWgStage;
-            for (int r = 0; r < 3; ++r)
-                tma_load_4d(sb + r * kWgRB, &tmap_x, 0, xs * kWgKB - 1, y - 1 + r, n, &full[s]);
-            tma_load_4d(sb + 3 * kWgRB, &tmap_dy, 0, xs * kWgKB, y, n, &full[s]);
-        }
-        // no copy may still be landing when the CTA exits
-        for (uint32_t i = it > (uint32_t)stages ? it - stages : 0; i < it; ++i)
-            mbar_drain(&full[i % stages], (i / stages) & 1, kTimeoutCycles);
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer.  A job's 24 MMAs use 6 A descriptors (tap pairs q) and
-        // one B descriptor, all built once per job; each K step of 16 pixels
-        // (2048 bytes further into every operand) only adds 2048 / 16 = 128
-        // to their start-address field (bits 0-13; shared-memory addresses
-        // stay far below the field's 256 KB).  The ring slot and its phase
-        // advance incrementally (no division per job).
-        const uint32_t ones = smem_u32(sOnes);
-        const uint32_t sbase = smem_u32(smem);
-        uint32_t it = 0, ph = 0;
-        int s = 0;
-        for (long long j = j0; j < j1; ++j, ++it) {
-            if (!mbar_wait(&full[s], ph, a.err)) break;
-            tc_fence_after();
-            const uint32_t base = sbase + (uint32_t)s * kWgStage;
-            const uint32_t top2 = base + 2 * kWgRB;
-            uint64_t ad[6];
-#pragma unroll
-            for (int q = 0; q < 6; ++q)
-                ad[q] = sdesc_mn((q < 3 ? base : top2) + (q % 3) * 128,
-                                 q < 3 ? (uint32_t)kWgRB : ones - top2);
-            const uint64_t bd0 = sdesc_mn(base + 3 * kWgRB, kWgBB);
-#pragma unroll
-            for (int kk = 0; kk < kWgKB / 16; ++kk) {
-                const uint64_t step = (uint64_t)(kk * 128);
-#pragma unroll
-                for (int q = 0; q < 6; ++q)
-                    mma_f16(tmem + q * 64, ad[q] + step, bd0 + step, IDESC,
-                            (it > 0 || kk > 0) ? 1u : 0u);
-            }
-            mma_commit(&empty[s]);
-            if (++s == stages) { s = 0; ph ^= 1u; }
-        }
-        mma_commit(done);   // arrives once every MMA issued above has completed
-    }
-    __syncwarp();
-
-    const bool ok = mbar_wait_warp(done, 0, a.err);
-    tc_fence_after();
-    if (ok) {
-        const bool have = j1 > j0;
-        const int m = 32 * warp + lane, c = m & 63;
-        float* P = a.part + (size_t)blockIdx.x * 9 * a.cout * a.cin;
-        for (int q = 0; q < 6; ++q) {
-            // TMEM lane m of MMA q: tap t (or the bias row when t < 0)
-            const int t = q < 3 ? (m < 64 ? q : 3 + q) : (m < 64 ? 3 + q : -1);
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                uint32_t r[16];
-                tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + q * 64 + h * 16, r);
-                tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int o = h * 16 + i;
-                    const float v = have ? __uint_as_float(r[i]) : 0.0f;
-                    if (o >= a.cout) continue;
-                    if (t >= 0) {
-                        if (c < a.cin) P[((size_t)t * a.cout + o) * a.cin + c] = v;
-                    } else if (q == 3 && m == 64) {
-                        a.dbpart[(size_t)blockIdx.x * a.cout + o] = v;
+    if (warp == 2) {
+        if (lane == 0) {
+            uint32_t it = 0, ph = 0;
+            int s = 0;
+            bool ok = true;
+            for (int u = u0; ok && u < u1; ++u) {
+                const WgDesc& d = tiles[units[u].tile];
+                // maps in global memory, written by the host before the launch
+                asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)&d.x) : "memory");
+                asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)&d.dy) : "memory");
+                const int XS = d.XS, H = d.H;
+                for (int g = units[u].w; ok && g < d.runs; g += classes) {
+                    const int je = wg_run(d, g + 1);
+                    for (int j = wg_run(d, g); j < je;
+                         ++j, ++it, s = (s + 1 == kWgStages ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
+                        const int xs = j % XS, r = j / XS, y = r % H, n = r / H;
+                        if (!mbar_wait(&empty[s], ph ^ 1, err)) { ok = false; break; }
+                        mbar_expect_tx(&full[s], kWgXBytes + kWgYBytes);
+                        uint8_t* sb = smem + (size_t)s * kWgStage;
+                        tma_load_4d(sb, &d.x, 0, xs * kWgKB - 1, y - 1, n, &full[s]);
+                        tma_load_4d(sb + kWgYOff, &d.dy, 0, xs * kWgKB, y, n, &full[s]);
                     }
                 }
             }
+            // no copy may still be landing when the CTA exits
+            for (uint32_t i = it > (uint32_t)kWgStages ? it - kWgStages : 0; i < it; ++i)
+                mbar_drain(&full[i % kWgStages], (i / kWgStages) & 1, kTimeoutCycles);
         }
+    } else if (warp == 3) {
+        if (lane == 0) {
+            // MMA issuer
+            const uint32_t ones = smem_u32(sOnes), sbase = smem_u32(smem);
+            uint32_t ph = 0, k = 0;
+            int s = 0;
+            bool ok = true;
+            for (int u = u0; ok && u < u1; ++u) {
+                const WgDesc& d = tiles[units[u].tile];
+                const int XS = d.XS, W = d.W;
+                const int half = units[u].half;
+                for (int g = units[u].w; ok && g < d.runs; g += classes, ++k) {
+                    const int jb = wg_run(d, g), je = wg_run(d, g + 1);
+                    // the previous run's accumulators have been read
+                    if (k > 0 && !mbar_wait(tfree, (k - 1) & 1, err)) { ok = false; break; }
+                    tc_fence_after();
+                    int xs = jb % XS;
+                    for (int j = jb; j < je; ++j) {
+                        if (!mbar_wait(&full[s], ph, err)) { ok = false; break; }
+                        tc_fence_after();
+                        const uint32_t base = sbase + (uint32_t)s * kWgStage, top2 = base + 2 * kWgXRow;
+                        const uint64_t a01 = sdesc_mn(base, kWgXRow), a2 = sdesc_mn(top2, ones - top2);
+                        const uint64_t bd = sdesc_mn(base + kWgYOff, kWgYBytes);
+                        const int ks = min(kWgKB / 16, (W - xs * kWgKB + 15) / 16);
+                        const uint32_t more = j > jb ? 1u : 0u;
+                        if (half == 0) wg_issue<0, 6>(tmem, a01, a2, bd, ks, more);
+                        else if (half == 1) wg_issue<0, 3>(tmem, a01, a2, bd, ks, more);
+                        else wg_issue<3, 6>(tmem, a01, a2, bd, ks, more);
+                        mma_commit(&empty[s]);
+                        if (++s == kWgStages) { s = 0; ph ^= 1u; }
+                        if (++xs == XS) xs = 0;
+                    }
+                    mma_commit(done);   // arrives once every MMA issued above has completed
+                }
+            }
+        }
+    } else if (warp != 7) {
+        const int quarter = warp & 3, m = 32 * quarter + lane, c = m & 63;
+        // this warp's columns: 96 from col0, or the bias row's 64
+        const bool bias = warp == 6;
+        const int col0 = bias ? 192 : 96 * (quarter < 2 ? warp >> 2 : (warp >> 2) - 2);
+        uint32_t k = 0;
+        bool ok = true;
+        for (int u = u0; ok && u < u1; ++u) {
+            const WgDesc& d = tiles[units[u].tile];
+            const int w = units[u].w, half = units[u].half, runs = d.runs, cin = d.cin, cout = d.cout;
+            const bool mine = half == 0 || (half == 1 ? col0 < 192 : col0 >= 192);
+            float acc[96];
+#pragma unroll
+            for (int i = 0; i < 96; ++i) acc[i] = 0.0f;
+            for (int g = w; g < runs; g += classes, ++k) {
+                if (!mbar_wait_warp(done, k & 1, err)) { ok = false; break; }
+                tc_fence_after();
+#pragma unroll
+                for (int h = 0; h < 12; ++h) {
+                    if (!mine || (h >= 8 && bias)) continue;
+                    uint32_t r[8];
+                    tmem_ld8(tmem + ((uint32_t)(32 * quarter) << 16) + col0 + 8 * h, r);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) acc[8 * h + i] += __uint_as_float(r[i]);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tfree);
+            }
+            if (!ok) break;
+            if (!mine) continue;
+            const size_t slot = (size_t)units[u].tile * classes + w;
+            float* P = part + slot * kWgPart;
+            if (bias) {
+                if (lane == 0)
+#pragma unroll
+                    for (int o = 0; o < 64; ++o)
+                        if (o < cout) dbpart[slot * 64 + o] = acc[o];
+            } else {
+#pragma unroll
+                for (int i = 0; i < 96; ++i) {
+                    // TMEM lane m of MMA q: tap t
+                    const int q = (col0 + i) >> 6, o = (col0 + i) & 63;
+                    const int t = q < 3 ? (m < 64 ? q : 3 + q) : 3 + q;
+                    if (o < cout && c < cin) P[((size_t)t * cout + o) * cin + c] = acc[i];
+                }
+            }
+        }
+        // on the error path MMAs may still run: TMEM is freed only after them
+        if (!ok && warp == 0 && lane == 0) mbar_drain(done, k & 1, kTimeoutCycles);
     }
-    // on the error path the MMAs may still run: TMEM is freed only after them
-    if (!ok && warp == 1 && lane == 0) mbar_drain(done, 0, kTimeoutCycles);
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 7) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(kTmemCols));
     }
 }
 
-size_t wgrad_smem(int stages)
-{
-    return 1024 + (size_t)stages * kWgStage + kWgRB + 8 * (2 * stages + 1) + 16;
-}
-
 }  // namespace
 
-int tc_wgrad_max_parts() { return sm_count(); }
-
-mrs_status tc_conv3x3_wgrad(const TcWgradArgs& a, int* nparts, cudaStream_t st)
+mrs_status tc_make_wg_x_map(CUtensorMap* m, const void* ptr, int N, int H, int W, long long px_stride,
+                            long long row_stride, long long img_stride)
 {
-    if (a.cin < 1 || a.cin > 64 || a.cout < 1 || a.cout > 64) {
-        set_error("tc_conv3x3_wgrad: cin, cout must be in [1, 64]");
-        return MRS_ERR_ARG;
+    return tc_make_view_map(m, ptr, N, H, W, px_stride, row_stride, img_stride, kWgKB + 2, 3);
+}
+mrs_status tc_make_wg_dy_map(CUtensorMap* m, const void* ptr, int N, int H, int W, long long px_stride,
+                             long long row_stride, long long img_stride)
+{
+    return tc_make_view_map(m, ptr, N, H, W, px_stride, row_stride, img_stride, kWgKB);
+}
+
+mrs_status tc_wgrad_plan(const std::vector<WgTile>& tiles, int classes, WgPlan& plan)
+{
+    const int nt = (int)tiles.size();
+    std::vector<WgDesc> d(nt);
+    struct Sized { long long cost; WgUnit u; };
+    std::vector<Sized> units;
+    plan.ntiles = nt;
+    plan.classes = classes;
+    long long total = 0;
+    plan.np.assign(nt, 0);
+    for (int t = 0; t < nt; ++t) {
+        const WgTile& w = tiles[t];
+        if (w.cin < 1 || w.cin > 64 || w.cout < 1 || w.cout > 64 || w.runs < 1) {
+            set_error("tc_wgrad_plan: cin, cout must be in [1, 64], runs >= 1");
+            return MRS_ERR_ARG;
+        }
+        WgDesc& e = d[t];
+        memset(&e, 0, sizeof(e));
+        e.x = w.x; e.dy = w.dy; e.H = w.H; e.W = w.W; e.cin = w.cin; e.cout = w.cout;
+        e.XS = (w.W + kWgKB - 1) / kWgKB;
+        const long long nj = (long long)w.N * w.H * e.XS;
+        if (nj > 0x7fffffff) { set_error("tc_wgrad_plan: too many jobs"); return MRS_ERR_CAPACITY; }
+        e.njobs = (int)nj;
+        e.runs = (int)std::min<long long>(nj, w.runs);
+        plan.np[t] = std::min(e.runs, classes);
+        for (int c = 0; c < plan.np[t]; ++c) {
+            long long cost = 0;
+            // K steps of the class's runs, and about six for each emptying
+            for (int g = c; g < e.runs; g += classes)
+                cost += (nj * (g + 1) / e.runs - nj * g / e.runs) * ((w.W + 15) / 16) / e.XS + 6;
+            units.push_back({cost, {t, c, 0}});
+            total += cost;
+        }
     }
-    int stages = 2;
-    while (wgrad_smem(stages + 1) <= 227 * 1024 && stages < 8) ++stages;
-    size_t smem = wgrad_smem(stages);
+    // a unit well above an SM's even share is done in two halves
+    for (size_t i = 0, n = units.size(); i < n; ++i)
+        if (units[i].cost * 4 * sm_count() > 5 * total) {
+            Sized b = units[i];
+            units[i].u.half = 1;
+            b.u.half = 2;
+            units[i].cost = b.cost = b.cost / 2 + 1;
+            units.push_back(b);
+        }
+    // the units to the CTAs, largest first, each to the least loaded
+    plan.units = (int)units.size();
+    plan.ctas = (int)std::min<size_t>(units.size(), (size_t)sm_count());
+    std::stable_sort(units.begin(), units.end(), [](const Sized& a, const Sized& b) { return a.cost > b.cost; });
+    std::vector<std::vector<WgUnit>> mine(plan.ctas);
+    typedef std::pair<long long, int> Load;
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> load;
+    for (int g = 0; g < plan.ctas; ++g) load.push({0, g});
+    for (const Sized& s : units) {
+        Load l = load.top();
+        load.pop();
+        mine[l.second].push_back(s.u);
+        load.push({l.first + s.cost, l.second});
+    }
+    std::vector<WgUnit> list;
+    std::vector<int> first;
+    for (const auto& m : mine) {
+        first.push_back((int)list.size());
+        list.insert(list.end(), m.begin(), m.end());
+    }
+    first.push_back((int)list.size());
+    const size_t a = nt * sizeof(WgDesc), b = list.size() * sizeof(WgUnit);
+    plan.blob.resize(a + b + first.size() * sizeof(int));
+    memcpy(plan.blob.data(), d.data(), a);
+    memcpy(plan.blob.data() + a, list.data(), b);
+    memcpy(plan.blob.data() + a + b, first.data(), first.size() * sizeof(int));
+    return MRS_OK;
+}
+
+mrs_status tc_conv3x3_wgrad(const WgPlan& plan, const void* d_blob, float* part, float* dbpart, int* err,
+                            cudaStream_t st)
+{
+    if (plan.ctas < 1) return MRS_OK;
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
         if (e != cudaSuccess) return cuda_status(e, "wgrad smem attribute");
         attr = true;
     }
-    long long njobs = (long long)a.N * a.H * ((a.W + kWgKB - 1) / kWgKB);
-    const int cap = a.max_ctas > 0 && a.max_ctas < sm_count() ? a.max_ctas : sm_count();
-    int grid = njobs < cap ? (int)njobs : cap;
-    *nparts = grid;
-    if (grid < 1) return MRS_OK;
-    MRS_TIMED(PK_WGRAD_TC, st, (k_wgrad_tc<<<grid, kWgThreads, smem, st>>>(*a.tmap_x, *a.tmap_dy, a, stages)));
+    const WgDesc* d = (const WgDesc*)d_blob;
+    const WgUnit* u = (const WgUnit*)(d + plan.ntiles);
+    const int* first = (const int*)(u + plan.units);
+    MRS_TIMED(PK_WGRAD_TC, st, (k_wgrad_tc<<<plan.ctas, kWgThreads, kWgSmem, st>>>(d, u, first, plan.classes, part, dbpart, err)));
     MRS_LAUNCHED(1);
     return cuda_status(cudaGetLastError(), "wgrad launch");
 }

@@ -6,6 +6,8 @@
 #include <cudaTypedefs.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "common.cuh"
 
 namespace mrs {
@@ -75,7 +77,7 @@ mrs_status tc_make_act_map(CUtensorMap* m, const void* ptr, int N, int H, int W,
 // an output) without moving data.
 mrs_status tc_make_view_map(CUtensorMap* m, const void* ptr, int N, int H, int W,
                             long long px_stride, long long row_stride, long long img_stride,
-                            int box_px);
+                            int box_px, int box_rows = 1);
 // Tensor map for packed weights [rows][64 (bf16) | 64 (fp8)].
 mrs_status tc_make_w_map(CUtensorMap* m, const void* ptr, int rows, int nout, int operand);
 
@@ -83,28 +85,41 @@ mrs_status tc_conv3x3(const TcConvArgs& a, cudaStream_t st);
 // input-row ring depth of every later conv launch (0: the most that fits)
 void tc_set_ring(int stages);
 
-// Weight and bias gradients of a 3x3 conv (zero padding 1) on the tensor
-// cores, as per-CTA partial sums:
-//   part[g][t][o][c] (t = ky * 3 + kx) = sum over CTA g's pixels p of
-//       dy[p][o] * x[p + (ky - 1, kx - 1)][c],   dbpart[g][o] = sum dy[p][o]
-// for o < cout, c < cin.  x and dy are bf16 [N][H][W][64] tensors described
-// by tc_make_act_map with box widths kWgKB + 2 (x) and kWgKB (dy).  *nparts
-// receives the number of partials written (at most tc_wgrad_max_parts()).
-constexpr int kWgKB = 64;
-struct TcWgradArgs {
-    const CUtensorMap* tmap_x;
-    const CUtensorMap* tmap_dy;
-    float* part;
-    float* dbpart;
+// Weight and bias gradients of 3x3 convs (zero padding 1) on the tensor cores:
+// one launch over a list of tiles (a tile: one conv's up to 64 x 64 channels),
+//   dw[o][t][c] (t = ky * 3 + kx) = sum over pixels p of
+//       dy[p][o] * x[p + (ky - 1, kx - 1)][c],   db[o] = sum dy[p][o]
+// for o < cout, c < cin.  A tile's jobs (kWgKB pixels of one row; strips, then
+// rows, then images) are cut into `runs` equal contiguous runs, each summed on
+// the tensor cores; runs w, w + C, ... (class w of C = `classes`) are added in
+// FP32 in that order and written as partial w of the tile's np = min(runs, C):
+//   part[(slot + w) * kWgPart + (tap * cout + o) * cin + c], dbpart[(slot + w) * 64 + o]
+// (slot: C times the tile's number).  The sums' order depends on the tiles alone.
+// C = 8 leaves few partials; a list of one tile takes C = runs, whose units of
+// work are enough for every SM.
+constexpr int kWgKB = 64;          // pixels per job
+constexpr int kWgPart = 9 * 64 * 64;
+struct WgTile {
+    CUtensorMap x, dy;             // tc_make_wg_x_map / tc_make_wg_dy_map
     int N, H, W, cin, cout;
-    int* err;
-    // at most this many CTAs (= partials), 0: one per SM.  Several small
-    // gradients launched side by side on different streams, each on a share
-    // of the SMs, write that many fewer partials each.
-    int max_ctas = 0;
+    int runs;                      // at most the tile's jobs are used
 };
-int tc_wgrad_max_parts();
-mrs_status tc_conv3x3_wgrad(const TcWgradArgs& a, int* nparts, cudaStream_t st);
+struct WgPlan {
+    int ntiles = 0, ctas = 0, units = 0, classes = 8;
+    std::vector<int> np;           // per tile: its partials
+    std::vector<uint8_t> blob;     // what the kernel reads: upload to 64-byte aligned device memory
+    size_t part_floats() const { return (size_t)ntiles * classes * kWgPart; }
+    size_t dbpart_floats() const { return (size_t)ntiles * classes * 64; }
+};
+mrs_status tc_wgrad_plan(const std::vector<WgTile>& tiles, int classes, WgPlan& plan);
+mrs_status tc_conv3x3_wgrad(const WgPlan& plan, const void* d_blob, float* part, float* dbpart,
+                            int* err, cudaStream_t st);
+// Operand maps of a tile: [N][H][W][64] bf16 with the given strides (bytes)
+// between pixels, rows and images (as tc_make_view_map).
+mrs_status tc_make_wg_x_map(CUtensorMap* m, const void* ptr, int N, int H, int W, long long px_stride,
+                            long long row_stride, long long img_stride);
+mrs_status tc_make_wg_dy_map(CUtensorMap* m, const void* ptr, int N, int H, int W, long long px_stride,
+                             long long row_stride, long long img_stride);
 
 // Launches a kernel whose bounded mbarrier wait can never complete; *gave_up
 // = 1 if the wait gave up after limit_cycles and raised the error word.

@@ -13,6 +13,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
 #include <string>
 #include <mutex>
 #include <vector>
@@ -590,18 +591,18 @@ __global__ void __launch_bounds__(256)
 }
 
 // grad[o][t][c] (params layout) = sum_g part[g][t][o][c]; grad_b[o] = sum_g dbpart[g][o]
+// (partials gstride floats apart, bias partials bstride).
 // A block takes 32 consecutive values; warp w sums partials w, w + 8, ... (one
 // coalesced 128-byte row per partial) and the eight sums are added in warp
 // order: a fixed order, so the result is deterministic.
 __global__ void __launch_bounds__(256) k_dw_reduce(const float* __restrict__ part,
-                                                   const float* __restrict__ dbpart, int G, int cin,
-                                                   int cout, float* __restrict__ gw,
-                                                   float* __restrict__ gb)
+                                                   const float* __restrict__ dbpart, int G,
+                                                   size_t gstride, int bstride, int cin, int cout,
+                                                   float* __restrict__ gw, float* __restrict__ gb)
 {
     __shared__ float red[8][32];
     const int nw = cout * 9 * cin, ntot = nw + cout;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const size_t gstride = (size_t)9 * cout * cin;
     for (int e0 = blockIdx.x * 32; e0 < ntot; e0 += gridDim.x * 32) {
         const int e = e0 + lane;
         float acc = 0.0f;
@@ -611,7 +612,7 @@ __global__ void __launch_bounds__(256) k_dw_reduce(const float* __restrict__ par
             for (int g = wp; g < G; g += 8) acc += src[(size_t)g * gstride];
         } else if (e < ntot) {
             const int o = e - nw;
-            for (int g = wp; g < G; g += 8) acc += dbpart[(size_t)g * cout + o];
+            for (int g = wp; g < G; g += 8) acc += dbpart[(size_t)g * bstride + o];
         }
         red[wp][lane] = acc;
         __syncthreads();
@@ -622,6 +623,36 @@ __global__ void __launch_bounds__(256) k_dw_reduce(const float* __restrict__ par
             else gb[e - nw] = v;
         }
         __syncthreads();
+    }
+}
+
+// Every tile's partial sums into the gradient (see WgRed): one thread per
+// value, reads coalesced along the input channels.
+__device__ __forceinline__ float sum_parts(const float* __restrict__ src, size_t stride, int np)
+{
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = i < np ? src[i * stride] : 0.0f;
+    float acc = v[0];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) acc += v[i];
+    return acc;
+}
+__global__ void __launch_bounds__(256) k_wg_reduce(const WgRed* __restrict__ reds, const float* __restrict__ part,
+                                                   const float* __restrict__ dbpart, float* __restrict__ grad)
+{
+    const int t = blockIdx.y;
+    const WgRed r = reds[t];
+    const int nw = r.cout * r.KK * r.cin, e = blockIdx.x * 256 + threadIdx.x;
+    if (e < nw) {
+        const int c = e % r.cin, tl = (e / r.cin) % r.KK, o = e / (r.cin * r.KK);
+        const float acc = sum_parts(part + (size_t)8 * t * kWgPart +
+                                        ((size_t)(r.KK == 9 ? tl : 4) * r.cout + o) * r.cin + c, kWgPart, r.np);
+        const int ci = r.q > 0 ? 64 + dsf_channel(c, (r.q - 1) / r.s, (r.q - 1) % r.s, r.D) : r.c0 + c;
+        grad[r.gw + ((long long)(r.o_mul * o + r.o_add) * r.KK + tl) * r.CIN + ci] = acc;
+    } else if (e - nw < r.cout && r.with_bias) {
+        const int o = e - nw;
+        grad[r.gb + r.o_mul * o + r.o_add] = sum_parts(dbpart + (size_t)8 * t * 64 + o, 64, r.np);
     }
 }
 
@@ -701,6 +732,15 @@ mrs_status dw_tiles_f32(const float* x, int cin, int xs, const float* dy, int co
                                                      centre_only ? 4 : 0, ctiles);
     MRS_LAUNCHED(1);
     return cuda_status(cudaGetLastError(), "dw tiles");
+}
+
+mrs_status wg_reduce(const WgRed* d_reds, int ntiles, const float* part, const float* dbpart, float* grad,
+                     cudaStream_t st)
+{
+    const dim3 grid((kWgPart + 64 + 255) / 256, ntiles);
+    MRS_TIMED(PK_TRAIN, st, k_wg_reduce<<<grid, 256, 0, st>>>(d_reds, part, dbpart, grad));
+    MRS_LAUNCHED(1);
+    return cuda_status(cudaGetLastError(), "wgrad reduce");
 }
 
 void wtrans_f32(const float* w, int cin, int cout, float* wt, cudaStream_t st)
@@ -814,6 +854,21 @@ Scratch& scratch()
 }  // namespace
 }  // namespace mrs
 
+namespace mrs {
+// What a BF16 training step of one shape needs besides its data: the tensor
+// maps of its activations (all inside the handle's workspace) and the
+// weight-gradient tiles.  Made again when the shape or the workspace changes.
+struct StepPlan {
+    int N = -1, H = -1, W = -1;
+    void* act = nullptr;
+    CUtensorMap x0A, dybA, hA[9], hO[9], rA[8], rO[8], dhA[9], dhO[9], daA[8], daO[8];
+    WgPlan wg;
+    Buf blob;                      // wg.blob, then the tiles' WgRed, on the device
+    const WgRed* reds = nullptr;
+    ~StepPlan() { blob.release(); }
+};
+}  // namespace mrs
+
 using namespace mrs;
 
 struct mrs_net_s {
@@ -840,6 +895,7 @@ struct mrs_net_s {
     Buf tact;                      // training activations
     Buf ttmp;                      // training scratch (transposed weights, dW partials, loss)
     int* err = nullptr;            // device error word
+    std::unique_ptr<mrs::StepPlan> plan;   // tensor maps and wgrad tiles of the last BF16 step's shape
     int loss_kind = MRS_LOSS_L1LOG;
     float loss_beta = 0.1f;
 };
@@ -1069,6 +1125,8 @@ extern "C" mrs_status mrs_net_free(mrs_net net)
         if (p) cudaFree(p);
     net->act.release();
     net->aux.release();
+    net->tact.release();
+    net->ttmp.release();
     delete net;
     return MRS_OK;
 }
@@ -1356,8 +1414,8 @@ mrs_status layer_dw(mrs_net_s* net, int l, const float* x, const float* dy, int 
     MRS_TIMED(PK_TRAIN, st, (k_dw_partial<float, float><<<grid, 256, 0, st>>>(x, L.cin, L.cin, dy, L.cout, L.cout, N, H, W, part, dbpart, 0, 1)));
     MRS_LAUNCHED(1);
     int nw = L.cout * 9 * L.cin + L.cout;
-    MRS_TIMED(PK_TRAIN, st, k_dw_reduce<<<(nw + 31) / 32, 256, 0, st>>>(part, dbpart, kDwSplits, L.cin, L.cout,
-                                                         net->grad + L.woff, net->grad + L.boff));
+    MRS_TIMED(PK_TRAIN, st, k_dw_reduce<<<(nw + 31) / 32, 256, 0, st>>>(part, dbpart, kDwSplits, (size_t)9 * L.cout * L.cin, L.cout,
+                                                         L.cin, L.cout, net->grad + L.woff, net->grad + L.boff));
     MRS_LAUNCHED(1);
     return cuda_status(cudaGetLastError(), "dw");
 }
@@ -1481,6 +1539,67 @@ mrs_status pack_bf16_T(mrs_net_s* net, cudaStream_t st)
     return cuda_status(cudaGetLastError(), "pack bf16 T");
 }
 
+// The plan of a step of this shape over the workspace tensors (see StepPlan)
+mrs_status step_plan(mrs_net_s* net, int N, int H, int W, __nv_bfloat16* x0, __nv_bfloat16* hs, __nv_bfloat16* rs,
+                     __nv_bfloat16* dyb, __nv_bfloat16* dhs, __nv_bfloat16* das)
+{
+    if (net->plan && net->plan->N == N && net->plan->H == H && net->plan->W == W && net->plan->act == x0)
+        return MRS_OK;
+    net->plan.reset();
+    std::unique_ptr<StepPlan> pl(new StepPlan());
+    const size_t F = (size_t)N * H * W * 64;
+    const auto& L = shapes(net->cin0);
+    mrs_status rc = MRS_OK;
+    // A operands (130-pixel boxes) and residual / output (128-pixel)
+    auto amap = [&](CUtensorMap* m, const void* ptr) {
+        if (rc == MRS_OK) rc = tc_make_act_map(m, ptr, N, H, W, TC_BF16, tc_a_box(TC_BF16));
+    };
+    auto omap = [&](CUtensorMap* m, const void* ptr) {
+        if (rc == MRS_OK) rc = tc_make_act_map(m, ptr, N, H, W, TC_BF16, tc_out_box(TC_BF16));
+    };
+    amap(&pl->x0A, x0);
+    amap(&pl->dybA, dyb);
+    for (int k = 0; k < 9; ++k) {
+        amap(&pl->hA[k], hs + k * F); omap(&pl->hO[k], hs + k * F);
+        amap(&pl->dhA[k], dhs + k * F); omap(&pl->dhO[k], dhs + k * F);
+    }
+    for (int k = 0; k < 8; ++k) {
+        amap(&pl->rA[k], rs + k * F); omap(&pl->rO[k], rs + k * F);
+        amap(&pl->daA[k], das + k * F); omap(&pl->daO[k], das + k * F);
+    }
+    std::vector<WgTile> tiles;
+    std::vector<WgRed> reds;
+    auto tile = [&](int l, const void* x, const void* dyp) {
+        WgTile t;
+        if (rc == MRS_OK) rc = tc_make_wg_x_map(&t.x, x, N, H, W, 128, 128LL * W, 128LL * W * H);
+        if (rc == MRS_OK) rc = tc_make_wg_dy_map(&t.dy, dyp, N, H, W, 128, 128LL * W, 128LL * W * H);
+        t.N = N; t.H = H; t.W = W; t.cin = L[l].cin; t.cout = L[l].cout; t.runs = sm_count();
+        tiles.push_back(t);
+        WgRed r;
+        memset(&r, 0, sizeof(r));
+        r.cin = r.CIN = L[l].cin; r.cout = L[l].cout; r.KK = 9; r.o_mul = 1; r.s = 1; r.with_bias = 1;
+        r.gw = (long long)L[l].woff; r.gb = (long long)L[l].boff;
+        reds.push_back(r);
+    };
+    tile(17, hs + 8 * F, dyb);
+    for (int k = 7; k >= 0; --k) {
+        tile(2 + 2 * k, rs + k * F, dhs + (k + 1) * F);
+        tile(1 + 2 * k, hs + k * F, das + k * F);
+    }
+    tile(0, x0, dhs);
+    if (rc == MRS_OK) rc = tc_wgrad_plan(tiles, 8, pl->wg);
+    if (rc != MRS_OK) return rc;
+    for (size_t t = 0; t < reds.size(); ++t) reds[t].np = pl->wg.np[t];
+    const size_t off = (pl->wg.blob.size() + 15) & ~(size_t)15;
+    if ((rc = pl->blob.ensure(off + reds.size() * sizeof(WgRed))) != MRS_OK) return rc;
+    MRS_CHECK(cudaMemcpy(pl->blob.p, pl->wg.blob.data(), pl->wg.blob.size(), cudaMemcpyHostToDevice));
+    MRS_CHECK(cudaMemcpy((uint8_t*)pl->blob.p + off, reds.data(), reds.size() * sizeof(WgRed), cudaMemcpyHostToDevice));
+    pl->reds = (const WgRed*)((uint8_t*)pl->blob.p + off);
+    pl->N = N; pl->H = H; pl->W = W; pl->act = x0;
+    net->plan = std::move(pl);
+    return MRS_OK;
+}
+
 // BF16 training step: forward and transposed convolutions on the tensor-core
 // kernel with BF16 activations / activation gradients, FP32 accumulation,
 // FP32 dW / db reductions and FP32 master weights + Adam
@@ -1491,61 +1610,32 @@ mrs_status train_step_bf16(mrs_net_s* net, const float* lrhs, const float* hrls,
     const size_t P = (size_t)N * H * W;
     const size_t F = P * 64;                       // bf16 elements of one [P][64] tensor
     const size_t nlr = (size_t)N * (H / s) * (W / s) * 3;
-    size_t need = (size_t)(1 + 9 + 8 + 3) * F * 2 + (2 * P * 3 + nlr + P * 3) * 4 + 4096;
+    size_t need = (size_t)(1 + 9 + 8 + 1 + 9 + 8) * F * 2 + (2 * P * 3 + nlr + P * 3) * 4 + 4096;
     mrs_status rc = net->tact.ensure(need);
     if (rc != MRS_OK) return rc;
-    const size_t maxp = (size_t)std::max(kDwSplits, tc_wgrad_max_parts());
-    size_t tneed = (64 * 9 * 64 + 64) * 4 + (maxp * 9 * 64 * 64 + maxp * 64) * 4 + (kRedBlocks + 8) * 8;
-    if ((rc = net->ttmp.ensure(tneed)) != MRS_OK) return rc;
-    if ((rc = pack_bf16(net, st)) != MRS_OK) return rc;
-    if ((rc = pack_bf16_T(net, st)) != MRS_OK) return rc;
     __nv_bfloat16* x0 = net->tact.as<__nv_bfloat16>();
     __nv_bfloat16* hs = x0 + F;
     __nv_bfloat16* rs = hs + 9 * F;
     __nv_bfloat16* dyb = rs + 8 * F;
-    __nv_bfloat16* dh = dyb + F;
-    __nv_bfloat16* da = dh + F;
-    float* y = (float*)(da + F);
+    __nv_bfloat16* dhs = dyb + F;                  // dL/dh_k, k = 0 .. 8
+    __nv_bfloat16* das = dhs + 9 * F;              // dL/d(inner conv of block k), masked
+    float* y = (float*)(das + 8 * F);
     float* dy = y + P * 3;
     float* lrc = dy + P * 3;
     float* hrc = lrc + nlr;
-    float* zero = net->ttmp.as<float>() + 64 * 9 * 64;
-    float* part = zero + 64;
-    float* dbpart = part + maxp * 9 * 64 * 64;
-    double* lparts = (double*)(dbpart + maxp * 64);
+    if ((rc = step_plan(net, N, H, W, x0, hs, rs, dyb, dhs, das)) != MRS_OK) return rc;
+    StepPlan& pl = *net->plan;
+    size_t tneed = 64 * 4 + (pl.wg.part_floats() + pl.wg.dbpart_floats()) * 4 + (kRedBlocks + 8) * 8;
+    if ((rc = net->ttmp.ensure(tneed)) != MRS_OK) return rc;
+    if ((rc = pack_bf16(net, st)) != MRS_OK) return rc;
+    if ((rc = pack_bf16_T(net, st)) != MRS_OK) return rc;
+    double* lparts = net->ttmp.as<double>();
     double* lres = lparts + kRedBlocks;
+    float* zero = (float*)(lres + 8);
+    float* part = zero + 64;
+    float* dbpart = part + pl.wg.part_floats();
     MRS_CHECK(cudaMemsetAsync(zero, 0, 64 * 4, st));
-    const auto& L = shapes(net->cin0);
 
-    // tensor maps: A operands (130-pixel boxes) and residual / output (128-pixel)
-    auto amap = [&](CUtensorMap* m, const void* ptr) { return tc_make_act_map(m, ptr, N, H, W, TC_BF16, tc_a_box(TC_BF16)); };
-    auto omap = [&](CUtensorMap* m, const void* ptr) { return tc_make_act_map(m, ptr, N, H, W, TC_BF16, tc_out_box(TC_BF16)); };
-    std::vector<CUtensorMap> hA(9), hO(9), rA(8), rO(8);
-    CUtensorMap x0A, dybA, dhA, dhO, daA, daO;
-    for (int k = 0; k < 9 && rc == MRS_OK; ++k) {
-        if ((rc = amap(&hA[k], hs + k * F)) == MRS_OK) rc = omap(&hO[k], hs + k * F);
-        if (k < 8 && rc == MRS_OK) { if ((rc = amap(&rA[k], rs + k * F)) == MRS_OK) rc = omap(&rO[k], rs + k * F); }
-    }
-    if (rc == MRS_OK) rc = amap(&x0A, x0);
-    if (rc == MRS_OK) rc = amap(&dybA, dyb);
-    if (rc == MRS_OK) rc = amap(&dhA, dh);
-    if (rc == MRS_OK) rc = omap(&dhO, dh);
-    if (rc == MRS_OK) rc = amap(&daA, da);
-    if (rc == MRS_OK) rc = omap(&daO, da);
-    // weight-gradient operands: x rows with a one-pixel halo, dy rows
-    auto xwmap = [&](CUtensorMap* m, const void* ptr) { return tc_make_act_map(m, ptr, N, H, W, TC_BF16, kWgKB + 2); };
-    auto dwmap = [&](CUtensorMap* m, const void* ptr) { return tc_make_act_map(m, ptr, N, H, W, TC_BF16, kWgKB); };
-    std::vector<CUtensorMap> hX(9), rX(8);
-    CUtensorMap x0X, dybD, dhD, daD;
-    for (int k = 0; k < 9 && rc == MRS_OK; ++k) {
-        rc = xwmap(&hX[k], hs + k * F);
-        if (k < 8 && rc == MRS_OK) rc = xwmap(&rX[k], rs + k * F);
-    }
-    if (rc == MRS_OK) rc = xwmap(&x0X, x0);
-    if (rc == MRS_OK) rc = dwmap(&dybD, dyb);
-    if (rc == MRS_OK) rc = dwmap(&dhD, dh);
-    if (rc == MRS_OK) rc = dwmap(&daD, da);
-    if (rc != MRS_OK) return rc;
     TcConvArgs a;
     memset(&a, 0, sizeof(a));
     a.N = N; a.H = H; a.W = W; a.scale = s; a.operand = TC_BF16; a.err = net->err; a.nout = 64;
@@ -1563,17 +1653,17 @@ mrs_status train_step_bf16(mrs_net_s* net, const float* lrhs, const float* hrls,
     MRS_LAUNCHED(1);
     k_input_q<<<grid1d(P), 256, 0, st>>>(lrc, hrc, alb, nrm, extra, H, W, s, P, x0, 0, 1.0f, kClip);
     MRS_LAUNCHED(1);
-    rc = conv(&x0A, &net->wmap_bf[0], net->bias, TC_RELU_BF16, nullptr, &hO[0], 64);
+    rc = conv(&pl.x0A, &net->wmap_bf[0], net->bias, TC_RELU_BF16, nullptr, &pl.hO[0], 64);
     for (int k = 0; k < 8 && rc == MRS_OK; ++k) {
-        rc = conv(&hA[k], &net->wmap_bf[1 + 2 * k], net->bias + (1 + 2 * k) * 64, TC_RELU_BF16,
-                  nullptr, &rO[k], 64);
+        rc = conv(&pl.hA[k], &net->wmap_bf[1 + 2 * k], net->bias + (1 + 2 * k) * 64, TC_RELU_BF16,
+                  nullptr, &pl.rO[k], 64);
         if (rc == MRS_OK)
-            rc = conv(&rA[k], &net->wmap_bf[2 + 2 * k], net->bias + (2 + 2 * k) * 64, TC_RESID_BF16,
-                      &hO[k], &hO[k + 1], 64);
+            rc = conv(&pl.rA[k], &net->wmap_bf[2 + 2 * k], net->bias + (2 + 2 * k) * 64, TC_RESID_BF16,
+                      &pl.hO[k], &pl.hO[k + 1], 64);
     }
     if (rc == MRS_OK) {
         a.out = y; a.lrhs = lrc; a.cout = 3;
-        rc = conv(&hA[8], &net->wmap_bf[17], net->bias + 17 * 64, TC_FINAL_F32, nullptr, nullptr, 16);
+        rc = conv(&pl.hA[8], &net->wmap_bf[17], net->bias + 17 * 64, TC_FINAL_F32, nullptr, nullptr, 16);
     }
     if (rc != MRS_OK) return rc;
 
@@ -1584,37 +1674,24 @@ mrs_status train_step_bf16(mrs_net_s* net, const float* lrhs, const float* hrls,
     k_reduce_parts<<<1, 256, 0, st>>>(lparts, kRedBlocks, 1, lres);
     MRS_LAUNCHED(1);
 
-    // backward: weight gradients on the tensor cores (per-CTA partials, then a
-    // deterministic reduction), data gradients as convs with the flipped,
-    // transposed weights
-    auto dw = [&](int l, const CUtensorMap* xm, const CUtensorMap* dym) {
-        const LayerShape& S_ = L[l];
-        TcWgradArgs wa;
-        wa.tmap_x = xm; wa.tmap_dy = dym; wa.part = part; wa.dbpart = dbpart;
-        wa.N = N; wa.H = H; wa.W = W; wa.cin = S_.cin; wa.cout = S_.cout; wa.err = net->err;
-        int np = 0;
-        mrs_status r = tc_conv3x3_wgrad(wa, &np, st);
-        if (r != MRS_OK) return r;
-        int nw = S_.cout * 9 * S_.cin + S_.cout;
-        MRS_TIMED(PK_TRAIN, st, k_dw_reduce<<<(nw + 31) / 32, 256, 0, st>>>(part, dbpart, np, S_.cin, S_.cout,
-                                                       net->grad + S_.woff, net->grad + S_.boff));
-        MRS_LAUNCHED(1);
-        return cuda_status(cudaGetLastError(), "dw");
-    };
+    // backward: data gradients as convs with the flipped, transposed weights,
+    // every one kept, then the weight gradients of all layers in one launch
+    // (18 launches of 152 partial sums each, and their reductions, took 1.37 of
+    // a step's 2.50 ms at 16 x 128^2)
     k_to_operand<<<1024, 256, 0, st>>>(dy, P, 3, dyb, 0, 1.0f);
     MRS_LAUNCHED(1);
-    if ((rc = dw(17, &hX[8], &dybD)) != MRS_OK) return rc;
-    if ((rc = conv(&dybA, &net->wmap_bfT[17], zero, TC_LIN_BF16, nullptr, &dhO, 64)) != MRS_OK) return rc;
+    if ((rc = conv(&pl.dybA, &net->wmap_bfT[17], zero, TC_LIN_BF16, nullptr, &pl.dhO[8], 64)) != MRS_OK) return rc;
     for (int k = 7; k >= 0; --k) {
         int l2 = 2 + 2 * k, l1 = 1 + 2 * k;
-        if ((rc = dw(l2, &rX[k], &dhD)) != MRS_OK) return rc;
-        if ((rc = conv(&dhA, &net->wmap_bfT[l2], zero, TC_MASK_BF16, &rO[k], &daO, 64)) != MRS_OK) return rc;
-        if ((rc = dw(l1, &hX[k], &daD)) != MRS_OK) return rc;
-        if ((rc = conv(&daA, &net->wmap_bfT[l1], zero, TC_RESID_BF16, &dhO, &dhO, 64)) != MRS_OK) return rc;
+        if ((rc = conv(&pl.dhA[k + 1], &net->wmap_bfT[l2], zero, TC_MASK_BF16, &pl.rO[k], &pl.daO[k], 64)) != MRS_OK)
+            return rc;
+        if ((rc = conv(&pl.daA[k], &net->wmap_bfT[l1], zero, TC_RESID_BF16, &pl.dhO[k + 1], &pl.dhO[k], 64)) != MRS_OK)
+            return rc;
     }
-    k_mask_bf16<<<grid1d(F), 256, 0, st>>>(dh, hs, F);
+    k_mask_bf16<<<grid1d(F), 256, 0, st>>>(dhs, hs, F);
     MRS_LAUNCHED(1);
-    if ((rc = dw(0, &x0X, &dhD)) != MRS_OK) return rc;
+    if ((rc = tc_conv3x3_wgrad(pl.wg, pl.blob.p, part, dbpart, net->err, st)) != MRS_OK) return rc;
+    if ((rc = wg_reduce(pl.reds, pl.wg.ntiles, part, dbpart, net->grad, st)) != MRS_OK) return rc;
 
     // Adam on the FP32 master weights
     net->step += 1;
@@ -1905,10 +1982,10 @@ extern "C" mrs_status mrs_conv3x3_wgrad(const float* x, const float* dy, int32_t
     cudaStream_t st = (cudaStream_t)stream;
     const size_t P = (size_t)N * H * W;
     const size_t nw = (size_t)cout * 9 * cin;
-    const size_t maxp = (size_t)std::max(kDwSplits, tc_wgrad_max_parts());
+    const size_t maxp = (size_t)std::max(kDwSplits, sm_count());
     Scratch& S = scratch();
     std::lock_guard<std::mutex> g(S.mu);
-    size_t need = (nw + cout) * 4 + maxp * (9 * 64 * 64 + 64) * 4 + 4096 +
+    size_t need = (nw + cout) * 4 + maxp * (9 * 64 * 64 + 64) * 4 + 8192 +
                   (precision == MRS_PREC_BF16 ? 2 * P * 128 : 0);
     mrs_status rc = S.b.ensure(need);
     if (rc != MRS_OK) return rc;
@@ -1931,15 +2008,21 @@ extern "C" mrs_status mrs_conv3x3_wgrad(const float* x, const float* dy, int32_t
         MRS_LAUNCHED(1);
         k_to_operand<<<1024, 256, 0, st>>>(dy, P, cout, dq, 0, 1.0f);
         MRS_LAUNCHED(1);
-        CUtensorMap mx, md;
-        if ((rc = tc_make_act_map(&mx, xq, N, H, W, TC_BF16, kWgKB + 2)) != MRS_OK) return rc;
-        if ((rc = tc_make_act_map(&md, dq, N, H, W, TC_BF16, kWgKB)) != MRS_OK) return rc;
-        TcWgradArgs wa;
-        wa.tmap_x = &mx; wa.tmap_dy = &md; wa.part = part; wa.dbpart = dbpart;
-        wa.N = N; wa.H = H; wa.W = W; wa.cin = cin; wa.cout = cout; wa.err = err;
-        if ((rc = tc_conv3x3_wgrad(wa, &np, st)) != MRS_OK) return rc;
+        std::vector<WgTile> tile(1);
+        WgTile& t = tile[0];
+        if ((rc = tc_make_wg_x_map(&t.x, xq, N, H, W, 128, 128LL * W, 128LL * W * H)) != MRS_OK) return rc;
+        if ((rc = tc_make_wg_dy_map(&t.dy, dq, N, H, W, 128, 128LL * W, 128LL * W * H)) != MRS_OK) return rc;
+        t.N = N; t.H = H; t.W = W; t.cin = cin; t.cout = cout; t.runs = sm_count();   // np partials at most
+        WgPlan plan;
+        if ((rc = tc_wgrad_plan(tile, t.runs, plan)) != MRS_OK) return rc;
+        void* blob = dq + P * 128;      // 1024-byte aligned or not, a multiple of 128
+        MRS_CHECK(cudaMemcpyAsync(blob, plan.blob.data(), plan.blob.size(), cudaMemcpyHostToDevice, st));
+        if ((rc = tc_conv3x3_wgrad(plan, blob, part, dbpart, err, st)) != MRS_OK) return rc;
+        np = plan.np[0];
     }
-    k_dw_reduce<<<(int)((nw + cout + 31) / 32), 256, 0, st>>>(part, dbpart, np, cin, cout, gw, gb);
+    const size_t gstride = precision == MRS_PREC_FP32 ? nw : (size_t)kWgPart;
+    k_dw_reduce<<<(int)((nw + cout + 31) / 32), 256, 0, st>>>(part, dbpart, np, gstride,
+                                                              precision == MRS_PREC_FP32 ? cout : 64, cin, cout, gw, gb);
     MRS_LAUNCHED(1);
     MRS_CHECK(cudaMemcpyAsync(dw, gw, nw * 4, cudaMemcpyDeviceToHost, st));
     MRS_CHECK(cudaMemcpyAsync(db, gb, cout * 4, cudaMemcpyDeviceToHost, st));

@@ -48,4 +48,28 @@ mrs_status loss_grad_f32(const float* y, const float* tgt, size_t n, float clip,
 mrs_status adam_f32(float* p, const float* g, float* m, float* v, size_t n, float lr, int64_t step,
                     cudaStream_t st);
 
+// ---- BF16 training: weight-gradient tiles into the gradient (fuse.cu) --------
+// Where the sums of tile t of tc_conv3x3_wgrad's partials go: the gradient of
+// a layer [cout][KK][CIN] at grad + gw (KK = 9, or 1 for a 1x1 layer: the tile's
+// centre tap) and its bias at grad + gb.  Tile output o is layer output
+// o_mul o + o_add, tile input c layer input c0 + c, or, for chunk q >= 1 of a
+// deshuffled input (D steps, scale s), 64 + the deshuffled channel of (c, view
+// q - 1).  Partials 8 t .. 8 t + np - 1, summed in that order (np <= 8).
+struct WgRed {
+    int cin, cout, KK, CIN, o_mul, o_add, c0, q, s, D, with_bias, np;
+    long long gw, gb;
+};
+// d_reds: ntiles entries in device memory
+mrs_status wg_reduce(const WgRed* d_reds, int ntiles, const float* part, const float* dbpart, float* grad,
+                     cudaStream_t st);
+// channel of the D-times deshuffled map that holds channel c of HR sub-pixel
+// (oy, ox) of each s x s block: c s^2 + sum over steps d = 1..D of
+// (2 dy_d + dx_d) 4^(D - d), dy_d / dx_d bit d - 1 of oy / ox
+__host__ __device__ __forceinline__ int dsf_channel(int c, int oy, int ox, int D)
+{
+    int k = c;
+    for (int d = 1; d <= D; ++d) k = 4 * k + 2 * ((oy >> (d - 1)) & 1) + ((ox >> (d - 1)) & 1);
+    return k;
+}
+
 }  // namespace mrs

@@ -73,16 +73,6 @@ size_t rdn_nparams(int s, int c_hr)
     return L.back().boff + L.back().cout;
 }
 
-// channel of the D-times deshuffled map that holds channel c of HR sub-pixel
-// (oy, ox) of each s x s block: c s^2 + sum over steps d = 1..D of
-// (2 dy_d + dx_d) 4^(D - d), dy_d / dx_d bit d - 1 of oy / ox
-__host__ __device__ __forceinline__ int dsf_channel(int c, int oy, int ox, int D)
-{
-    int k = c;
-    for (int d = 1; d <= D; ++d) k = 4 * k + 2 * ((oy >> (d - 1)) & 1) + ((ox >> (d - 1)) & 1);
-    return k;
-}
-
 // ---- elementwise kernels ----------------------------------------------------
 // I_HRLS of one pixel: RGB, albedo, normal (+ diffuse, specular, log(1 + var))
 __device__ __forceinline__ int hr_pixel(const float* hrls, const float* alb, const float* nrm,
@@ -405,53 +395,6 @@ __global__ void k_f32_to_bf16_rows(const float* __restrict__ x, size_t P, int ci
     }
 }
 
-// One tensor-core weight-gradient tile (part [G][9][cout_t][cin_t], dbpart
-// [G][cout_t]) summed over its G partials into a layer's gradient
-// [cout][KK][cin] (KK = 9, or 1 for a 1x1 layer: tap 4 of the tile):
-// tile output o' is layer output o_mul o' + o_add, tile input c' is layer input
-// c0 + c', or, for chunk q >= 1 of the fuse conv, 64 + dsf_channel(c', oy, ox, D)
-// with q - 1 = oy s + ox.  The bias is written when with_bias.  A block takes
-// 32 consecutive values; warp w sums partials w, w + 8, ... (one coalesced
-// 128-byte row per partial), the eight sums are added in warp order: a fixed
-// order, so the result is deterministic.
-__global__ void __launch_bounds__(256) k_wg_reduce(const float* __restrict__ part,
-                                                   const float* __restrict__ dbpart, int G, int cin_t,
-                                                   int cout_t, int KK, int CIN, int o_mul, int o_add,
-                                                   int c0, int q, int s, int D, int with_bias,
-                                                   float* __restrict__ gw, float* __restrict__ gb)
-{
-    __shared__ float red[8][32];
-    const size_t nw = (size_t)cout_t * KK * cin_t, ntot = nw + (with_bias ? cout_t : 0);
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const size_t gstride = (size_t)9 * cout_t * cin_t;
-    for (size_t e0 = (size_t)blockIdx.x * 32; e0 < ntot; e0 += (size_t)gridDim.x * 32) {
-        const size_t e = e0 + lane;
-        float acc = 0.0f;
-        if (e < nw) {
-            const int c = (int)(e % cin_t), tl = (int)((e / cin_t) % KK), o = (int)(e / ((size_t)cin_t * KK));
-            const float* src = part + ((size_t)(KK == 9 ? tl : 4) * cout_t + o) * cin_t + c;
-            for (int g = wp; g < G; g += 8) acc += src[(size_t)g * gstride];
-        } else if (e < ntot) {
-            const int o = (int)(e - nw);
-            for (int g = wp; g < G; g += 8) acc += dbpart[(size_t)g * cout_t + o];
-        }
-        red[wp][lane] = acc;
-        __syncthreads();
-        if (wp == 0 && e < ntot) {
-            float v = red[0][lane];
-            for (int k = 1; k < 8; ++k) v += red[k][lane];
-            if (e < nw) {
-                const int c = (int)(e % cin_t), tl = (int)((e / cin_t) % KK), o = (int)(e / ((size_t)cin_t * KK));
-                const int ci = q > 0 ? 64 + dsf_channel(c, (q - 1) / s, (q - 1) % s, D) : c0 + c;
-                gw[((size_t)(o_mul * o + o_add) * KK + tl) * CIN + ci] = v;
-            } else {
-                gb[o_mul * (int)(e - nw) + o_add] = v;
-            }
-        }
-        __syncthreads();
-    }
-}
-
 inline int grid_for(size_t n)
 {
     size_t g = (n + 255) / 256;
@@ -504,8 +447,8 @@ struct mrs_rdn_s {
     mrs::TrainKey tkey;
     uint64_t tgraph_kernels = 0;
     cudaStream_t tcap = nullptr;        // stream they are recorded on
-    cudaStream_t side[3] = {nullptr, nullptr, nullptr};   // weight-gradient tiles side by side
-    cudaEvent_t ev_fork = nullptr, ev_join[3] = {nullptr, nullptr, nullptr};
+    mrs::WgPlan wg;                // its weight-gradient tiles
+    Buf wgblob;                    // ... as the kernel reads them, then their WgRed
     Buf tdmaps;                    // its multi-chunk A-operand maps on the device
     CUtensorMap wmap_all;          // every chunk's weights as one [rows][64] tensor
     std::vector<CUtensorMap> hmaps;  // A-operand maps of the multi-chunk convs of a call
@@ -1214,8 +1157,9 @@ mrs_status repack_if_stale(mrs_rdn_s* r, cudaStream_t st)
 // input gradients as tensor-core convs with the transposed, tap-flipped chunk
 // weights (ReLU masks as epilogues or elementwise passes, the dense parts'
 // gradients accumulated in place by residual epilogues, the shuffle and
-// deshuffle exchanged through strided views), weight gradients on k_wgrad_tc
-// per 64 x 64 tile with a fixed-order reduction into the FP32 gradient, Adam
+// deshuffle exchanged through strided views), then every layer's weight
+// gradients in one k_wgrad_tc launch over 64 x 64 tiles with a fixed-order
+// reduction into the FP32 gradient, Adam
 // on the FP32 weights.  Activations and their gradients are BF16.
 mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, const float* alb,
                           const float* nrm, const float* extra, const float* tgt, int N, int H, int W,
@@ -1243,9 +1187,10 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
             return rc;
     }
     // workspace: BF16 [P][64] tensors, then FP32
-    const size_t rows = Pl * (3 + 15 + 4 * nblk + 10) + Ph * 6 + nUrows;
-    const int maxp = tc_wgrad_max_parts();
-    const size_t nf = Ph * 6 + (size_t)maxp * 9 * 4096 + (size_t)maxp * 64 + 64 + Pl * 3 + Ph * 21;
+    const size_t rows = Pl * (3 + 15 + 4 * nblk + 4 * nblk + 5) + Ph * 4 + 2 * nUrows;
+    // tiles of the weight gradients: H_Rec, 4 per upsampling stage, 10 per block, the fuse conv's chunks, encoders
+    const size_t maxp = (size_t)8 * (1 + 4 * D + 10 * nblk + 1 + SS + 2);
+    const size_t nf = Ph * 6 + maxp * kWgPart + maxp * 64 + 64 + Pl * 3 + Ph * 21;
     if ((rc = r->trb.ensure(rows * 128 + nf * 4 + (kLossParts + 2) * 8 + 4096)) != MRS_OK) return rc;
     __nv_bfloat16* bp = r->trb.as<__nv_bfloat16>();
     auto take = [&](size_t P) { __nv_bfloat16* q = bp; bp += P * 64; return q; };
@@ -1264,12 +1209,14 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     U[0] = X[nblk];
     for (int d = 1; d <= D; ++d) U[d] = take(Pd[d]);
     __nv_bfloat16* dyb = take(Ph);
-    __nv_bfloat16* dU[2] = {take(Ph), take(Ph)};
+    __nv_bfloat16* dUl[4];                    // gradient of U[d] ([P_d][64]); level 0: dL/dF_DF
+    for (int d = 0; d <= D; ++d) dUl[d] = take(Pd[d]);
     __nv_bfloat16* G = take(Pl);              // gradient of the current block's output / input
-    __nv_bfloat16* dp[4];                     // dp[0] = G; dp[1..3]: the block's F_1..F_3 gradients
-    dp[0] = G;
-    for (int j = 1; j < 4; ++j) dp[j] = take(Pl);
-    __nv_bfloat16* dz4 = take(Pl);
+    // per block: the gradients of F_1..F_3 (dp[1..3]) and of its local fusion
+    // (dz4), kept for the weight gradients at the end; dp[0] = G
+    __nv_bfloat16* dpb[kRDG * kRDB][4];
+    for (int k = 0; k < nblk; ++k)
+        for (int j = 0; j < 4; ++j) dpb[k][j] = take(Pl);
     __nv_bfloat16* dSkip = take(Pl);
     __nv_bfloat16* dzf = take(Pl);
     __nv_bfloat16* dzlr = take(Pl);
@@ -1277,8 +1224,8 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     float* y = (float*)bp;
     float* dy = y + Ph * 3;
     float* part = dy + Ph * 3;
-    float* dbpart = part + (size_t)maxp * 9 * 4096;
-    float* zero = dbpart + (size_t)maxp * 64;   // zero biases of the input-gradient convs
+    float* dbpart = part + maxp * kWgPart;
+    float* zero = dbpart + maxp * 64;   // zero biases of the input-gradient convs
     // staging: the caller's batch, copied here every step (the recorded launches read these)
     float* sLr = zero + 64;
     float* sHr = sLr + Pl * 3;
@@ -1311,8 +1258,8 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     // tensor maps
     auto amap = [&](CUtensorMap* m, const void* q, int hh, int ww) { return tc_make_act_map(m, q, N, hh, ww, TC_BF16, kABox); };
     auto omap = [&](CUtensorMap* m, const void* q, int hh, int ww) { return tc_make_act_map(m, q, N, hh, ww, TC_BF16, kOutBox); };
-    auto xmap = [&](CUtensorMap* m, const void* q, int hh, int ww) { return tc_make_act_map(m, q, N, hh, ww, TC_BF16, kWgKB + 2); };
-    auto ymap = [&](CUtensorMap* m, const void* q, int hh, int ww) { return tc_make_act_map(m, q, N, hh, ww, TC_BF16, kWgKB); };
+    auto xmap = [&](CUtensorMap* m, const void* q, int hh, int ww) { return tc_make_wg_x_map(m, q, N, hh, ww, 128, 128LL * ww, 128LL * ww * hh); };
+    auto ymap = [&](CUtensorMap* m, const void* q, int hh, int ww) { return tc_make_wg_dy_map(m, q, N, hh, ww, 128, 128LL * ww, 128LL * ww * hh); };
     // sub-pixel (oy, ox) of every sub x sub block of a [N][HH][WW][64] tensor
     auto view = [&](CUtensorMap* m, const __nv_bfloat16* base, int sub, int oy, int ox, int HH, int WW, int box) {
         return tc_make_view_map(m, base + ((size_t)oy * WW + ox) * 64, N, HH / sub, WW / sub,
@@ -1326,8 +1273,8 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
         if (e == MRS_OK) e = ymap(&m.y, q, hh, ww);
         return e;
     };
-    M4 mInL, mInH, mFlr, mFh0, mX[kRDG * kRDB + 1], mF[kRDG * kRDB][4], mU[4], mDyb, mDU[2], mDp[4], mDz4,
-        mDzf, mDzlr, mDz1;
+    M4 mInL, mInH, mFlr, mFh0, mX[kRDG * kRDB + 1], mF[kRDG * kRDB][4], mU[4], mDyb, mDUl[4], mG,
+        mDp[kRDG * kRDB][4], mDzf, mDzlr, mDz1;   // mDp[k][0]: the local fusion's (dz4), 1..3: F_1..F_3's
     if (rc == MRS_OK) rc = all4(mInL, inL, h, w);
     if (rc == MRS_OK) rc = all4(mInH, inH, H, W);
     if (rc == MRS_OK) rc = all4(mFlr, Flr, h, w);
@@ -1337,22 +1284,25 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
         for (int j = 0; j < 4 && rc == MRS_OK; ++j) rc = all4(mF[k][j], Fk[k][j], h, w);
     for (int d = 0; d <= D && rc == MRS_OK; ++d) rc = all4(mU[d], U[d], hd[d], wd[d]);
     if (rc == MRS_OK) rc = all4(mDyb, dyb, H, W);
-    for (int j = 0; j < 4 && rc == MRS_OK; ++j) rc = all4(mDp[j], dp[j], h, w);
-    if (rc == MRS_OK) rc = all4(mDz4, dz4, h, w);
+    if (rc == MRS_OK) rc = all4(mG, G, h, w);
+    for (int k = 0; k < nblk; ++k)
+        for (int j = 0; j < 4 && rc == MRS_OK; ++j) rc = all4(mDp[k][j], dpb[k][j], h, w);
     if (rc == MRS_OK) rc = all4(mDzf, dzf, h, w);
     if (rc == MRS_OK) rc = all4(mDzlr, dzlr, h, w);
     if (rc == MRS_OK) rc = all4(mDz1, dz1, H, W);
     if (rc != MRS_OK) return rc;
-    // the level-(d + 1) gradient of the upsampling path sits in dU[(D - 1 - d) & 1]
-    // ([P_{d+1}][64]); its plain maps per level, and the deshuffle views
-    std::vector<M4> mDUl(D + 1);
-    for (int d = 0; d <= D && rc == MRS_OK; ++d) rc = all4(mDUl[d], dU[(D - d) & 1], hd[d], wd[d]);
+    for (int d = 0; d <= D && rc == MRS_OK; ++d) rc = all4(mDUl[d], dUl[d], hd[d], wd[d]);
+    auto wview = [&](CUtensorMap* m, const __nv_bfloat16* base, int sub, int oy, int ox, int HH, int WW, bool x) {
+        const __nv_bfloat16* q = base + ((size_t)oy * WW + ox) * 64;
+        return x ? tc_make_wg_x_map(m, q, N, HH / sub, WW / sub, sub * 128LL, sub * 128LL * WW, 128LL * HH * WW)
+                 : tc_make_wg_dy_map(m, q, N, HH / sub, WW / sub, sub * 128LL, sub * 128LL * WW, 128LL * HH * WW);
+    };
     std::vector<CUtensorMap> dsfA(SS), dsfO(SS), dsfX(SS), dz1O(SS);
     for (int q = 0; q < SS && rc == MRS_OK; ++q) {
         const int oy = q / s, ox = q % s;
         rc = view(&dsfA[q], Fh0, s, oy, ox, H, W, kABox);
         if (rc == MRS_OK) rc = view(&dsfO[q], Fh0, s, oy, ox, H, W, kOutBox);
-        if (rc == MRS_OK) rc = view(&dsfX[q], Fh0, s, oy, ox, H, W, kWgKB + 2);
+        if (rc == MRS_OK) rc = wview(&dsfX[q], Fh0, s, oy, ox, H, W, true);
         if (rc == MRS_OK) rc = view(&dz1O[q], dz1, s, oy, ox, H, W, kOutBox);
     }
     // upsampling stage d: output views of U[d + 1] (forward) and views of the
@@ -1361,10 +1311,10 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     for (int d = 0; d < D && rc == MRS_OK; ++d)
         for (int q = 0; q < 4 && rc == MRS_OK; ++q) {
             const int dy_ = q >> 1, dx_ = q & 1;
-            const __nv_bfloat16* g = dU[(D - 1 - d) & 1];
+            const __nv_bfloat16* g = dUl[d + 1];
             rc = view(&upO[d][q], U[d + 1], 2, dy_, dx_, hd[d + 1], wd[d + 1], kOutBox);
             if (rc == MRS_OK) rc = view(&dupA[d][q], g, 2, dy_, dx_, hd[d + 1], wd[d + 1], kABox);
-            if (rc == MRS_OK) rc = view(&dupY[d][q], g, 2, dy_, dx_, hd[d + 1], wd[d + 1], kWgKB);
+            if (rc == MRS_OK) rc = wview(&dupY[d][q], g, 2, dy_, dx_, hd[d + 1], wd[d + 1], false);
         }
     if (rc != MRS_OK) return rc;
     // multi-chunk A-operand arrays: the fuse conv's 17 inputs, each block's 4
@@ -1386,6 +1336,38 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     if ((rc = r->tdmaps.ensure(mc.size() * sizeof(CUtensorMap) + 64)) != MRS_OK) return rc;
     const CUtensorMap* dmc = r->tdmaps.as<CUtensorMap>();
     MRS_CHECK(cudaMemcpyAsync(r->tdmaps.p, mc.data(), mc.size() * sizeof(CUtensorMap),
+                              cudaMemcpyHostToDevice, st));
+
+    // the weight gradients' 64 x 64 tiles (mappings into the layer gradients: WgRed)
+    std::vector<WgTile> tiles;
+    std::vector<WgRed> reds;
+    // a conv of n tiles cuts each into sm_count / min(n, 4) runs
+    auto tile = [&](int n, const CUtensorMap& xm, const CUtensorMap& ym, int hh, int ww, int cin, int cout, int li,
+                    int o_mul, int o_add, int c0, int q, bool with_bias) {
+        const RLayer& l = r->L[li];
+        tiles.push_back(WgTile{xm, ym, N, hh, ww, cin, cout, sm_count() / (n < 4 ? n : 4)});
+        reds.push_back(WgRed{cin, cout, l.k * l.k, l.cin, o_mul, o_add, c0, q, s, D, with_bias ? 1 : 0, 0,
+                             (long long)l.woff, (long long)l.boff});
+    };
+    tile(1, mU[D].x, mDyb.y, H, W, 64, 3, nl - 1, 1, 0, 0, 0, true);
+    for (int d = D - 1; d >= 0; --d)
+        for (int q = 0; q < 4; ++q)
+            tile(4, mU[d].x, dupY[d][q], hd[d], wd[d], 64, 64, 3 + kConv * nblk + d, 4, q, 0, 0, true);
+    for (int k = nblk - 1; k >= 0; --k)
+        for (int c = kConv; c >= 1; --c)      // conv c reads the concatenation's first c parts
+            for (int j = 0; j < c; ++j)
+                tile(c, j ? mF[k][j - 1].x : mX[k].x, c == kConv ? mDp[k][0].y : mDp[k][c].y, h, w, 64, 64,
+                     3 + kConv * k + c - 1, 1, 0, 64 * j, 0, j == 0);
+    for (int q = 0; q <= SS; ++q)
+        tile(SS + 1, q ? dsfX[q - 1] : mFlr.x, mDzf.y, h, w, 64, 64, 2, 1, 0, 0, q, q == 0);
+    tile(2, mInL.x, mDzlr.y, h, w, 3, 64, 0, 1, 0, 0, 0, true);
+    tile(2, mInH.x, mDz1.y, H, W, r->c_hr, 64, 1, 1, 0, 0, 0, true);
+    if ((rc = tc_wgrad_plan(tiles, 8, r->wg)) != MRS_OK) return rc;
+    for (size_t t = 0; t < reds.size(); ++t) reds[t].np = r->wg.np[t];
+    const size_t red_off = (r->wg.blob.size() + 15) & ~(size_t)15;
+    if ((rc = r->wgblob.ensure(red_off + reds.size() * sizeof(WgRed))) != MRS_OK) return rc;
+    MRS_CHECK(cudaMemcpyAsync(r->wgblob.p, r->wg.blob.data(), r->wg.blob.size(), cudaMemcpyHostToDevice, st));
+    MRS_CHECK(cudaMemcpyAsync((uint8_t*)r->wgblob.p + red_off, reds.data(), reds.size() * sizeof(WgRed),
                               cudaMemcpyHostToDevice, st));
 
     auto body = [&](cudaStream_t st) -> mrs_status {
@@ -1454,109 +1436,46 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     MRS_LAUNCHED(1);
 
     // ---- backward
-    // Weight gradients, one 64 x 64 tile per launch (see k_wg_reduce for the
-    // mappings into the layer gradient).  A group of tiles (a conv's input
-    // parts, an upsampling conv's four views, the fuse conv's 17 chunks) runs
-    // side by side on up to kWgStreams streams, each tile on its stream's
-    // share of the SMs: at the LR grid a tile is little work, and a tile on
-    // fewer CTAs writes (and its reduction reads) that many fewer partials.
-    struct WgTile {
-        const CUtensorMap* xm;
-        const CUtensorMap* ym;
-        int hh, ww, cin_t, cout_t, lidx, o_mul, o_add, c0, q;
-        bool with_bias;
-    };
-    constexpr int kWgStreams = 4;
-    auto wgrad_group = [&](int ntile, auto tile) -> mrs_status {
-        const int S = ntile < kWgStreams ? ntile : kWgStreams;
-        const int cap = maxp / S;
-        cudaStream_t ss[kWgStreams] = {st, nullptr, nullptr, nullptr};
-        for (int i = 1; i < S; ++i) {
-            if (!r->side[i - 1]) MRS_CHECK(cudaStreamCreateWithFlags(&r->side[i - 1], cudaStreamNonBlocking));
-            if (!r->ev_join[i - 1]) MRS_CHECK(cudaEventCreateWithFlags(&r->ev_join[i - 1], cudaEventDisableTiming));
-            ss[i] = r->side[i - 1];
-        }
-        if (S > 1) {
-            if (!r->ev_fork) MRS_CHECK(cudaEventCreateWithFlags(&r->ev_fork, cudaEventDisableTiming));
-            MRS_CHECK(cudaEventRecord(r->ev_fork, st));
-            for (int i = 1; i < S; ++i) MRS_CHECK(cudaStreamWaitEvent(ss[i], r->ev_fork, 0));
-        }
-        for (int i = 0; i < ntile; ++i) {
-            const WgTile t = tile(i);
-            cudaStream_t sq = ss[i % S];
-            float* pt = part + (size_t)(i % S) * cap * 9 * 4096;
-            float* pb = dbpart + (size_t)(i % S) * cap * 64;
-            TcWgradArgs wa;
-            wa.tmap_x = t.xm; wa.tmap_dy = t.ym; wa.part = pt; wa.dbpart = pb;
-            wa.N = N; wa.H = t.hh; wa.W = t.ww; wa.cin = t.cin_t; wa.cout = t.cout_t; wa.err = r->err;
-            wa.max_ctas = cap;
-            int np = 0;
-            mrs_status e = tc_conv3x3_wgrad(wa, &np, sq);
-            if (e != MRS_OK) return e;
-            const RLayer& l = r->L[t.lidx];
-            const int KK = l.k * l.k;
-            const size_t n = (size_t)t.cout_t * KK * t.cin_t + t.cout_t;
-            k_wg_reduce<<<(int)((n + 31) / 32), 256, 0, sq>>>(pt, pb, np, t.cin_t, t.cout_t, KK, l.cin, t.o_mul,
-                                                              t.o_add, t.c0, t.q, s, D, t.with_bias ? 1 : 0,
-                                                              r->grad + l.woff, r->grad + l.boff);
-            MRS_LAUNCHED(1);
-        }
-        for (int i = 1; i < S; ++i) {
-            MRS_CHECK(cudaEventRecord(r->ev_join[i - 1], ss[i]));
-            MRS_CHECK(cudaStreamWaitEvent(st, r->ev_join[i - 1], 0));
-        }
-        return cuda_status(cudaGetLastError(), "rdn wgrad");
-    };
     auto mask = [&](const __nv_bfloat16* d, const __nv_bfloat16* act, size_t P, __nv_bfloat16* out) {
         k_mask_copy_bf16<<<grid_for(P * 64), 256, 0, st>>>(d, act, P * 64, out);
         MRS_LAUNCHED(1);
     };
     const CUtensorMap* WT = &r->wmapT_all;
     // H_Rec
-    if ((rc = wgrad_group(1, [&](int) { return WgTile{&mU[D].x, &mDyb.y, H, W, 64, 3, li_rec, 1, 0, 0, 0, true}; }))
-        != MRS_OK) return rc;
     if ((rc = conv(H, W, &mDyb.a, -1, 1, WT, trow(li_rec, 0), zero, 64, TC_LIN_BF16, nullptr, &mDUl[D].o)) != MRS_OK)
         return rc;
     // upsampling stages in reverse: the level-(d + 1) gradient masked by U[d + 1] > 0
     for (int d = D - 1; d >= 0; --d) {
         const int lu = 3 + kConv * nblk + d;
-        __nv_bfloat16* gd = dU[(D - 1 - d) & 1];
-        mask(gd, U[d + 1], Pd[d + 1], gd);
-        if ((rc = wgrad_group(4, [&](int q) {
-                 return WgTile{&mU[d].x, &dupY[d][q], hd[d], wd[d], 64, 64, lu, 4, q, 0, 0, true}; })) != MRS_OK)
-            return rc;
+        mask(dUl[d + 1], U[d + 1], Pd[d + 1], dUl[d + 1]);
         if ((rc = conv(hd[d], wd[d], &dupA[d][0], (long)mc_up[d], 4, WT, trow(lu, 0), zero, 64, TC_LIN_BF16,
                        nullptr, &mDUl[d].o)) != MRS_OK) return rc;
     }
-    __nv_bfloat16* gdf = dU[D & 1];               // dL/dF_DF: to F_G (the chain) and to F_0
+    __nv_bfloat16* gdf = dUl[0];                  // dL/dF_DF: to F_G (the chain) and to F_0
     MRS_CHECK(cudaMemcpyAsync(G, gdf, Pl * 128, cudaMemcpyDeviceToDevice, st));
     for (int g = kRDG - 1; g >= 0; --g) {
         MRS_CHECK(cudaMemcpyAsync(dSkip, G, Pl * 128, cudaMemcpyDeviceToDevice, st));
         for (int b = kRDB - 1; b >= 0; --b) {
             const int k = kRDB * g + b, lb = 3 + kConv * k;
-            // local fusion: dz4 = G masked by its ReLU output; one weight tile per
-            // concatenation part; part 0's gradient = G + conv^T, parts 1..3 start here
-            mask(G, Fk[k][3], Pl, dz4);
-            if ((rc = wgrad_group(4, [&](int j) {
-                     return WgTile{j ? &mF[k][j - 1].x : &mX[k].x, &mDz4.y, h, w, 64, 64, lb + 3, 1, 0, 64 * j, 0,
-                                   j == 0}; })) != MRS_OK) return rc;
-            if ((rc = conv(h, w, &mDz4.a, -1, 1, WT, trow(lb + 3, 0), zero, 64, TC_RESID_BF16, &mDp[0].o,
-                           &mDp[0].o)) != MRS_OK) return rc;
+            // local fusion: dz4 = G masked by its ReLU output; part 0's gradient =
+            // G + conv^T, parts 1..3 start here
+            mask(G, Fk[k][3], Pl, dpb[k][0]);
+            if ((rc = conv(h, w, &mDp[k][0].a, -1, 1, WT, trow(lb + 3, 0), zero, 64, TC_RESID_BF16, &mG.o,
+                           &mG.o)) != MRS_OK) return rc;
             for (int j = 1; j < 4; ++j)
-                if ((rc = conv(h, w, &mDz4.a, -1, 1, WT, trow(lb + 3, j), zero, 64, TC_LIN_BF16, nullptr,
-                               &mDp[j].o)) != MRS_OK) return rc;
+                if ((rc = conv(h, w, &mDp[k][0].a, -1, 1, WT, trow(lb + 3, j), zero, 64, TC_LIN_BF16, nullptr,
+                               &mDp[k][j].o)) != MRS_OK) return rc;
             // dense convs 3, 2, 1: the gradient of F_c is complete once the later
-            // convs have added theirs; masked by F_c, then its weight tiles and
-            // its input gradients added into parts 0 .. c - 1
+            // convs have added theirs; masked by F_c, then its input gradients
+            // added into parts 0 .. c - 1
             for (int c = kConv - 1; c >= 1; --c) {
                 const int lc = lb + c - 1;
-                mask(dp[c], Fk[k][c - 1], Pl, dp[c]);
-                if ((rc = wgrad_group(c, [&](int j) {
-                         return WgTile{j ? &mF[k][j - 1].x : &mX[k].x, &mDp[c].y, h, w, 64, 64, lc, 1, 0, 64 * j, 0,
-                                       j == 0}; })) != MRS_OK) return rc;
-                for (int j = 0; j < c; ++j)
-                    if ((rc = conv(h, w, &mDp[c].a, -1, 1, WT, trow(lc, j), zero, 64, TC_RESID_BF16, &mDp[j].o,
-                                   &mDp[j].o)) != MRS_OK) return rc;
+                mask(dpb[k][c], Fk[k][c - 1], Pl, dpb[k][c]);
+                for (int j = 0; j < c; ++j) {
+                    const CUtensorMap* into = j ? &mDp[k][j].o : &mG.o;
+                    if ((rc = conv(h, w, &mDp[k][c].a, -1, 1, WT, trow(lc, j), zero, 64, TC_RESID_BF16, into,
+                                   into)) != MRS_OK) return rc;
+                }
             }
         }
         // F_g = chain(F_{g-1}) + F_{g-1}
@@ -1566,9 +1485,6 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     // fuse: dz = (dL/dF_DF + the chain's gradient) masked by F_0
     k_sum_bf16<<<grid_for(Pl * 64), 256, 0, st>>>(dzf, gdf, G, nullptr, nullptr, F0, Pl * 64);
     MRS_LAUNCHED(1);
-    if ((rc = wgrad_group(SS + 1, [&](int q) {
-             return WgTile{q ? &dsfX[q - 1] : &mFlr.x, &mDzf.y, h, w, 64, 64, 2, 1, 0, 0, q, q == 0}; })) != MRS_OK)
-        return rc;
     // its input gradients, masked by the encoders' ReLU outputs: chunk 0 into
     // F_LRHS's gradient, chunk q into deshuffle view q of F0_HRLS's
     if ((rc = conv(h, w, &mDzf.a, -1, 1, WT, trow(2, 0), zero, 64, TC_MASK_BF16, &mFlr.o, &mDzlr.o)) != MRS_OK)
@@ -1576,10 +1492,11 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     for (int q = 1; q <= SS; ++q)
         if ((rc = conv(h, w, &mDzf.a, -1, 1, WT, trow(2, q), zero, 64, TC_MASK_BF16, &dsfO[q - 1],
                        &dz1O[q - 1])) != MRS_OK) return rc;
-    // encoders
-    if ((rc = wgrad_group(2, [&](int e) {
-             return e == 0 ? WgTile{&mInL.x, &mDzlr.y, h, w, 3, 64, 0, 1, 0, 0, 0, true}
-                           : WgTile{&mInH.x, &mDz1.y, H, W, r->c_hr, 64, 1, 1, 0, 0, 0, true}; })) != MRS_OK)
+    // the weight gradients of every layer in one launch, their sums in another
+    // (178 launches each, with 38 to 152 partial sums apiece, were 55% of the
+    // step's kernel time)
+    if ((rc = tc_conv3x3_wgrad(r->wg, r->wgblob.p, part, dbpart, r->err, st)) != MRS_OK) return rc;
+    if ((rc = wg_reduce((const WgRed*)((uint8_t*)r->wgblob.p + red_off), r->wg.ntiles, part, dbpart, r->grad, st)) != MRS_OK)
         return rc;
 
     return MRS_OK;
@@ -1651,15 +1568,12 @@ extern "C" mrs_status mrs_rdn_free(mrs_rdn r)
         if (p) cudaFree(p);
     if (r->tgraph) cudaGraphExecDestroy(r->tgraph);
     if (r->tcap) cudaStreamDestroy(r->tcap);
-    for (int i = 0; i < 3; ++i) {
-        if (r->side[i]) cudaStreamDestroy(r->side[i]);
-        if (r->ev_join[i]) cudaEventDestroy(r->ev_join[i]);
-    }
-    if (r->ev_fork) cudaEventDestroy(r->ev_fork);
     r->f32.release();
     r->bf.release();
     r->tr.release();
     r->trb.release();
+    r->wgblob.release();
+    r->tdmaps.release();
     r->dmaps.release();
     delete r;
     return MRS_OK;
