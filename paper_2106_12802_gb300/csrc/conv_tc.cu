@@ -113,6 +113,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
     return mbar_wait_limit(bar, parity, err, kTimeoutCycles, 1000000u);
 }
 
+// every lane polls; the answer is the same for the whole warp
+__device__ __forceinline__ bool mbar_wait_all(uint64_t* bar, uint32_t parity, int* err)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
+}
+
 // warp-wide wait: lane 0 polls, then every lane observes the completed phase
 // once (acquiring the data the phase guards)
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err)
@@ -155,7 +161,8 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, int row_bytes)
     return d;
 }
 
-// executed by the lane whose `leader` is set
+// executed by the lane whose `leader` is set; the whole warp runs the code that
+// forms the operands, so that they stay in uniform registers
 __device__ __forceinline__ void mma_f16(bool leader, uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc,
                                         uint32_t accum)
 {
@@ -492,7 +499,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         // MMA issuer: for each input row r of a piece, the blocks j whose output
         // row r + 1 - j lies in the piece, in one MMA per (dx, K step) (two
         // where the slots wrap)
-        if (lane == 0) {
+        {
+            const bool leader = lane == 0;
             bool ok = true;
             uint32_t it = 0, k = 0;
             int s = 0;                                          // ring slot of row `it`
@@ -509,7 +517,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   const int ye = min(y1, ys + maxr);
                   for (int j = 0; ok && j < kc; ++j, ++k) {
                     // weights of this pass (loaded once when kc == 1)
-                    if ((kc > 1 || k == 0) && !mbar_wait(wbar, k & 1, a.err)) { ok = false; break; }
+                    if ((kc > 1 || k == 0) && !mbar_wait_all(wbar, k & 1, a.err)) { ok = false; break; }
                     for (int r = ys - 1; ok && r <= ye; ++r, ++it, s = (s + 1 == stages ? 0 : s + 1),
                                                         ph ^= (s == 0 ? 1u : 0u)) {
                         const int jlo = max(0, r + 2 - ye), jhi = min(2, r + 1 - ys);
@@ -520,9 +528,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                             // have been read and zeroed by the epilogue of row tlo - NS
                             const int sl = (int)(tlo % NS);
                             const uint32_t use = (uint32_t)(tlo / NS);
-                            if (!mbar_wait(&sfree[(NS - sl) % NS], (use & 1) ^ 1, a.err)) { ok = false; break; }
+                            if (!mbar_wait_all(&sfree[(NS - sl) % NS], (use & 1) ^ 1, a.err)) { ok = false; break; }
                         }
-                        if (!mbar_wait(&full[s], ph, a.err)) { ok = false; break; }
+                        if (!mbar_wait_all(&full[s], ph, a.err)) { ok = false; break; }
                         tc_fence_after();
                         const int nb = jhi - jlo + 1;
                         const int c0 = (int)((NS - (int)(tlo % NS)) % NS);   // slot of block jlo
@@ -545,20 +553,20 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 for (int kk = 0; kk < KSTEPS; ++kk) {
                                     const uint64_t ad = arow + (uint64_t)((dx * ROWB + kk * 32) >> 4);
                                     const uint64_t bd = brow0 + (uint64_t)((dx * BROWS * ROWB + kk * 32) >> 4);
-                                    if (OPER == TC_BF16) mma_f16(true, tmem + dcol, ad, bd, idesc, 1u);
-                                    else mma_f8(true, tmem + dcol, ad, bd, idesc, 1u);
+                                    if (OPER == TC_BF16) mma_f16(leader, tmem + dcol, ad, bd, idesc, 1u);
+                                    else mma_f8(leader, tmem + dcol, ad, bd, idesc, 1u);
                                 }
                             }
                         }
-                        mma_commit(&empty[s]);
+                        if (leader) mma_commit(&empty[s]);
                         if (jhi == 2 && j == kc - 1) {
                             // output row r - 1 (block 2 of the last chunk) is complete
                             const long long td = tlo - (2 - jlo);
-                            mma_commit(&tfull[(NS - (int)(td % NS)) % NS]);
+                            if (leader) mma_commit(&tfull[(NS - (int)(td % NS)) % NS]);
                         }
                     }
                     // the weight buffer is free once this pass's MMAs complete
-                    if (kc > 1) mma_commit(wempty);
+                    if (kc > 1 && leader) mma_commit(wempty);
                   }
                   t0 += ye - ys;
                 }
