@@ -159,170 +159,283 @@ __global__ void k_input_q(const float* lrhs, const float* hrls, const float* alb
 }
 
 // ---- FP32 SIMT direct convolution -------------------------------------------
-// block = (8 SP) x 16 output pixels and 16 output channels (grid.z over images
-// x channel groups), 128 threads; a thread computes SP consecutive pixels of
-// one row x 16 channels (16 SP accumulators).  Input channels go through
-// shared memory in stages (8 channels for SP = 2, 4 for SP = 4, whose 64
-// accumulators leave registers for 4 blocks per SM), with a 1-pixel halo, in
-// two buffers: the asynchronous copies (cp.async, zero-filled outside the
-// image and past cin) of the next stage are in flight while the current one
-// is used.  Per (channel, kernel row) a thread reads SP + 2 inputs and, per
-// column tap, 16 weights (broadcast) for 16 SP FMAs.  The input rows are
-// padded so that a warp's reads (8 threads along x, 4 rows) fall in distinct
-// banks (SP = 4) or at most two to a bank (SP = 2).
-constexpr int kSY = 16, kSO = 16;
-constexpr int simt_pitch(int sp) { return sp == 4 ? 37 : 19; }
-constexpr int simt_stage(int sp) { return sp == 4 ? 4 : 8; }
-__device__ __forceinline__ void cp_async4(float* dst, const float* src, bool ok)
+// A block of 128 threads computes 8 OG output channels (OG = 8 or 2) of 32 x
+// (32 / OG) pixels; a thread 8 consecutive pixels of one row x 8 channels, as
+// packed pairs of channels (fma.rn.f32x2: each half rounds as fmaf does, so a
+// value's chain over input channel, kernel row and column is that of one
+// fmaf after another).  Input channels go through shared memory four at a time
+// in two buffers: the weights by asynchronous copies from a packed layout
+// ([c][tap][o], so that a thread's 8 are two 16-byte loads), the input through
+// registers (one 16-byte load per pixel, stored channel by channel: neighbouring
+// lanes store neighbouring words), both under way while the other buffer is
+// used.  Per (channel, kernel row) a thread reads 3 + 6 16-byte words for 96
+// packed FMAs; rows are 36 words apart, so a warp's input reads (4 pixel
+// groups x 4 rows) take the two wavefronts that their bytes need.  What bounds
+// it is the FMA pipe (a packed FMA holds it two cycles).  The form before (4
+// pixels x 16 channels, scalar FMAs, 4-byte copies with the channel fastest)
+// was bound by shared-memory wavefronts (86%), a third of them bank conflicts:
+// the 21-channel network on 486 x 330 7.42 -> 3.80 ms (26 -> 51 TFLOP/s of the
+// 80.5 of 152 SMs x 128 lanes), the 35 convolutions of its training step at 6 x
+// 128^2 9.40 -> 5.13 ms.  Up to 16 outputs (the 3-channel heads) run as two
+// groups of 8 on four times the rows, so that the rest is not padding.
+constexpr int kSC = 4;           // input channels per stage
+constexpr int kSX = 32;          // pixels of a block along x
+constexpr int kSPitch = 36;
+__device__ __forceinline__ void cp_async16(void* dst, const void* src)
 {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
-                     (uint32_t)__cvta_generic_to_shared(dst)),
-                 "l"(src), "r"(ok ? 4 : 0)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int kPending>
-__device__ __forceinline__ void cp_async_wait()
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+// two FP32 values in one 64-bit register pair
+typedef unsigned long long f2_t;
+__device__ __forceinline__ f2_t f2_dup(float a)
 {
-    asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
+    f2_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+    return r;
 }
+__device__ __forceinline__ f2_t f2_fma(f2_t a, f2_t b, f2_t c)
+{
+    f2_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ void f2_get(f2_t a, float& x, float& y)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a));
+}
+
+// packed weights wp[c][t][o] (c < ceil4(cin), o < cop, zero beyond cin / cout) of
+// w [cout][9][cin], or, transposed, of the gradient conv's flipped taps: its
+// inputs are w's outputs, wp[o][t][c] = w[o][8 - t][c]
+__global__ void k_pack_simt(const float* __restrict__ w, int cin, int cout, int transposed, int cop,
+                            float* __restrict__ wp)
+{
+    const int ci = transposed ? cout : cin, co = transposed ? cin : cout;
+    const int n = ((ci + 3) & ~3) * 9 * cop;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int o = i % cop, t = (i / cop) % 9, c = i / (9 * cop);
+        float v = 0.0f;
+        if (c < ci && o < co)
+            v = transposed ? w[((size_t)c * 9 + (8 - t)) * cin + o] : w[((size_t)o * 9 + t) * cin + c];
+        wp[i] = v;
+    }
+}
+
 // x [P][xs] (first cin channels read), out / res [P][os] / [P][rs] (first
 // cout written / read): strides let a layer read a prefix of a concatenation
-// buffer and write into a channel slice of another
-template <int kSP>
-__global__ void __launch_bounds__(128, kSP == 4 ? 4 : 5)
-    k_conv_simt(const float* __restrict__ x, int cin, int xs, const float* __restrict__ w,
+// buffer and write into a channel slice of another.  kVec: every pixel's
+// channels start on a 16-byte boundary and come in fours
+template <int OG, bool kVec>
+__global__ void __launch_bounds__(128, 4)
+    k_conv_simt(const float* __restrict__ x, int cin, int xs, const float* __restrict__ wp, int cop,
                 const float* __restrict__ b, int cout, int mode, int relu,
                 const float* __restrict__ res, int rs, float* __restrict__ out, int os,
                 const float* __restrict__ lrhs, int H, int W, int s)
 {
-    constexpr int kSX = 8 * kSP, kSPitch = simt_pitch(kSP), kSC = simt_stage(kSP);
-    __shared__ float sin_[2][kSC][kSY + 2][kSPitch];
-    __shared__ __align__(16) float sw[2][9][kSC][kSO];
-    const int tx = threadIdx.x % (kSX / kSP), ty = threadIdx.x / (kSX / kSP);
-    const int x0 = blockIdx.x * kSX, y0 = blockIdx.y * kSY;
-    const int ngrp = (cout + kSO - 1) / kSO;
+    constexpr int kRows = 32 / OG, kPx = (kRows + 2) * (kSX + 2), kNX = (kPx + 127) / 128;
+    constexpr int kWChunks = kSC * 9 * OG * 2;
+    __shared__ __align__(16) float sin_[2][kSC][kRows + 2][kSPitch];
+    __shared__ __align__(16) float sw[2][kSC][9][OG * 8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gx = lane & 3, ty = ((lane & 15) >> 2) + (OG == 8 ? 0 : 4 * warp);
+    const int og = (lane >> 4) + (OG == 8 ? 2 * warp : 0);
+    const int x0 = blockIdx.x * kSX, y0 = blockIdx.y * kRows;
+    const int ngrp = (cout + 8 * OG - 1) / (8 * OG);
     const int n = blockIdx.z / ngrp;
-    const int o0 = (blockIdx.z % ngrp) * kSO;
+    const int o0 = (blockIdx.z % ngrp) * 8 * OG;
     const float* xin = x + (size_t)n * H * W * xs;
-    // channels c0 .. c0 + 7 of the input tile and of the weights into buffer q
-    auto stage = [&](int c0, int q) {
-        for (int i = threadIdx.x; i < (kSY + 2) * (kSX + 2) * kSC; i += 128) {
-            const int c = i % kSC, px = (i / kSC) % (kSX + 2), py = i / (kSC * (kSX + 2));
-            const int gx = x0 + px - 1, gy = y0 + py - 1;
-            const bool ok = gx >= 0 && gx < W && gy >= 0 && gy < H && c0 + c < cin;
-            cp_async4(&sin_[q][c][py][px], ok ? xin + ((size_t)gy * W + gx) * xs + c0 + c : x, ok);
-        }
-        for (int i = threadIdx.x; i < 9 * kSC * kSO; i += 128) {
-            const int c = i % kSC, t = (i / kSC) % 9, o = i / (kSC * 9);
-            const bool ok = o0 + o < cout && c0 + c < cin;
-            cp_async4(&sw[q][t][c][o], ok ? w + ((size_t)(o0 + o) * 9 + t) * cin + c0 + c : w, ok);
-        }
-        cp_async_commit();
-    };
-    float acc[kSP][kSO];
+    float4 xr[kNX];
+    // input channels c0 .. c0 + 3 of this thread's pixels of the tile
+    auto fetch = [&](int c0) {
 #pragma unroll
-    for (int p = 0; p < kSP; ++p)
-#pragma unroll
-        for (int o = 0; o < kSO; ++o) acc[p][o] = 0.0f;
-    const int nk = (cin + kSC - 1) / kSC;
-    stage(0, 0);
-    for (int k = 0; k < nk; ++k) {
-        if (k + 1 < nk) {
-            stage((k + 1) * kSC, (k + 1) & 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-        const int q = k & 1;
-#pragma unroll 2
-        for (int c = 0; c < kSC; ++c) {
-#pragma unroll
-            for (int dy = 0; dy < 3; ++dy) {
-                const float* row = &sin_[q][c][ty + dy][tx * kSP];
-                float in[kSP + 2];
-#pragma unroll
-                for (int k2 = 0; k2 < kSP + 2; ++k2) in[k2] = row[k2];
-#pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    const float4* w4 = (const float4*)sw[q][dy * 3 + dx][c];
-                    float wv[kSO];
-#pragma unroll
-                    for (int j = 0; j < kSO / 4; ++j) {
-                        const float4 t4 = w4[j];
-                        wv[4 * j] = t4.x; wv[4 * j + 1] = t4.y; wv[4 * j + 2] = t4.z; wv[4 * j + 3] = t4.w;
-                    }
-#pragma unroll
-                    for (int p = 0; p < kSP; ++p)
-#pragma unroll
-                        for (int o = 0; o < kSO; ++o) acc[p][o] += in[p + dx] * wv[o];
+        for (int i = 0; i < kNX; ++i) {
+            const int idx = threadIdx.x + 128 * i, px = idx % (kSX + 2), py = idx / (kSX + 2);
+            const int ix = x0 + px - 1, iy = y0 + py - 1;
+            xr[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (idx < kPx && ix >= 0 && ix < W && iy >= 0 && iy < H) {
+                const float* q = xin + ((size_t)iy * W + ix) * xs + c0;
+                if (kVec) {
+                    xr[i] = __ldg((const float4*)q);
+                } else {
+                    if (c0 < cin) xr[i].x = __ldg(q);
+                    if (c0 + 1 < cin) xr[i].y = __ldg(q + 1);
+                    if (c0 + 2 < cin) xr[i].z = __ldg(q + 2);
+                    if (c0 + 3 < cin) xr[i].w = __ldg(q + 3);
                 }
             }
         }
-        // the next iteration's copies overwrite the buffer read here
+    };
+    auto put = [&](int q) {
+#pragma unroll
+        for (int i = 0; i < kNX; ++i) {
+            const int idx = threadIdx.x + 128 * i, px = idx % (kSX + 2), py = idx / (kSX + 2);
+            if (idx < kPx) {
+                sin_[q][0][py][px] = xr[i].x;
+                sin_[q][1][py][px] = xr[i].y;
+                sin_[q][2][py][px] = xr[i].z;
+                sin_[q][3][py][px] = xr[i].w;
+            }
+        }
+    };
+    auto weights = [&](int c0, int q) {
+#pragma unroll
+        for (int i = 0; i < (kWChunks + 127) / 128; ++i) {
+            const int j = threadIdx.x + 128 * i, row = j / (OG * 2), col = 4 * (j % (OG * 2));
+            if (j < kWChunks) cp_async16(&sw[q][0][0][0] + row * OG * 8 + col, wp + ((size_t)c0 * 9 + row) * cop + o0 + col);
+        }
+        cp_async_commit();
+    };
+    f2_t acc[8][4];
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) acc[p][o] = 0ull;
+    const int nk = (cin + kSC - 1) / kSC;
+    fetch(0);
+    weights(0, 0);
+    put(0);
+    cp_async_wait_all();
+    __syncthreads();
+    for (int k = 0; k < nk; ++k) {
+        const int q = k & 1;
+        if (k + 1 < nk) {
+            fetch((k + 1) * kSC);
+            weights((k + 1) * kSC, q ^ 1);
+        }
+#pragma unroll 1
+        for (int c = 0; c < kSC; ++c) {
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) {
+                const float4* row = (const float4*)&sin_[q][c][ty + dy][gx * 8];
+                const float4 r0 = row[0], r1 = row[1], r2 = row[2];
+                const float in[10] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x, r2.y};
+                f2_t in2[10];
+#pragma unroll
+                for (int i = 0; i < 10; ++i) in2[i] = f2_dup(in[i]);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+                    const ulonglong2* w2 = (const ulonglong2*)&sw[q][c][dy * 3 + dx][og * 8];
+                    const ulonglong2 wa = w2[0], wb = w2[1];
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) {
+                        acc[p][0] = f2_fma(in2[p + dx], wa.x, acc[p][0]);
+                        acc[p][1] = f2_fma(in2[p + dx], wa.y, acc[p][1]);
+                        acc[p][2] = f2_fma(in2[p + dx], wb.x, acc[p][2]);
+                        acc[p][3] = f2_fma(in2[p + dx], wb.y, acc[p][3]);
+                    }
+                }
+            }
+        }
+        if (k + 1 < nk) {
+            put(q ^ 1);
+            cp_async_wait_all();
+        }
+        // the next iteration reads what was stored here and its copies
+        // overwrite the buffer read here
         __syncthreads();
     }
     const int gy = y0 + ty;
     if (gy >= H) return;
+    const int ob = o0 + og * 8;
+    if (ob >= cout) return;
+    // 16-byte stores (and loads of res) where all 8 channels exist and are aligned
+    const bool vec = ob + 8 <= cout && (os & 3) == 0 && ((uintptr_t)out & 15) == 0 &&
+                     (!res || ((rs & 3) == 0 && ((uintptr_t)res & 15) == 0));
+    float bias[8];
 #pragma unroll
-    for (int p = 0; p < kSP; ++p) {
-        const int gx = x0 + tx * kSP + p;
-        if (gx >= W) break;
-        const size_t pp = ((size_t)n * H + gy) * W + gx;
+    for (int o = 0; o < 8; ++o) bias[o] = ob + o < cout ? __ldg(b + ob + o) : 0.0f;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        const int ix = x0 + gx * 8 + p;
+        if (ix >= W) break;
+        const size_t pp = ((size_t)n * H + gy) * W + ix;
+        float v[8];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) f2_get(acc[p][o], v[2 * o], v[2 * o + 1]);
         if (mode == SIMT_FINAL) {
             float up[3];
             const int h = H / s, wl = W / s;
-            up_pixel(lrhs + (size_t)n * h * wl * 3, h, wl, s, gx, gy, up);
-            for (int o = 0; o < kSO; ++o)
-                if (o0 + o < 3) out[pp * 3 + o0 + o] = (acc[p][o] + __ldg(b + o0 + o)) + up[o0 + o];
+            up_pixel(lrhs + (size_t)n * h * wl * 3, h, wl, s, ix, gy, up);
+#pragma unroll
+            for (int o = 0; o < 3; ++o)
+                if (ob + o < 3) out[pp * 3 + ob + o] = (v[o] + bias[o]) + up[o];
             continue;
         }
+        const float* rp = res + pp * rs + ob;
+        float* op = out + pp * os + ob;
+        float r[8];
+        const bool reads = mode == SIMT_RESID || mode == SIMT_MASK || mode == SIMT_RESRELU;
+        if (reads && vec) {
+            const float4 ra = *(const float4*)rp, rb = *(const float4*)(rp + 4);
+            r[0] = ra.x; r[1] = ra.y; r[2] = ra.z; r[3] = ra.w;
+            r[4] = rb.x; r[5] = rb.y; r[6] = rb.z; r[7] = rb.w;
+        } else if (reads) {
 #pragma unroll
-        for (int o = 0; o < kSO; ++o) {
-            if (o0 + o >= cout) break;
-            float v = acc[p][o] + __ldg(b + o0 + o);
-            if (mode == SIMT_RESID) v = res[pp * rs + o0 + o] + v;
-            else if (mode == SIMT_MASK) v = res[pp * rs + o0 + o] > 0.0f ? v : 0.0f;
-            else if (mode == SIMT_RESRELU) v = res[pp * rs + o0 + o] + fmaxf(v, 0.0f);
-            else if (relu) v = fmaxf(v, 0.0f);
-            out[pp * os + o0 + o] = v;
+            for (int o = 0; o < 8; ++o) r[o] = ob + o < cout ? rp[o] : 0.0f;
+        }
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {
+            float t = v[o] + bias[o];
+            if (mode == SIMT_RESID) t = r[o] + t;
+            else if (mode == SIMT_MASK) t = r[o] > 0.0f ? t : 0.0f;
+            else if (mode == SIMT_RESRELU) t = r[o] + fmaxf(t, 0.0f);
+            else if (relu) t = fmaxf(t, 0.0f);
+            v[o] = t;
+        }
+        if (vec) {
+            *(float4*)op = make_float4(v[0], v[1], v[2], v[3]);
+            *(float4*)(op + 4) = make_float4(v[4], v[5], v[6], v[7]);
+        } else {
+#pragma unroll
+            for (int o = 0; o < 8; ++o)
+                if (ob + o < cout) op[o] = v[o];
         }
     }
 }
 
-// Four pixels per thread (4 blocks per SM) pays on large grids, two (5 blocks
-// per SM, more warps to hide latency) below about four waves of the former
-int simt_sp(int N, int H, int W, int cout)
-{
-    const long long blocks4 = (long long)((W + 31) / 32) * ((H + kSY - 1) / kSY) * N *
-                              ((cout + kSO - 1) / kSO);
-    return blocks4 >= 16LL * sm_count() ? 4 : 2;
-}
-
 }  // namespace
 
-mrs_status simt_conv3x3(const float* x, int cin, int xs, const float* w, const float* b, int cout,
+// channels of a packed row: whole groups of the kernel that runs `cout` outputs
+static int simt_cop(int cout) { return cout > 16 ? (cout + 63) / 64 * 64 : 16; }
+size_t simt_pack_floats(int cin, int cout) { return (size_t)((cin + 3) & ~3) * 9 * simt_cop(cout); }
+
+mrs_status simt_pack(const float* w, int cin, int cout, int transposed, float* wp, cudaStream_t st)
+{
+    const int cop = simt_cop(transposed ? cin : cout);
+    const size_t n = transposed ? simt_pack_floats(cout, cin) : simt_pack_floats(cin, cout);
+    k_pack_simt<<<(int)std::min<size_t>((n + 255) / 256, 2048), 256, 0, st>>>(w, cin, cout, transposed, cop, wp);
+    MRS_LAUNCHED(1);
+    return cuda_status(cudaGetLastError(), "simt pack");
+}
+
+mrs_status simt_conv3x3(const float* x, int cin, int xs, const float* wp, const float* b, int cout,
                         int mode, int relu, const float* res, int rs, float* out, int os,
                         const float* lrhs, int N, int H, int W, int s, cudaStream_t st)
 {
-    const int sp = simt_sp(N, H, W, cout);
-    dim3 grid((W + 8 * sp - 1) / (8 * sp), (H + kSY - 1) / kSY, N * ((cout + kSO - 1) / kSO));
-    if (sp == 4)
-        MRS_TIMED(PK_CONV_SIMT, st, k_conv_simt<4><<<grid, 128, 0, st>>>(x, cin, xs, w, b, cout, mode, relu, res, rs, out, os, lrhs, H, W, s));
-    else
-        MRS_TIMED(PK_CONV_SIMT, st, k_conv_simt<2><<<grid, 128, 0, st>>>(x, cin, xs, w, b, cout, mode, relu, res, rs, out, os, lrhs, H, W, s));
+    const bool vec = (cin & 3) == 0 && (xs & 3) == 0 && ((uintptr_t)x & 15) == 0;
+    const int cop = simt_cop(cout), og = cout > 16 ? 8 : 2, rows = 32 / og;
+    const dim3 grid((W + kSX - 1) / kSX, (H + rows - 1) / rows, N * ((cout + 8 * og - 1) / (8 * og)));
+    auto launch = [&](auto kernel) {
+        kernel<<<grid, 128, 0, st>>>(x, cin, xs, wp, cop, b, cout, mode, relu, res, rs, out, os, lrhs, H, W, s);
+    };
+    if (og == 8 && vec) MRS_TIMED(PK_CONV_SIMT, st, launch(k_conv_simt<8, true>));
+    else if (og == 8) MRS_TIMED(PK_CONV_SIMT, st, launch(k_conv_simt<8, false>));
+    else if (vec) MRS_TIMED(PK_CONV_SIMT, st, launch(k_conv_simt<2, true>));
+    else MRS_TIMED(PK_CONV_SIMT, st, launch(k_conv_simt<2, false>));
     MRS_LAUNCHED(1);
     return cuda_status(cudaGetLastError(), "conv_simt launch");
 }
 
 namespace {
 
-mrs_status conv_simt(const float* x, int cin, const float* w, const float* b, int cout, int mode,
+mrs_status conv_simt(const float* x, int cin, const float* wp, const float* b, int cout, int mode,
                      int relu, const float* res, float* out, const float* lrhs, int N, int H,
                      int W, int s, cudaStream_t st)
 {
-    return simt_conv3x3(x, cin, cin, w, b, cout, mode, relu, res, cout, out, cout, lrhs, N, H, W,
+    return simt_conv3x3(x, cin, cin, wp, b, cout, mode, relu, res, cout, out, cout, lrhs, N, H, W,
                         s, st);
 }
 
@@ -505,15 +618,6 @@ __global__ void k_amax_f32(const float* __restrict__ x, size_t n, float* out)
 }
 
 // ---- training kernels (FP32) -----------------------------------------------
-// transposed-conv weights: wt[c][t][o] = w[o][8 - t][c]  (flipped taps)
-__global__ void k_wtrans(const float* __restrict__ w, int cin, int cout, float* __restrict__ wt)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cin * 9 * cout) return;
-    int o = i % cout, t = (i / cout) % 9, c = i / (cout * 9);
-    wt[i] = w[((size_t)o * 9 + (8 - t)) * cin + c];
-}
-
 // dW[o][t][c] = sum_p dy[p][o] * x[p shifted by tap t][c] (zero padded), db[o] = sum_p dy[p][o]
 // grid (G, ntaps, otiles * ctiles): block (g, j, z) reduces pixel tiles g, g+G, ... for tap
 // t = t0 + j of the 64 x 64 channel tile z = (output tile ot, input tile ct) into
@@ -743,13 +847,6 @@ mrs_status wg_reduce(const WgRed* d_reds, int ntiles, const float* part, const f
     return cuda_status(cudaGetLastError(), "wgrad reduce");
 }
 
-void wtrans_f32(const float* w, int cin, int cout, float* wt, cudaStream_t st)
-{
-    int n = cin * 9 * cout;
-    k_wtrans<<<(n + 255) / 256, 256, 0, st>>>(w, cin, cout, wt);
-    MRS_LAUNCHED(1);
-}
-
 mrs_status loss_grad_f32(const float* y, const float* tgt, size_t n, float clip, int kind,
                          float beta, float* dy, double* parts, double* sum, cudaStream_t st)
 {
@@ -874,6 +971,7 @@ using namespace mrs;
 struct mrs_net_s {
     int cin0 = 12;                 // input channels of the first conv (12 or 21)
     size_t np = kParams12;         // parameter count
+    Buf block;                     // holds the arrays below
     float* master = nullptr;       // [np]
     float* adam_m = nullptr;
     float* adam_v = nullptr;
@@ -890,6 +988,8 @@ struct mrs_net_s {
     CUtensorMap wmap_bf[kLayers], wmap_f8[kLayers], wmap_bfT[kLayers];
     __nv_bfloat16* wbfT = nullptr; // [18][9][64][64] transposed, tap-flipped (backward)
     bool bfT_valid = false;
+    float* wsimt = nullptr;        // FP32 weights as the SIMT conv reads them, layer after layer
+    bool simt_valid = false;
     Buf act;                       // activation workspace
     Buf aux;                       // small device scratch
     Buf tact;                      // training activations
@@ -937,34 +1037,49 @@ mrs_status pack_fp8(mrs_net_s* net, cudaStream_t st)
     return cuda_status(cudaGetLastError(), "pack fp8");
 }
 
+// packed FP32 weights of layer l (after pack_simt)
+size_t simt_off(mrs_net_s* net, int l) { return l ? simt_pack_floats(net->cin0, 64) + (size_t)(l - 1) * simt_pack_floats(64, 64) : 0; }
+const float* wsimt(mrs_net_s* net, int l) { return net->wsimt + simt_off(net, l); }
+mrs_status pack_simt(mrs_net_s* net, cudaStream_t st)
+{
+    if (net->simt_valid) return MRS_OK;
+    const auto& L = shapes(net->cin0);
+    mrs_status rc = MRS_OK;
+    for (int l = 0; l < kLayers && rc == MRS_OK; ++l)
+        rc = simt_pack(net->master + L[l].woff, L[l].cin, L[l].cout, 0, net->wsimt + simt_off(net, l), st);
+    net->simt_valid = rc == MRS_OK && !recording(st);
+    return rc;
+}
+
 mrs_status fuse_f32(mrs_net_s* net, const float* lrhs, const float* hrls, const float* alb,
                     const float* nrm, const float* extra, int N, int H, int W, int s, float* out,
                     cudaStream_t st)
 {
     size_t P = (size_t)N * H * W;
     const int c0 = net->cin0;
-    mrs_status rc = net->act.ensure(P * (c0 + 64 + 64) * 4);
+    mrs_status rc = net->act.ensure(P * (c0 + 64 + 64) * 4 + 16);
     if (rc != MRS_OK) return rc;
+    if ((rc = pack_simt(net, st)) != MRS_OK) return rc;
     float* x0 = net->act.as<float>();
-    float* h = x0 + P * c0;
+    float* h = x0 + ((P * c0 + 3) & ~(size_t)3);     // 16-byte aligned
     float* r = h + P * 64;
     const auto& L = shapes(net->cin0);
     k_input_f32<<<(int)((P + 255) / 256 < 65535 ? (P + 255) / 256 : 65535), 256, 0, st>>>(
         lrhs, hrls, alb, nrm, extra, H, W, s, P, x0);
     MRS_LAUNCHED(1);
-    rc = conv_simt(x0, c0, net->master + L[0].woff, net->master + L[0].boff, 64, SIMT_PLAIN, 1,
+    rc = conv_simt(x0, c0, wsimt(net, 0), net->master + L[0].boff, 64, SIMT_PLAIN, 1,
                    nullptr, h, nullptr, N, H, W, s, st);
     for (int k = 0; k < 8 && rc == MRS_OK; ++k) {
         const LayerShape& a = L[1 + 2 * k];
         const LayerShape& b = L[2 + 2 * k];
-        rc = conv_simt(h, 64, net->master + a.woff, net->master + a.boff, 64, SIMT_PLAIN, 1,
+        rc = conv_simt(h, 64, wsimt(net, 1 + 2 * k), net->master + a.boff, 64, SIMT_PLAIN, 1,
                        nullptr, r, nullptr, N, H, W, s, st);
         if (rc == MRS_OK)
-            rc = conv_simt(r, 64, net->master + b.woff, net->master + b.boff, 64, SIMT_RESID, 0, h,
+            rc = conv_simt(r, 64, wsimt(net, 2 + 2 * k), net->master + b.boff, 64, SIMT_RESID, 0, h,
                            h, nullptr, N, H, W, s, st);
     }
     if (rc == MRS_OK)
-        rc = conv_simt(h, 64, net->master + L[17].woff, net->master + L[17].boff, 3, SIMT_FINAL, 0,
+        rc = conv_simt(h, 64, wsimt(net, 17), net->master + L[17].boff, 3, SIMT_FINAL, 0,
                        nullptr, out, lrhs, N, H, W, s, st);
     return rc;
 }
@@ -1095,9 +1210,9 @@ extern "C" mrs_status mrs_net_create(const float* params, int32_t n_params, mrs_
     net->np = (size_t)n_params;
     net->cin0 = n_params == (int32_t)kParams21 ? 21 : 12;
     mrs_status s = MRS_OK;
-    auto alloc = [&](void** p, size_t bytes) {
-        if (s == MRS_OK) s = cuda_status(cudaMalloc(p, bytes), "cudaMalloc(net)");
-    };
+    // one allocation, carved up (a cudaMalloc each was most of the call)
+    std::vector<std::pair<void**, size_t>> parts;
+    auto alloc = [&](void** p, size_t bytes) { parts.push_back({p, (bytes + 255) & ~(size_t)255}); };
     alloc((void**)&net->master, net->np * 4);
     alloc((void**)&net->adam_m, net->np * 4);
     alloc((void**)&net->adam_v, net->np * 4);
@@ -1109,6 +1224,14 @@ extern "C" mrs_status mrs_net_create(const float* params, int32_t n_params, mrs_
     alloc((void**)&net->bias8, kLayers * 64 * 4);
     alloc((void**)&net->wscale, kLayers * 64 * 4);
     alloc((void**)&net->err, 4);
+    alloc((void**)&net->wsimt, (simt_off(net, kLayers - 1) + simt_pack_floats(64, 3)) * 4);
+    size_t total = 0;
+    for (const auto& p : parts) total += p.second;
+    s = net->block.ensure(total);
+    if (s == MRS_OK) {
+        uint8_t* q = net->block.as<uint8_t>();
+        for (const auto& p : parts) { *p.first = q; q += p.second; }
+    }
     if (s == MRS_OK) s = mrs_net_set_params(net, params);
     if (s != MRS_OK) { mrs_net_free(net); return s; }
     *out = net;
@@ -1119,10 +1242,7 @@ extern "C" mrs_status mrs_net_free(mrs_net net)
 {
     if (!net) return MRS_OK;
     cudaDeviceSynchronize();
-    void* ptrs[] = {net->master, net->adam_m, net->adam_v, net->grad, net->wbf, net->wbfT, net->wf8,
-                    net->bias, net->bias8, net->wscale, net->err};
-    for (void* p : ptrs)
-        if (p) cudaFree(p);
+    net->block.release();
     net->act.release();
     net->aux.release();
     net->tact.release();
@@ -1139,7 +1259,7 @@ extern "C" mrs_status mrs_net_set_params(mrs_net net, const float* params)
     MRS_CHECK(cudaMemset(net->adam_v, 0, net->np * 4));
     MRS_CHECK(cudaMemset(net->err, 0, 4));
     net->step = 0;
-    net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = false;
+    net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = net->simt_valid = false;
     return MRS_OK;
 }
 
@@ -1324,7 +1444,7 @@ extern "C" mrs_status mrs_conv3x3(const float* x, int32_t N, int32_t H, int32_t 
         return conv3x3_chunked(S, x, N, H, W, cin, cout, w, b, relu, out, st);
     size_t wbytes = (size_t)cout * 9 * cin * 4;
     size_t need = wbytes + cout * 4 + 9 * 64 * 64 * 2 + 64 * 4 * 2 + 1024 +
-                  (precision == MRS_PREC_FP32 ? 0 : P * 128) + 16;
+                  (precision == MRS_PREC_FP32 ? simt_pack_floats(cin, cout) * 4 : P * 128) + 16;
     mrs_status rc = S.b.ensure(need);
     if (rc != MRS_OK) return rc;
     uint8_t* base = S.b.as<uint8_t>();
@@ -1334,7 +1454,8 @@ extern "C" mrs_status mrs_conv3x3(const float* x, int32_t N, int32_t H, int32_t 
     MRS_CHECK(cudaMemcpyAsync(dw, w, wbytes, cudaMemcpyHostToDevice, st));
     MRS_CHECK(cudaMemcpyAsync(db, b, cout * 4, cudaMemcpyHostToDevice, st));
     if (precision == MRS_PREC_FP32) {
-        rc = conv_simt(x, cin, dw, db, cout, SIMT_PLAIN, relu, nullptr, out, nullptr, N, H, W, 1, st);
+        if ((rc = simt_pack(dw, cin, cout, 0, (float*)q, st)) != MRS_OK) return rc;
+        rc = conv_simt(x, cin, (const float*)q, db, cout, SIMT_PLAIN, relu, nullptr, out, nullptr, N, H, W, 1, st);
         if (rc == MRS_OK) rc = cuda_status(cudaStreamSynchronize(st), "conv3x3 sync");
         return rc;
     }
@@ -1425,9 +1546,8 @@ mrs_status layer_dx(mrs_net_s* net, int l, const float* dy, float* wt, const flo
                     int mode, const float* res, float* dx, int N, int H, int W, cudaStream_t st)
 {
     const LayerShape& L = shapes(net->cin0)[l];
-    int n = L.cin * 9 * L.cout;
-    k_wtrans<<<(n + 255) / 256, 256, 0, st>>>(net->master + L.woff, L.cin, L.cout, wt);
-    MRS_LAUNCHED(1);
+    mrs_status rc = simt_pack(net->master + L.woff, L.cin, L.cout, 1, wt, st);
+    if (rc != MRS_OK) return rc;
     return conv_simt(dy, L.cout, wt, zero, L.cin, mode, 0, res, dx, nullptr, N, H, W, 1, st);
 }
 
@@ -1440,18 +1560,18 @@ mrs_status train_step_f32(mrs_net_s* net, const float* lrhs, const float* hrls, 
     const size_t F = P * 64;
     const size_t nlr = (size_t)N * (H / s) * (W / s) * 3;
     // activations: x0 | h0..h8 | r0..r7 | y | dy | dh | da | lrhs_clipped
-    size_t need = (P * c0 + 9 * F + 8 * F + 2 * P * 3 + 2 * F + nlr) * 4;
+    size_t need = (P * c0 + 9 * F + 8 * F + 2 * P * 3 + 2 * F + nlr) * 4 + 32;
     mrs_status rc = net->tact.ensure(need);
     if (rc != MRS_OK) return rc;
     size_t tneed = (64 * 9 * 64 + 64) * 4 + ((size_t)kDwSplits * 9 * 64 * 64 + kDwSplits * 64) * 4 +
                    (kRedBlocks + 8) * 8;
     if ((rc = net->ttmp.ensure(tneed)) != MRS_OK) return rc;
     float* x0 = net->tact.as<float>();
-    float* hs = x0 + P * c0;
+    float* hs = x0 + ((P * c0 + 3) & ~(size_t)3);    // 16-byte aligned
     float* rs = hs + 9 * F;
     float* y = rs + 8 * F;
     float* dy = y + P * 3;
-    float* dh = dy + P * 3;
+    float* dh = y + ((2 * P * 3 + 3) & ~(size_t)3);
     float* da = dh + F;
     float* lrc = da + F;
     float* wt = net->ttmp.as<float>();
@@ -1463,24 +1583,25 @@ mrs_status train_step_f32(mrs_net_s* net, const float* lrhs, const float* hrls, 
     MRS_CHECK(cudaMemsetAsync(zero, 0, 64 * 4, st));
     const auto& L = shapes(net->cin0);
     const float* M = net->master;
+    if ((rc = pack_simt(net, st)) != MRS_OK) return rc;
 
     // forward, keeping every activation the backward needs
     k_clip_copy<<<grid1d(nlr), 256, 0, st>>>(lrhs, nlr, kClip, lrc);
     MRS_LAUNCHED(1);
     k_input_f32<<<grid1d(P), 256, 0, st>>>(lrc, hrls, alb, nrm, extra, H, W, s, P, x0, kClip);
     MRS_LAUNCHED(1);
-    rc = conv_simt(x0, c0, M + L[0].woff, M + L[0].boff, 64, SIMT_PLAIN, 1, nullptr, hs, nullptr, N, H, W, s, st);
+    rc = conv_simt(x0, c0, wsimt(net, 0), M + L[0].boff, 64, SIMT_PLAIN, 1, nullptr, hs, nullptr, N, H, W, s, st);
     for (int k = 0; k < 8 && rc == MRS_OK; ++k) {
         const LayerShape& a = L[1 + 2 * k];
         const LayerShape& b = L[2 + 2 * k];
-        rc = conv_simt(hs + k * F, 64, M + a.woff, M + a.boff, 64, SIMT_PLAIN, 1, nullptr, rs + k * F,
+        rc = conv_simt(hs + k * F, 64, wsimt(net, 1 + 2 * k), M + a.boff, 64, SIMT_PLAIN, 1, nullptr, rs + k * F,
                        nullptr, N, H, W, s, st);
         if (rc == MRS_OK)
-            rc = conv_simt(rs + k * F, 64, M + b.woff, M + b.boff, 64, SIMT_RESID, 0, hs + k * F,
+            rc = conv_simt(rs + k * F, 64, wsimt(net, 2 + 2 * k), M + b.boff, 64, SIMT_RESID, 0, hs + k * F,
                            hs + (k + 1) * F, nullptr, N, H, W, s, st);
     }
     if (rc == MRS_OK)
-        rc = conv_simt(hs + 8 * F, 64, M + L[17].woff, M + L[17].boff, 3, SIMT_FINAL, 0, nullptr, y, lrc,
+        rc = conv_simt(hs + 8 * F, 64, wsimt(net, 17), M + L[17].boff, 3, SIMT_FINAL, 0, nullptr, y, lrc,
                        N, H, W, s, st);
     if (rc != MRS_OK) return rc;
 
@@ -1513,7 +1634,7 @@ mrs_status train_step_f32(mrs_net_s* net, const float* lrhs, const float* hrls, 
     MRS_TIMED(PK_TRAIN, st, k_adam<<<grid1d(net->np), 256, 0, st>>>(net->master, net->grad, net->adam_m, net->adam_v,
                                                         net->np, lr, (float)b1, (float)b2, 1e-8f, bc1, bc2));
     MRS_LAUNCHED(1);
-    net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = false;
+    net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = net->simt_valid = false;
     if (loss_out) {
         double h = 0;
         MRS_CHECK(cudaMemcpyAsync(&h, lres, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1701,7 +1822,7 @@ mrs_status train_step_bf16(mrs_net_s* net, const float* lrhs, const float* hrls,
     MRS_TIMED(PK_TRAIN, st, k_adam<<<grid1d(net->np), 256, 0, st>>>(net->master, net->grad, net->adam_m, net->adam_v,
                                                         net->np, lr, (float)b1, (float)b2, 1e-8f, bc1, bc2));
     MRS_LAUNCHED(1);
-    net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = false;
+    net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = net->simt_valid = false;
     if (loss_out) {
         double h = 0;
         MRS_CHECK(cudaMemcpyAsync(&h, lres, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1773,7 +1894,7 @@ extern "C" mrs_status mrs_net_set_state(mrs_net net, const float* params, const 
     MRS_CHECK(cudaMemcpy(net->adam_m, adam_m, net->np * 4, cudaMemcpyHostToDevice));
     MRS_CHECK(cudaMemcpy(net->adam_v, adam_v, net->np * 4, cudaMemcpyHostToDevice));
     net->step = step;
-    net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = false;
+    net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = net->simt_valid = false;
     return MRS_OK;
 }
 
@@ -2066,8 +2187,7 @@ extern "C" mrs_status mrs_conv3x3_dgrad(const float* dy, int32_t N, int32_t H, i
         // the FP32 training step's transposed conv: flipped, transposed
         // weights through the SIMT convolution with the step's epilogues
         float* wt = (float*)q;
-        k_wtrans<<<(int)((nw + 255) / 256), 256, 0, st>>>(dw, cin, cout, wt);
-        MRS_LAUNCHED(1);
+        if ((rc = simt_pack(dw, cin, cout, 1, wt, st)) != MRS_OK) return rc;
         int sm = mode == MRS_DGRAD_LINEAR ? SIMT_PLAIN : mode == MRS_DGRAD_RELU_MASK ? SIMT_MASK : SIMT_RESID;
         rc = conv_simt(dy, cout, wt, zero, cin, sm, 0, aux, out, nullptr, N, H, W, 1, st);
         if (rc == MRS_OK) rc = cuda_status(cudaStreamSynchronize(st), "conv3x3 dgrad sync");

@@ -16,10 +16,24 @@ enum SimtMode {
     SIMT_RESRELU = 4,  // out = res + relu(acc + b)
 };
 
+// whether launches on st are being recorded: what they would write does not
+// exist yet when the recording call returns
+inline bool recording(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
+}
+
 // FP32 3x3 convolution with zero padding 1 on [N][H][W][.] tensors:
 // out[p][o] (o < cout, pixel stride os) from x[p][c] (c < cin, pixel stride
-// xs); res has pixel stride rs.  Asynchronous on st.
-mrs_status simt_conv3x3(const float* x, int cin, int xs, const float* w, const float* b, int cout,
+// xs) with the weights that simt_pack packed (16-byte aligned,
+// simt_pack_floats(cin, cout) floats); res has pixel stride rs.  Asynchronous
+// on st.
+size_t simt_pack_floats(int cin, int cout);
+// w [cout][9][cin]; transposed: for the gradient with respect to the input
+// (inputs cout, outputs cin, taps flipped; simt_pack_floats(cout, cin) floats)
+mrs_status simt_pack(const float* w, int cin, int cout, int transposed, float* wp, cudaStream_t st);
+mrs_status simt_conv3x3(const float* x, int cin, int xs, const float* wp, const float* b, int cout,
                         int mode, int relu, const float* res, int rs, float* out, int os,
                         const float* lrhs, int N, int H, int W, int s, cudaStream_t st);
 
@@ -37,8 +51,6 @@ constexpr int kLossParts = 1024;   // float64 partial sums of loss_grad_f32
 // g are left to the caller.
 mrs_status dw_tiles_f32(const float* x, int cin, int xs, const float* dy, int cout, int ys, int N,
                         int H, int W, int centre_only, float* part, float* dbpart, cudaStream_t st);
-// transposed-conv weights wt[c][t][o] = w[o][8 - t][c] (w [cout][9][cin])
-void wtrans_f32(const float* w, int cin, int cout, float* wt, cudaStream_t st);
 // training loss (MRS_LOSS_*) of y against min(target, clip) over n values:
 // dy = dL/dy, *sum (device double) = the sum of the per-value losses,
 // parts = kLossParts doubles of scratch

@@ -454,6 +454,9 @@ struct mrs_rdn_s {
     std::vector<CUtensorMap> hmaps;  // A-operand maps of the multi-chunk convs of a call
     Buf dmaps;                     // their device copy
     Buf f32, bf;                   // activation workspaces
+    Buf simt;                      // FP32 weights as the SIMT conv reads them
+    std::vector<size_t> simt_off;  // ... of each layer (floats)
+    bool simt_valid = false;
     int* err = nullptr;
     // training state (allocated by the first training step)
     float* grad = nullptr;         // gradient of the last step (parameter layout)
@@ -550,6 +553,28 @@ mrs_status pack_chunks(mrs_rdn_s* r, const float* P)
     return tc_make_w_map(&r->wmap_all, r->wbf, (int)(wb.size() / 64), 64, TC_BF16);
 }
 
+// every layer's packed FP32 weights (the 1x1 fuse conv as a centre tap)
+mrs_status pack_simt(mrs_rdn_s* r, cudaStream_t st)
+{
+    if (r->simt_valid) return MRS_OK;
+    size_t n = 0;
+    r->simt_off.clear();
+    for (const RLayer& l : r->L) {
+        r->simt_off.push_back(n);
+        n += simt_pack_floats(l.cin, l.cout);
+    }
+    mrs_status rc = r->simt.ensure(n * 4);
+    if (rc != MRS_OK) return rc;
+    k_centre_tap<<<grid_for((size_t)64 * 9 * r->L[2].cin), 256, 0, st>>>(r->master + r->L[2].woff, r->L[2].cin, r->w_fuse3);
+    MRS_LAUNCHED(1);
+    for (size_t li = 0; li < r->L.size() && rc == MRS_OK; ++li) {
+        const RLayer& l = r->L[li];
+        rc = simt_pack(li == 2 ? r->w_fuse3 : r->master + l.woff, l.cin, l.cout, 0, r->simt.as<float>() + r->simt_off[li], st);
+    }
+    r->simt_valid = rc == MRS_OK && !recording(st);
+    return rc;
+}
+
 mrs_status rdn_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, const float* alb,
                    const float* nrm, const float* extra, int N, int H, int W, float* out,
                    cudaStream_t st)
@@ -572,23 +597,23 @@ mrs_status rdn_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, const flo
     float* T = Pg + Pl * 64;
     float* U = T + nT;
     const float* M = r->master;
+    if ((rc = pack_simt(r, st)) != MRS_OK) return rc;
+    auto WP = [&](size_t li) { return r->simt.as<float>() + r->simt_off[li]; };
     const auto& L = r->L;
 
     k_hr_input_f32<<<grid_for(Ph), 256, 0, st>>>(hrls, alb, nrm, extra, Ph, inH);
     MRS_LAUNCHED(1);
     // F_LRHS into cat[:, 0:64]; F0_HRLS; deshuffle into cat[:, 64:]
-    rc = simt_conv3x3(lrhs, 3, 3, M + L[0].woff, M + L[0].boff, kF, SIMT_PLAIN, 1, nullptr, 0, cat,
+    rc = simt_conv3x3(lrhs, 3, 3, WP(0), M + L[0].boff, kF, SIMT_PLAIN, 1, nullptr, 0, cat,
                       Ccat, nullptr, N, h, w, 1, st);
     if (rc == MRS_OK)
-        rc = simt_conv3x3(inH, r->c_hr, r->c_hr, M + L[1].woff, M + L[1].boff, kF, SIMT_PLAIN, 1,
+        rc = simt_conv3x3(inH, r->c_hr, r->c_hr, WP(1), M + L[1].boff, kF, SIMT_PLAIN, 1,
                           nullptr, 0, Fh0, kF, nullptr, N, H, W, 1, st);
     if (rc != MRS_OK) return rc;
     k_deshuffle_f32<<<grid_for(Ph * 64), 256, 0, st>>>(Fh0, N, H, W, s, D, cat, Ccat);
     MRS_LAUNCHED(1);
-    k_centre_tap<<<grid_for((size_t)64 * 9 * Ccat), 256, 0, st>>>(M + L[2].woff, Ccat, r->w_fuse3);
-    MRS_LAUNCHED(1);
     // F_0 = relu(fuse(cat)) into A[:, 0:64] and F0
-    rc = simt_conv3x3(cat, Ccat, Ccat, r->w_fuse3, M + L[2].boff, kF, SIMT_PLAIN, 1, nullptr, 0, A,
+    rc = simt_conv3x3(cat, Ccat, Ccat, WP(2), M + L[2].boff, kF, SIMT_PLAIN, 1, nullptr, 0, A,
                       256, nullptr, N, h, w, 1, st);
     if (rc != MRS_OK) return rc;
     k_ch64_f32<<<grid_for(Pl * 64), 256, 0, st>>>(F0, 64, A, 256, Pl, 0);
@@ -599,10 +624,10 @@ mrs_status rdn_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, const flo
         MRS_LAUNCHED(1);
         for (int b = 0; b < kRDB && rc == MRS_OK; ++b) {
             for (int c = 1; c < kConv && rc == MRS_OK; ++c, ++li)
-                rc = simt_conv3x3(A, kF * c, 256, M + L[li].woff, M + L[li].boff, kF, SIMT_PLAIN, 1,
+                rc = simt_conv3x3(A, kF * c, 256, WP(li), M + L[li].boff, kF, SIMT_PLAIN, 1,
                                   nullptr, 0, A + kF * c, 256, nullptr, N, h, w, 1, st);
             if (rc != MRS_OK) break;
-            rc = simt_conv3x3(A, 256, 256, M + L[li].woff, M + L[li].boff, kF, SIMT_RESRELU, 0, A,
+            rc = simt_conv3x3(A, 256, 256, WP(li), M + L[li].boff, kF, SIMT_RESRELU, 0, A,
                               256, B, 256, nullptr, N, h, w, 1, st);
             ++li;
             float* t = A;
@@ -620,7 +645,7 @@ mrs_status rdn_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, const flo
     int cs = 256, ch = h, cw = w;
     float* dst = U;
     for (int d = 0; d < D && rc == MRS_OK; ++d, ++li) {
-        rc = simt_conv3x3(cur, kF, cs, M + L[li].woff, M + L[li].boff, 4 * kF, SIMT_PLAIN, 1,
+        rc = simt_conv3x3(cur, kF, cs, WP(li), M + L[li].boff, 4 * kF, SIMT_PLAIN, 1,
                           nullptr, 0, T, 256, nullptr, N, ch, cw, 1, st);
         if (rc != MRS_OK) break;
         k_shuffle_f32<<<grid_for((size_t)N * 4 * ch * cw * 64), 256, 0, st>>>(T, 256, N, ch, cw, dst);
@@ -632,7 +657,7 @@ mrs_status rdn_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, const flo
         dst = dst == U ? Fh0 : U;
     }
     if (rc != MRS_OK) return rc;
-    rc = simt_conv3x3(cur, kF, kF, M + L[li].woff, M + L[li].boff, 3, SIMT_PLAIN, 0, nullptr, 0, out,
+    rc = simt_conv3x3(cur, kF, kF, WP(li), M + L[li].boff, 3, SIMT_PLAIN, 0, nullptr, 0, out,
                       3, nullptr, N, H, W, 1, st);
     if (rc != MRS_OK) return rc;
     return cuda_status(cudaGetLastError(), "rdn fp32");
@@ -907,23 +932,23 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
     auto X = [&](int k) { return blk + (size_t)k * Pl * 256; };
     auto Rk = [&](int k) { return R + (size_t)k * Pl * 64; };
     const float* M = r->master;
+    if ((rc = pack_simt(r, st)) != MRS_OK) return rc;
+    auto WP = [&](size_t li) { return r->simt.as<float>() + r->simt_off[li]; };
     const auto& L = r->L;
     MRS_CHECK(cudaMemsetAsync(zero, 0, (size_t)Ccat * 4, st));
 
     // ---- forward with the tape
     k_hr_input_f32<<<grid_for(Ph), 256, 0, st>>>(hrls, alb, nrm, extra, Ph, inH);
     MRS_LAUNCHED(1);
-    rc = simt_conv3x3(lrhs, 3, 3, M + L[0].woff, M + L[0].boff, kF, SIMT_PLAIN, 1, nullptr, 0, cat,
+    rc = simt_conv3x3(lrhs, 3, 3, WP(0), M + L[0].boff, kF, SIMT_PLAIN, 1, nullptr, 0, cat,
                       Ccat, nullptr, N, h, w, 1, st);
     if (rc == MRS_OK)
-        rc = simt_conv3x3(inH, c_hr, c_hr, M + L[1].woff, M + L[1].boff, kF, SIMT_PLAIN, 1, nullptr,
+        rc = simt_conv3x3(inH, c_hr, c_hr, WP(1), M + L[1].boff, kF, SIMT_PLAIN, 1, nullptr,
                           0, Fh0, kF, nullptr, N, H, W, 1, st);
     if (rc != MRS_OK) return rc;
     k_deshuffle_f32<<<grid_for(Ph * 64), 256, 0, st>>>(Fh0, N, H, W, s, D, cat, Ccat);
     MRS_LAUNCHED(1);
-    k_centre_tap<<<grid_for((size_t)64 * 9 * Ccat), 256, 0, st>>>(M + L[2].woff, Ccat, r->w_fuse3);
-    MRS_LAUNCHED(1);
-    rc = simt_conv3x3(cat, Ccat, Ccat, r->w_fuse3, M + L[2].boff, kF, SIMT_PLAIN, 1, nullptr, 0, F0,
+    rc = simt_conv3x3(cat, Ccat, Ccat, WP(2), M + L[2].boff, kF, SIMT_PLAIN, 1, nullptr, 0, F0,
                       kF, nullptr, N, h, w, 1, st);
     if (rc != MRS_OK) return rc;
     k_ch64_f32<<<grid_for(Pl * 64), 256, 0, st>>>(X(0), 256, F0, 64, Pl, 0);
@@ -935,10 +960,10 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
             const int k = kRDB * g + b;
             float* x = X(k);
             for (int c = 1; c < kConv && rc == MRS_OK; ++c, ++li)
-                rc = simt_conv3x3(x, kF * c, 256, M + L[li].woff, M + L[li].boff, kF, SIMT_PLAIN, 1,
+                rc = simt_conv3x3(x, kF * c, 256, WP(li), M + L[li].boff, kF, SIMT_PLAIN, 1,
                                   nullptr, 0, x + kF * c, 256, nullptr, N, h, w, 1, st);
             if (rc == MRS_OK)
-                rc = simt_conv3x3(x, 256, 256, M + L[li].woff, M + L[li].boff, kF, SIMT_PLAIN, 1,
+                rc = simt_conv3x3(x, 256, 256, WP(li), M + L[li].boff, kF, SIMT_PLAIN, 1,
                                   nullptr, 0, Rk(k), 64, nullptr, N, h, w, 1, st);
             if (rc != MRS_OK) return rc;
             ++li;
@@ -954,7 +979,7 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
     }
     int ch = h, cw = w;
     for (int d = 0; d < D; ++d, ++li) {
-        rc = simt_conv3x3(U[d], kF, kF, M + L[li].woff, M + L[li].boff, 4 * kF, SIMT_PLAIN, 1, nullptr,
+        rc = simt_conv3x3(U[d], kF, kF, WP(li), M + L[li].boff, 4 * kF, SIMT_PLAIN, 1, nullptr,
                           0, T[d], 256, nullptr, N, ch, cw, 1, st);
         if (rc != MRS_OK) return rc;
         k_shuffle_f32<<<grid_for(Pd[d + 1] * 64), 256, 0, st>>>(T[d], 256, N, ch, cw, U[d + 1]);
@@ -962,7 +987,7 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
         ch *= 2;
         cw *= 2;
     }
-    rc = simt_conv3x3(U[D], kF, kF, M + L[li].woff, M + L[li].boff, 3, SIMT_PLAIN, 0, nullptr, 0, y, 3,
+    rc = simt_conv3x3(U[D], kF, kF, WP(li), M + L[li].boff, 3, SIMT_PLAIN, 0, nullptr, 0, y, 3,
                       nullptr, N, H, W, 1, st);
     if (rc != MRS_OK) return rc;
     if (yout) MRS_CHECK(cudaMemcpyAsync(yout, y, Ph * 3 * 4, cudaMemcpyDeviceToDevice, st));
@@ -973,7 +998,7 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
 
     // ---- backward: H_Rec, then the upsampling convs through the shuffles
     if ((rc = layer_grad(r, li, U[D], kF, dy, 3, N, H, W, part, dbpart, st)) != MRS_OK) return rc;
-    wtrans_f32(M + L[li].woff, kF, 3, wt, st);
+    if ((rc = simt_pack(M + L[li].woff, kF, 3, 1, wt, st)) != MRS_OK) return rc;
     rc = simt_conv3x3(dy, 3, 3, wt, zero, kF, SIMT_PLAIN, 0, nullptr, 0, dA, kF, nullptr, N, H, W, 1, st);
     if (rc != MRS_OK) return rc;
     for (int d = D - 1; d >= 0; --d) {
@@ -983,7 +1008,7 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
         k_unshuffle_mask<<<grid_for(Pd[d] * 256), 256, 0, st>>>(dA, T[d], N, ch, cw, dB);
         MRS_LAUNCHED(1);
         if ((rc = layer_grad(r, li, U[d], kF, dB, 256, N, ch, cw, part, dbpart, st)) != MRS_OK) return rc;
-        wtrans_f32(M + L[li].woff, kF, 4 * kF, wt, st);
+        if ((rc = simt_pack(M + L[li].woff, kF, 4 * kF, 1, wt, st)) != MRS_OK) return rc;
         rc = simt_conv3x3(dB, 4 * kF, 4 * kF, wt, zero, kF, SIMT_PLAIN, 0, nullptr, 0, dA, kF, nullptr,
                           N, ch, cw, 1, st);
         if (rc != MRS_OK) return rc;
@@ -1003,7 +1028,7 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
             MRS_LAUNCHED(1);
             // local fusion: dCat[:, 0:256] += conv^T(dz)
             if ((rc = layer_grad(r, lb + 3, x, 256, dz, kF, N, h, w, part, dbpart, st)) != MRS_OK) return rc;
-            wtrans_f32(M + L[lb + 3].woff, 256, kF, wt, st);
+            if ((rc = simt_pack(M + L[lb + 3].woff, 256, kF, 1, wt, st)) != MRS_OK) return rc;
             rc = simt_conv3x3(dz, kF, kF, wt, zero, 256, SIMT_RESID, 0, dCat, 256, dCat, 256, nullptr, N,
                               h, w, 1, st);
             // dense conv c: its output's gradient (channels 64 (c + 1) ..) is
@@ -1015,7 +1040,7 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
                 const int ci = kF * (c + 1);
                 if ((rc = layer_grad(r, lb + c, x, 256, dzc, 256, N, h, w, part, dbpart, st)) != MRS_OK)
                     return rc;
-                wtrans_f32(M + L[lb + c].woff, ci, kF, wt, st);
+                if ((rc = simt_pack(M + L[lb + c].woff, ci, kF, 1, wt, st)) != MRS_OK) return rc;
                 rc = simt_conv3x3(dzc, kF, 256, wt, zero, ci, SIMT_RESID, 0, dCat, 256, dCat, 256,
                                   nullptr, N, h, w, 1, st);
             }
@@ -1032,7 +1057,7 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
     k_mask64<<<grid_for(Pl * 64), 256, 0, st>>>(dz, 64, F0, 64, dz, 64, Pl);
     MRS_LAUNCHED(1);
     if ((rc = layer_grad(r, 2, cat, Ccat, dz, kF, N, h, w, part, dbpart, st)) != MRS_OK) return rc;
-    wtrans_f32(r->w_fuse3, Ccat, kF, wt, st);
+    if ((rc = simt_pack(r->w_fuse3, Ccat, kF, 1, wt, st)) != MRS_OK) return rc;
     rc = simt_conv3x3(dz, kF, kF, wt, zero, Ccat, SIMT_PLAIN, 0, nullptr, 0, dxf, Ccat, nullptr, N, h, w,
                       1, st);
     if (rc != MRS_OK) return rc;
@@ -1049,6 +1074,7 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
     if ((rc = adam_f32(r->master, r->grad, r->adam_m, r->adam_v, r->np, lr, r->step, st)) != MRS_OK)
         return rc;
     r->bf_stale = true;
+    r->simt_valid = false;
     if (loss_out) {
         double hsum = 0;
         MRS_CHECK(cudaMemcpyAsync(&hsum, lsum, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1530,6 +1556,7 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     r->step += 1;
     if ((rc = adam_f32(r->master, r->grad, r->adam_m, r->adam_v, r->np, lr, r->step, st)) != MRS_OK) return rc;
     r->bf_stale = true;
+    r->simt_valid = false;
     if (loss_out) {
         double hsum = 0;
         int herr = 0;
@@ -1569,6 +1596,7 @@ extern "C" mrs_status mrs_rdn_free(mrs_rdn r)
     if (r->tgraph) cudaGraphExecDestroy(r->tgraph);
     if (r->tcap) cudaStreamDestroy(r->tcap);
     r->f32.release();
+    r->simt.release();
     r->bf.release();
     r->tr.release();
     r->trb.release();
@@ -1703,6 +1731,7 @@ extern "C" mrs_status mrs_rdn_set_state(mrs_rdn r, const float* params, const fl
     }
     r->step = step;
     r->bf_stale = true;
+    r->simt_valid = false;
     return MRS_OK;
 }
 
