@@ -8,6 +8,7 @@
 // per-output-channel weight scales and calibrated per-layer activation scales).
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
+#include <float.h>
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -834,12 +835,34 @@ __global__ void __launch_bounds__(256) k_wg_reduce(const WgRed* __restrict__ red
 //     |e| / (beta + |e|) per value; dy = sign(e) beta / (beta + |e|)^2 / n
 __device__ __forceinline__ double slog(double x) { return x < 0.0 ? -log1p(-x) : log1p(x); }
 
+// moves v's binary exponent (v >= 1) into e
+__device__ __forceinline__ void take_exponent(double& v, int& e)
+{
+    const int h = __double2hiint(v);
+    e += (h >> 20) - 1023;
+    v = __hiloint2double((h & 0xfffff) | 0x3ff00000, __double2loint(v));
+}
+
+// log1p(x), 0 <= x < 2^-20, to a relative 2^-62
+__device__ __forceinline__ double log1p_tiny(double x) { return x * (1.0 - x * (0.5 - x * (1.0 / 3.0))); }
+
+// L1-log is bound by the float64 units (2 lanes a clock per SM): two log1p a
+// value were 164 float64 operations.  A block sums |slog(y) - slog(t)| as the
+// logarithm of a quotient instead: num collects 1 + the larger magnitude and
+// den 1 + the smaller one (num both, where the signs differ), their exponents
+// are counted in integers, and one logarithm of each is taken per block.  1 + |x|
+// is exact for a float |x| >= 2^-29; below 2^-20 a short series keeps the
+// relative precision.  slog is strictly increasing on floats, so the
+// gradient's sign is the values' own order.  1.77 M values: 460 -> 47 us,
+// 0.79 M: 189 -> 34 us.
 __global__ void k_loss(const float* __restrict__ y, const float* __restrict__ tgt, size_t n,
                        float clip, int kind, float beta, float* __restrict__ dy,
                        double* __restrict__ part)
 {
-    __shared__ double sh[256];
-    double acc = 0.0;
+    __shared__ double sh[256], sn[256], sd[256];
+    __shared__ int se[256];
+    double acc = 0.0, num = 1.0, den = 1.0;
+    int ex = 0;                                  // exponent of num / den
     const float inv_n = 1.0f / (float)n;
     const double b = (double)beta, dinv_n = 1.0 / (double)n;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
@@ -852,17 +875,60 @@ __global__ void k_loss(const float* __restrict__ y, const float* __restrict__ tg
             acc += a / (b + a);
             if (e != 0.0) g = (float)((e > 0.0 ? b : -b) / ((b + a) * (b + a)) * dinv_n);
         } else {
-            double d = slog((double)yp) - slog((double)tv);
-            acc += fabs(d);
-            if (d != 0.0) g = (d > 0.0 ? 1.0f : -1.0f) / (1.0f + fabsf(yp)) * inv_n;
+            const float ay = fabsf(yp), at = fabsf(tv);
+            bool differ = yp != tv, above = yp > tv;
+            if (!(ay <= FLT_MAX && at <= FLT_MAX)) {
+                const double d = slog((double)yp) - slog((double)tv);
+                acc += fabs(d);
+                differ = d != 0.0;
+                above = d > 0.0;
+            } else {
+                const double hi = (double)fmaxf(ay, at), lo = (double)fminf(ay, at);
+                const bool same = (__float_as_int(yp) ^ __float_as_int(tv)) >= 0;
+                if (hi < 0x1p-20) {
+                    const double l = log1p_tiny(lo);
+                    acc += log1p_tiny(hi) + (same ? -l : l);
+                } else {
+                    num *= 1.0 + hi;
+                    if (same) den *= 1.0 + lo;
+                    else num *= 1.0 + lo;
+                    int de = 0;
+                    take_exponent(num, ex);
+                    take_exponent(den, de);
+                    ex -= de;
+                }
+            }
+            if (differ) g = (above ? 1.0f : -1.0f) / (1.0f + ay) * inv_n;
         }
         dy[i] = g;
     }
     sh[threadIdx.x] = acc;
+    sn[threadIdx.x] = num;
+    sd[threadIdx.x] = den;
+    se[threadIdx.x] = ex;
     __syncthreads();
     for (int w = 128; w; w >>= 1) {
         if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
         __syncthreads();
+    }
+    if (kind != MRS_LOSS_ROBUST && threadIdx.x < 32) {
+        int de = 0;
+        for (int k = threadIdx.x + 32; k < 256; k += 32) {
+            num *= sn[k];
+            den *= sd[k];
+            ex += se[k];
+            take_exponent(num, ex);
+            take_exponent(den, de);
+        }
+        for (int w = 16; w; w >>= 1) {
+            num *= __shfl_xor_sync(0xffffffffu, num, w);
+            den *= __shfl_xor_sync(0xffffffffu, den, w);
+        }                                        // below 2^32
+        for (int w = 16; w; w >>= 1) {
+            ex += __shfl_xor_sync(0xffffffffu, ex, w);
+            de += __shfl_xor_sync(0xffffffffu, de, w);
+        }
+        if (threadIdx.x == 0) sh[0] += (double)(ex - de) * 0.693147180559945309 + (log(num) - log(den));
     }
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
