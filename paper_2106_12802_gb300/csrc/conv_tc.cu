@@ -248,7 +248,8 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // Work split: the layer is T = N * XB * H tiles (one tile = one output row of
-// one 128-pixel column strip), flattened as f = (n * XB + xb) * H + y.  CTA c
+// one 128-pixel column strip; N counts groups of tc_images images, narrow
+// images sharing the strip), flattened as f = (n * XB + xb) * H + y.  CTA c
 // takes the contiguous run [T c / G, T (c + 1) / G), cut at strip boundaries
 // into pieces; a piece is a run of rows of one strip, streamed through the
 // input-row ring with its own halo rows.  piece_rows returns the piece that
@@ -339,7 +340,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int XB = (a.W + kFoldTile - 1) / kFoldTile;
-    const long long T = (long long)a.N * XB * a.H;
+    const int im = tc_images(a.N, a.W), pitch = a.W + 2;      // images per tile, their rows apart
+    const long long T = (long long)((a.N + im - 1) / im) * XB * a.H;
     const long long f0 = T * blockIdx.x / gridDim.x, f1 = T * (blockIdx.x + 1) / gridDim.x;
     const bool bf_out = a.mode == TC_RELU_BF16 || a.mode == TC_RESID_BF16 ||
                         a.mode == TC_LIN_BF16 || a.mode == TC_MASK_BF16 ||
@@ -413,6 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int t = 0; t < 9; ++t)
                 tma_load_2d(sW + ((t % 3) * 3 + t / 3) * NOUT * ROWB, &tmap_w, 0, a.w_row0 + t * NOUT, wbar);
             asm volatile("griddepcontrol.wait;" ::: "memory");
+            const uint32_t abytes = (uint32_t)((im > 1 ? im * pitch : kFoldABox) * ROWB);
             uint32_t it = 0;
             bool ok = true;
             for (long long f = f0; ok && f < f1;) {
@@ -431,8 +434,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                         for (int r = ys - 1; r <= ye; ++r, ++it) {
                             int s = it % stages;
                             if (!mbar_wait(&empty[s], ((it / stages) & 1) ^ 1, a.err)) { ok = false; break; }
-                            mbar_expect_tx(&full[s], kFoldABox * ROWB);
-                            tma_load_4d(sA + s * ASLOT, am, 0, xb * kFoldTile - 1, r, n, &full[s]);
+                            mbar_expect_tx(&full[s], abytes);
+                            tma_load_4d(sA + s * ASLOT, am, 0, xb * kFoldTile - 1, r, n * im, &full[s]);
                         }
                     }
                 }
@@ -467,8 +470,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     uint32_t slot = j % kSlots, use = j / kSlots;
                     if (!mbar_wait(&rempty[slot], (use & 1) ^ 1, a.err)) { ok = false; break; }
                     if (loads_res) {
-                        mbar_expect_tx(&rfull[slot], SBYTES);
-                        tma_load_4d(sS + slot * SBYTES, &tmap_res, 0, xb * kFoldTile, y, n, &rfull[slot]);
+                        mbar_expect_tx(&rfull[slot], im > 1 ? (uint32_t)(im * pitch * 128) : (uint32_t)SBYTES);
+                        tma_load_4d(sS + slot * SBYTES, &tmap_res, 0, xb * kFoldTile, y, n * im, &rfull[slot]);
                     } else {
                         mbar_arrive(&rfull[slot]);
                     }
@@ -486,7 +489,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     uint32_t slot = j % kSlots, use = j / kSlots;
                     if (!mbar_wait(&edone[slot], use & 1, a.err)) { ok = false; break; }
                     if (stores_bf) {
-                        tma_store_4d(&tmap_out, sS + slot * SBYTES, 0, xb * kFoldTile, y, n);
+                        tma_store_4d(&tmap_out, sS + slot * SBYTES, 0, xb * kFoldTile, y, n * im);
                         bulk_commit();
                         bulk_wait_read0();
                     }
@@ -579,6 +582,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int q = warp & 3, grp = (warp - 2) >> 2;
         const int j = q * 32 + lane;
         const bool active = grp * 16 < NOUT;
+        // the lane's image in its tile and pixel in the strip
+        const int ji = im > 1 ? j / pitch : 0, jx = j - ji * pitch;
         uint32_t lt = 0;
         bool stop = false;
         for (long long f = f0; !stop && f < f1;) {
@@ -588,9 +593,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int sl = (int)((NS - (int)(lt % NS)) % NS);
             const uint32_t use = lt / NS;
             const uint32_t slot = lt % kSlots, suse = lt / kSlots;
-            const int x = xb * kFoldTile + j;
-            const bool valid = x < a.W;
-            const size_t p = ((size_t)n * a.H + y) * a.W + (valid ? x : 0);
+            const int x = xb * kFoldTile + jx, img = n * im + ji;
+            const bool valid = x < a.W && ji < im && img < a.N;
+            const size_t p = valid ? ((size_t)img * a.H + y) * a.W + x : 0;
             if (!mbar_wait_warp(&tfull[sl], use & 1, a.err)) { stop = true; break; }
             tc_fence_after();
             if (!mbar_wait_warp(&rfull[slot], suse & 1, a.err)) { stop = true; break; }
@@ -673,7 +678,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (a.mode == TC_FINAL_F32) {
                         if (c0 == 0) {
                             float up[3];
-                            bilinear(a.lrhs + (size_t)n * (a.H / a.scale) * (a.W / a.scale) * 3,
+                            bilinear(a.lrhs + (size_t)img * (a.H / a.scale) * (a.W / a.scale) * 3,
                                      a.H / a.scale, a.W / a.scale, a.scale, x, y, up);
                             float* op = (float*)a.out + p * 3;
                             for (int c = 0; c < 3; ++c) op[c] = (v[c] + sBias[c]) + up[c];
@@ -758,7 +763,8 @@ mrs_status launch_fold(const TcConvArgs& a, cudaStream_t st)
     const int stages = want >= 3 ? (want < smax ? want : smax) : smax;
     size_t smem = fold_smem_bytes<NOUT, OPER>(stages);
     TcConvArgs b = a;
-    const long long T = (long long)a.N * ((a.W + kFoldTile - 1) / kFoldTile) * a.H;
+    const int im = tc_images(a.N, a.W);
+    const long long T = (long long)((a.N + im - 1) / im) * ((a.W + kFoldTile - 1) / kFoldTile) * a.H;
     int grid = T < sm_count() ? (int)T : sm_count();
     if (grid < 1) return MRS_OK;
     const CUtensorMap* res = a.tmap_res ? a.tmap_res : a.tmap_x;
@@ -781,6 +787,14 @@ mrs_status launch_fold(const TcConvArgs& a, cudaStream_t st)
     return cuda_status(cudaGetLastError(), "conv launch");
 }
 
+// images of a box: a conv's operand or output box (tc_images), else one
+int conv_box(int& box_px, int box_rows, int N, int W)
+{
+    const int im = box_rows == 1 && (box_px == kABox || box_px == kOutBox) ? tc_images(N, W) : 1;
+    if (im > 1) box_px = W + 2;
+    return im;
+}
+
 }  // namespace
 
 mrs_status tc_make_act_map(CUtensorMap* m, const void* ptr, int N, int H, int W, int operand,
@@ -791,7 +805,8 @@ mrs_status tc_make_act_map(CUtensorMap* m, const void* ptr, int N, int H, int W,
     int rowb = operand == TC_BF16 ? 128 : 64;
     cuuint64_t dims[4] = {64, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
     cuuint64_t strides[3] = {(cuuint64_t)rowb, (cuuint64_t)rowb * W, (cuuint64_t)rowb * W * H};
-    cuuint32_t box[4] = {64, (cuuint32_t)box_px, 1, 1};
+    const int im = conv_box(box_px, 1, N, W);
+    cuuint32_t box[4] = {64, (cuuint32_t)box_px, 1, (cuuint32_t)im};
     cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = fn(m, operand == TC_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8,
                     4, const_cast<void*>(ptr), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -813,7 +828,8 @@ mrs_status tc_make_view_map(CUtensorMap* m, const void* ptr, int N, int H, int W
     }
     cuuint64_t dims[4] = {64, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
     cuuint64_t strides[3] = {(cuuint64_t)px_stride, (cuuint64_t)row_stride, (cuuint64_t)img_stride};
-    cuuint32_t box[4] = {64, (cuuint32_t)box_px, (cuuint32_t)box_rows, 1};
+    const int im = conv_box(box_px, box_rows, N, W);
+    cuuint32_t box[4] = {64, (cuuint32_t)box_px, (cuuint32_t)box_rows, (cuuint32_t)im};
     cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides,
                     box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
