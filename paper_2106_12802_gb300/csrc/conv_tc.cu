@@ -14,7 +14,7 @@
 // Warp roles (640 threads, one CTA per SM):
 //   warp 0: TMA producer (weights once, then one A box per input row through
 //           an S-stage ring)
-//   warp 1: TMEM allocator and MMA issuer (one thread)
+//   warp 1: TMEM allocator and MMA issuer (all lanes form the operands, one issues)
 //   warps 2-17: epilogue; warp w reads TMEM lanes 32 (w % 4) .. + 31 and 16 of
 //           the 64 output channels: dequantisation (fp8), bias, ReLU /
 //           residual / mask / FP32 partial sum / bilinear skip, BF16 results
@@ -32,6 +32,7 @@
 #include <algorithm>
 #include <atomic>
 #include <queue>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -305,12 +306,19 @@ template <int NOUT, int OPER> size_t fold_smem_bytes(int stages)
            (size_t)kSlots * kFoldTile * 128 + 64 * 4 + 8 * (2 * stages + 2 + 2 * (512 / NOUT) + 3 * kSlots) + 16;
 }
 
-template <int NOUT, int OPER>
+__device__ __forceinline__ const TcConvArgs& more_of(const TcConvArgs& a) { return a; }
+__device__ __forceinline__ TcConvArgs more_of(const TcConvBase&) { return TcConvArgs{}; }
+
+// kMore: groups, masked sums and second results (TcConvArgs::ng, mask, op2);
+// tested for at run time in every conv they cost the inference layers 1 to 2%
+template <int NOUT, int OPER, bool kMore>
 __global__ void __launch_bounds__(kThreads, 1)
     k_conv_fold(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                 const __grid_constant__ CUtensorMap tmap_res,
-                const __grid_constant__ CUtensorMap tmap_out, TcConvArgs a, int stages)
+                const __grid_constant__ CUtensorMap tmap_out,
+                const std::conditional_t<kMore, TcConvArgs, TcConvBase> a, int stages)
 {
+    const auto& more = more_of(a);
     constexpr int NS = 512 / NOUT;                            // TMEM accumulator slots
     constexpr int ROWB = fold_rowb(OPER);                     // bytes per operand row
     constexpr int ASLOT = fold_aslot(OPER);
@@ -342,12 +350,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int XB = (a.W + kFoldTile - 1) / kFoldTile;
     const int im = tc_images(a.N, a.W), pitch = a.W + 2;      // images per tile, their rows apart
     const long long T = (long long)((a.N + im - 1) / im) * XB * a.H;
-    const long long f0 = T * blockIdx.x / gridDim.x, f1 = T * (blockIdx.x + 1) / gridDim.x;
-    const bool bf_out = a.mode == TC_RELU_BF16 || a.mode == TC_RESID_BF16 ||
-                        a.mode == TC_LIN_BF16 || a.mode == TC_MASK_BF16 ||
-                        a.mode == TC_RESRELU_BF16;
-    const bool loads_res = a.mode == TC_RESID_BF16 || a.mode == TC_MASK_BF16 ||
-                           a.mode == TC_RESRELU_BF16;
+    // the CTA's group (of ng convolutions of the same input) and its place in it
+    const int ng = kMore && more.ng > 1 ? more.ng : 1, group = kMore ? (int)blockIdx.x * ng / (int)gridDim.x : 0;
+    const int cta0 = kMore ? (group * (int)gridDim.x + ng - 1) / ng : 0;
+    const int cta1 = kMore ? ((group + 1) * (int)gridDim.x + ng - 1) / ng : (int)gridDim.x;
+    const long long f0 = T * ((int)blockIdx.x - cta0) / (cta1 - cta0), f1 = T * ((int)blockIdx.x - cta0 + 1) / (cta1 - cta0);
+    const int mode = kMore && ng > 1 ? more.gmode[min(group, 3)] : a.mode, w_row0 = a.w_row0 + 9 * NOUT * group;
+    const CUtensorMap* mres = kMore && ng > 1 ? more.gmaps + 2 * group : &tmap_res;
+    const CUtensorMap* mout = kMore && ng > 1 ? more.gmaps + 2 * group + 1 : &tmap_out;
+    const bool bf_out = mode == TC_RELU_BF16 || mode == TC_RESID_BF16 ||
+                        mode == TC_LIN_BF16 || mode == TC_MASK_BF16 ||
+                        mode == TC_RESRELU_BF16;
+    const bool loads_res = mode == TC_RESID_BF16 || mode == TC_MASK_BF16 ||
+                           mode == TC_RESRELU_BF16;
     // a bf16 result that nobody reads (fp8 operands: only the fp8 copy) is
     // neither staged nor stored
     const bool stores_bf = bf_out && !(a.fp8_only && a.out_fp8);
@@ -368,7 +383,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (threadIdx.x < 64) sBias[threadIdx.x] = threadIdx.x < NOUT ? a.bias[threadIdx.x] : 0.0f;
+    if (threadIdx.x < 64) sBias[threadIdx.x] = threadIdx.x < NOUT ? a.bias[threadIdx.x + (kMore && more.gbias ? 64 * group : 0)] : 0.0f;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(tslot)),
@@ -413,7 +428,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_expect_tx(wbar, WBYTES);
             // tap (dy, dx) at B row (3 dx + dy) NOUT: per dx the three kernel rows are contiguous
             for (int t = 0; t < 9; ++t)
-                tma_load_2d(sW + ((t % 3) * 3 + t / 3) * NOUT * ROWB, &tmap_w, 0, a.w_row0 + t * NOUT, wbar);
+                tma_load_2d(sW + ((t % 3) * 3 + t / 3) * NOUT * ROWB, &tmap_w, 0, w_row0 + t * NOUT, wbar);
             asm volatile("griddepcontrol.wait;" ::: "memory");
             const uint32_t abytes = (uint32_t)((im > 1 ? im * pitch : kFoldABox) * ROWB);
             uint32_t it = 0;
@@ -461,6 +476,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == kResWarp) {
         if (lane == 0) {
+            if (kMore && ng > 1 && loads_res)
+                asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)mres) : "memory");
             uint32_t j = 0;
             bool ok = true;
             for (long long f = f0; ok && f < f1;) {
@@ -471,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (!mbar_wait(&rempty[slot], (use & 1) ^ 1, a.err)) { ok = false; break; }
                     if (loads_res) {
                         mbar_expect_tx(&rfull[slot], im > 1 ? (uint32_t)(im * pitch * 128) : (uint32_t)SBYTES);
-                        tma_load_4d(sS + slot * SBYTES, &tmap_res, 0, xb * kFoldTile, y, n * im, &rfull[slot]);
+                        tma_load_4d(sS + slot * SBYTES, mres, 0, xb * kFoldTile, y, n * im, &rfull[slot]);
                     } else {
                         mbar_arrive(&rfull[slot]);
                     }
@@ -480,6 +497,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == kStoreWarp) {
         if (lane == 0) {
+            if (kMore && ng > 1 && stores_bf)
+                asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)mout) : "memory");
             uint32_t j = 0;
             bool ok = true;
             for (long long f = f0; ok && f < f1;) {
@@ -489,7 +508,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     uint32_t slot = j % kSlots, use = j / kSlots;
                     if (!mbar_wait(&edone[slot], use & 1, a.err)) { ok = false; break; }
                     if (stores_bf) {
-                        tma_store_4d(&tmap_out, sS + slot * SBYTES, 0, xb * kFoldTile, y, n * im);
+                        tma_store_4d(mout, sS + slot * SBYTES, 0, xb * kFoldTile, y, n * im);
                         bulk_commit();
                         bulk_wait_read0();
                     }
@@ -583,6 +602,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int j = q * 32 + lane;
         const bool active = grp * 16 < NOUT;
         // the lane's image in its tile and pixel in the strip
+        const bool masked = kMore && more.mask && group == ng - 1 && mode == TC_RESID_BF16;
+        const __nv_bfloat16* aux = (const __nv_bfloat16*)(masked ? more.mask : kMore && more.op2 ? more.x2 : nullptr);
         const int ji = im > 1 ? j / pitch : 0, jx = j - ji * pitch;
         uint32_t lt = 0;
         bool stop = false;
@@ -596,6 +617,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int x = xb * kFoldTile + jx, img = n * im + ji;
             const bool valid = x < a.W && ji < im && img < a.N;
             const size_t p = valid ? ((size_t)img * a.H + y) * a.W + x : 0;
+            // the mask's or second result's operand, read while the row is computed
+            uint4 u2[2];
+            if (kMore && aux && active && valid) {
+                u2[0] = *(const uint4*)(aux + p * 64 + grp * 16);
+                u2[1] = *(const uint4*)(aux + p * 64 + grp * 16 + 8);
+            }
             if (!mbar_wait_warp(&tfull[sl], use & 1, a.err)) { stop = true; break; }
             tc_fence_after();
             if (!mbar_wait_warp(&rfull[slot], suse & 1, a.err)) { stop = true; break; }
@@ -622,10 +649,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                     float o[16];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) o[e] = v[e] + sBias[c0 + e];
-                    if (a.mode == TC_RELU_BF16) {
+                    if (mode == TC_RELU_BF16) {
 #pragma unroll
                         for (int e = 0; e < 16; ++e) o[e] = fmaxf(o[e], 0.0f);
-                    } else if (a.mode == TC_MASK_BF16) {
+                    } else if (mode == TC_MASK_BF16) {
 #pragma unroll
                         for (int jj = 0; jj < 2; ++jj) {
                             uint4 u = *(const uint4*)(srow + sw128(j, c0 / 8 + jj));
@@ -637,8 +664,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 if (!(fv.y > 0.0f)) o[8 * jj + 2 * e + 1] = 0.0f;
                             }
                         }
-                    } else if (a.mode == TC_RESID_BF16 || a.mode == TC_RESRELU_BF16) {
-                        const bool rl = a.mode == TC_RESRELU_BF16;
+                    } else if (mode == TC_RESID_BF16 || mode == TC_RESRELU_BF16) {
+                        const bool rl = mode == TC_RESRELU_BF16;
 #pragma unroll
                         for (int jj = 0; jj < 2; ++jj) {
                             uint4 u = *(const uint4*)(srow + sw128(j, c0 / 8 + jj));
@@ -652,6 +679,32 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 o[8 * jj + 2 * e + 1] = fv.y + o1;
                             }
                         }
+                        if (kMore && masked && valid) {
+                            const __nv_bfloat16* h = (const __nv_bfloat16*)u2;
+#pragma unroll
+                            for (int e = 0; e < 16; ++e)
+                                if (!(__bfloat162float(h[e]) > 0.0f)) o[e] = 0.0f;
+                        }
+                    }
+                    if (kMore && more.op2 && valid) {
+                        const __nv_bfloat162* h2 = (const __nv_bfloat162*)u2;
+                        __nv_bfloat162 t2[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const float2 x2 = __bfloat1622float2(h2[e]);
+                            float2 b2 = __bfloat1622float2(__floats2bfloat162_rn(o[2 * e], o[2 * e + 1]));
+                            if (more.op2 == 1) {
+                                if (!(x2.x > 0.0f)) b2.x = 0.0f;
+                                if (!(x2.y > 0.0f)) b2.y = 0.0f;
+                            } else {
+                                b2.x = x2.x + b2.x;
+                                b2.y = x2.y + b2.y;
+                            }
+                            t2[e] = __floats2bfloat162_rn(b2.x, b2.y);
+                        }
+                        __nv_bfloat16* o2 = (__nv_bfloat16*)more.out2 + p * 64 + c0;
+                        *(uint4*)o2 = ((const uint4*)t2)[0];
+                        *(uint4*)(o2 + 8) = ((const uint4*)t2)[1];
                     }
                     if (stores_bf) {
 #pragma unroll
@@ -675,7 +728,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         *(uint4*)((uint8_t*)a.out_fp8 + p * 64 + c0) = u;
                     }
                 } else if (valid) {
-                    if (a.mode == TC_FINAL_F32) {
+                    if (mode == TC_FINAL_F32) {
                         if (c0 == 0) {
                             float up[3];
                             bilinear(a.lrhs + (size_t)img * (a.H / a.scale) * (a.W / a.scale) * 3,
@@ -746,14 +799,14 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 // input-row ring depth of the conv (0: the most that fits shared memory)
 std::atomic<int> g_fold_ring{0};
 
-template <int NOUT, int OPER>
+template <int NOUT, int OPER, bool kMore>
 mrs_status launch_fold(const TcConvArgs& a, cudaStream_t st)
 {
     int smax = 4;
     while (fold_smem_bytes<NOUT, OPER>(smax + 1) <= 227 * 1024 && smax < 12) ++smax;
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_fold<NOUT, OPER>,
+        cudaError_t e = cudaFuncSetAttribute(k_conv_fold<NOUT, OPER, kMore>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)fold_smem_bytes<NOUT, OPER>(smax));
         if (e != cudaSuccess) return cuda_status(e, "conv smem attribute");
@@ -762,10 +815,11 @@ mrs_status launch_fold(const TcConvArgs& a, cudaStream_t st)
     const int want = g_fold_ring.load(std::memory_order_relaxed);
     const int stages = want >= 3 ? (want < smax ? want : smax) : smax;
     size_t smem = fold_smem_bytes<NOUT, OPER>(stages);
-    TcConvArgs b = a;
+    const std::conditional_t<kMore, TcConvArgs, TcConvBase> b = a;
     const int im = tc_images(a.N, a.W);
     const long long T = (long long)((a.N + im - 1) / im) * ((a.W + kFoldTile - 1) / kFoldTile) * a.H;
-    int grid = T < sm_count() ? (int)T : sm_count();
+    const long long tiles = T * (a.ng > 1 ? a.ng : 1);
+    int grid = tiles < sm_count() ? (int)tiles : sm_count();
     if (grid < 1) return MRS_OK;
     const CUtensorMap* res = a.tmap_res ? a.tmap_res : a.tmap_x;
     const CUtensorMap* out = a.tmap_out ? a.tmap_out : a.tmap_x;
@@ -781,7 +835,7 @@ mrs_status launch_fold(const TcConvArgs& a, cudaStream_t st)
     cfg.attrs = la;
     cfg.numAttrs = 1;
     cudaError_t le = cudaSuccess;
-    MRS_TIMED(PK_CONV_TC, st, (le = cudaLaunchKernelEx(&cfg, k_conv_fold<NOUT, OPER>, *a.tmap_x, *a.tmap_w, *res, *out, b, stages)));
+    MRS_TIMED(PK_CONV_TC, st, (le = cudaLaunchKernelEx(&cfg, k_conv_fold<NOUT, OPER, kMore>, *a.tmap_x, *a.tmap_w, *res, *out, b, stages)));
     MRS_LAUNCHED(1);
     if (le != cudaSuccess) return cuda_status(le, "conv launch");
     return cuda_status(cudaGetLastError(), "conv launch");
@@ -897,8 +951,23 @@ mrs_status tc_conv3x3(const TcConvArgs& a, cudaStream_t st)
         set_error("tc_conv3x3: kc > 1 needs a 64-byte aligned device array of kc maps");
         return MRS_ERR_ARG;
     }
-    if (a.nout == 64) return a.operand == TC_BF16 ? launch_fold<64, TC_BF16>(a, st) : launch_fold<64, TC_FP8>(a, st);
-    if (a.nout == 16) return a.operand == TC_BF16 ? launch_fold<16, TC_BF16>(a, st) : launch_fold<16, TC_FP8>(a, st);
+    if (a.ng > 1 && (a.kc > 1 || a.op2 || a.ng > sm_count() || !a.gmaps || ((uintptr_t)a.gmaps & 63))) {
+        set_error("tc_conv3x3: a group of convs takes one input chunk and a 64-byte aligned device array of maps");
+        return MRS_ERR_ARG;
+    }
+    if (a.mask && a.op2) {
+        set_error("tc_conv3x3: mask and op2 exclude each other");
+        return MRS_ERR_ARG;
+    }
+    if (a.ng > 1 || a.mask || a.op2) {
+        if (a.nout == 64 && a.operand == TC_BF16) return launch_fold<64, TC_BF16, true>(a, st);
+        set_error("tc_conv3x3: groups, masks and second results need 64 BF16 channels");
+        return MRS_ERR_ARG;
+    }
+    if (a.nout == 64)
+        return a.operand == TC_BF16 ? launch_fold<64, TC_BF16, false>(a, st) : launch_fold<64, TC_FP8, false>(a, st);
+    if (a.nout == 16)
+        return a.operand == TC_BF16 ? launch_fold<16, TC_BF16, false>(a, st) : launch_fold<16, TC_FP8, false>(a, st);
     set_error("tc_conv3x3: nout must be 64 or 16");
     return MRS_ERR_ARG;
 }

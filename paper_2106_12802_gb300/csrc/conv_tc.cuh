@@ -25,7 +25,7 @@ enum TcMode : int {
 
 enum TcOperand : int { TC_BF16 = 0, TC_FP8 = 1 };
 
-struct TcConvArgs {
+struct TcConvBase {
     const CUtensorMap* tmap_x;   // A operand [N][H][W][64] (bf16 or fp8, kABox-pixel boxes)
     const CUtensorMap* tmap_res; // TC_RESID_BF16 residual (bf16, kOutBox-pixel boxes)
     const CUtensorMap* tmap_out; // TC_RELU_BF16 / TC_RESID_BF16 output (bf16, kOutBox-pixel boxes)
@@ -56,6 +56,26 @@ struct TcConvArgs {
     const CUtensorMap* amaps;
     int kc;
     int w_row0;
+};
+
+// (kept apart: the kernels that know none of it take the short parameter block)
+struct TcConvArgs : TcConvBase {
+    // ng > 1 convolutions of ONE input in one launch (bf16 results, kc <= 1): the
+    // CTAs are shared out among them.  Group g takes the weights at rows
+    // w_row0 + 9 g nout, the bias at bias + 64 g where gbias is set, mode
+    // gmode[min(g, 3)], and its residual and output maps from the device array
+    // gmaps [2 g], [2 g + 1] (64-byte aligned, alive until the kernel completes)
+    int ng;
+    int gbias;
+    int gmode[4];
+    const CUtensorMap* gmaps;
+    // TC_RESID_BF16 (of the last group): the sum is kept where mask[p] > 0, else 0
+    const void* mask;            // bf16 [p][64], or NULL
+    // a second bf16 result of bf16 modes, ng <= 1: out2 = x2 > 0 ? out : 0 (op2 = 1)
+    // or x2 + out (op2 = 2)
+    int op2;
+    const void* x2;              // bf16 [p][64]
+    void* out2;
 };
 
 // Box widths (pixels): the conv reads one 130-pixel A box per input row (a

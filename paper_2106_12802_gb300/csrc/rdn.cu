@@ -358,28 +358,55 @@ __global__ void k_gather_f32(const float* __restrict__ src, const int* __restric
 }
 
 // ---- training (BF16): elementwise steps ------------------------------------
-// out[i] = act[i] > 0 ? d[i] : 0 (out may be d)
+// The tensors are whole 128-byte rows, 8 values (16 bytes) a thread.
+// out[i] = act[i] > 0 ? d[i] : 0 (out may be d); n groups of 8 values
 __global__ void k_mask_copy_bf16(const __nv_bfloat16* d, const __nv_bfloat16* __restrict__ act,
                                  size_t n, __nv_bfloat16* out)
 {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x)
-        out[i] = __bfloat162float(act[i]) > 0.0f ? d[i] : __float2bfloat16_rn(0.0f);
+         i += (size_t)gridDim.x * blockDim.x) {
+        uint4 v = ((const uint4*)d)[i];
+        const uint4 m = __ldg((const uint4*)act + i);
+        __nv_bfloat16* vh = (__nv_bfloat16*)&v;
+        const __nv_bfloat16* mh = (const __nv_bfloat16*)&m;
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (!(__bfloat162float(mh[e]) > 0.0f)) vh[e] = __float2bfloat16_rn(0.0f);
+        ((uint4*)out)[i] = v;
+    }
 }
 
 // out = a + b (+ c) (+ e), summed in FP32 and rounded once; when act is given,
-// out = act > 0 ? that : 0
+// out = act > 0 ? that : 0 (out may be a); n groups of 8 values
 __global__ void k_sum_bf16(__nv_bfloat16* out, const __nv_bfloat16* a, const __nv_bfloat16* b,
                            const __nv_bfloat16* c, const __nv_bfloat16* e,
                            const __nv_bfloat16* __restrict__ act, size_t n)
 {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
          i += (size_t)gridDim.x * blockDim.x) {
-        float v = __bfloat162float(a[i]) + __bfloat162float(b[i]);
-        if (c) v += __bfloat162float(c[i]);
-        if (e) v += __bfloat162float(e[i]);
-        if (act && !(__bfloat162float(act[i]) > 0.0f)) v = 0.0f;
-        out[i] = __float2bfloat16_rn(v);
+        float v[8];
+        auto add = [&](const __nv_bfloat16* x, bool first) {
+            const uint4 u = ((const uint4*)x)[i];
+            const __nv_bfloat16* h = (const __nv_bfloat16*)&u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = first ? __bfloat162float(h[k]) : v[k] + __bfloat162float(h[k]);
+        };
+        add(a, true);
+        add(b, false);
+        if (c) add(c, false);
+        if (e) add(e, false);
+        if (act) {
+            const uint4 u = __ldg((const uint4*)act + i);
+            const __nv_bfloat16* h = (const __nv_bfloat16*)&u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (!(__bfloat162float(h[k]) > 0.0f)) v[k] = 0.0f;
+        }
+        uint4 o;
+        __nv_bfloat16* oh = (__nv_bfloat16*)&o;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) oh[k] = __float2bfloat16_rn(v[k]);
+        ((uint4*)out)[i] = o;
     }
 }
 
@@ -1181,12 +1208,18 @@ mrs_status repack_if_stale(mrs_rdn_s* r, cudaStream_t st)
 // its input + that ReLU output, summed in FP32 and rounded once, plus the
 // group and Eq. F_DF skips), the loss on the FP32 I_SR, then the backward:
 // input gradients as tensor-core convs with the transposed, tap-flipped chunk
-// weights (ReLU masks as epilogues or elementwise passes, the dense parts'
-// gradients accumulated in place by residual epilogues, the shuffle and
-// deshuffle exchanged through strided views), then every layer's weight
+// weights (ReLU masks as epilogues, the dense parts' gradients accumulated in
+// place by residual epilogues, the shuffle and deshuffle exchanged through
+// strided views), then every layer's weight
 // gradients in one k_wgrad_tc launch over 64 x 64 tiles with a fixed-order
 // reduction into the FP32 gradient, Adam
 // on the FP32 weights.  Activations and their gradients are BF16.
+// A crop's layers are a few tiles a CTA, so a launch is mostly its prologue,
+// halo rows and drain: convs of one input (a block's dgrads of one layer, the
+// fuse conv's 1 + s^2, an upsampling stage's 4) are one launch, and a mask or sum
+// that follows a conv is in its epilogue.  As 242 conv launches and 81
+// elementwise ones a step of 16 crops of 48 x 48 (x 4) took 5.37 ms of device
+// time, as 130 and 12 3.96 ms.
 mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, const float* alb,
                           const float* nrm, const float* extra, const float* tgt, int N, int H, int W,
                           int kind, float beta, float lr, float* yout, double* loss_out,
@@ -1359,6 +1392,34 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
         mc_up[d] = mc.size();
         for (int q = 0; q < 4; ++q) mc.push_back(dupA[d][q]);
     }
+    // (residual, output) maps of the launches that hold several convs of one
+    // input: a block's local fusion (parts 0..3) and dense convs 3 and 2, the
+    // fuse conv's input gradients, each upsampling stage
+    std::vector<std::array<size_t, 3>> mg_blk(nblk);
+    std::vector<size_t> mg_up(D);
+    for (int k = 0; k < nblk; ++k)
+        for (int c = kConv; c >= 2; --c) {
+            mg_blk[k][kConv - c] = mc.size();
+            for (int j = 0; j < c; ++j) {
+                const CUtensorMap& o = j ? mDp[k][j].o : mG.o;
+                mc.push_back(c == kConv && j == 3 ? mF[k][2].o : o);   // the last part is masked by F_3
+                mc.push_back(o);
+            }
+        }
+    const size_t mg_fuse = mc.size();
+    mc.push_back(mFlr.o);
+    mc.push_back(mDzlr.o);
+    for (int q = 0; q < SS; ++q) {
+        mc.push_back(dsfO[q]);
+        mc.push_back(dz1O[q]);
+    }
+    for (int d = 0; d < D; ++d) {
+        mg_up[d] = mc.size();
+        for (int q = 0; q < 4; ++q) {
+            mc.push_back(upO[d][q]);
+            mc.push_back(upO[d][q]);
+        }
+    }
     if ((rc = r->tdmaps.ensure(mc.size() * sizeof(CUtensorMap) + 64)) != MRS_OK) return rc;
     const CUtensorMap* dmc = r->tdmaps.as<CUtensorMap>();
     MRS_CHECK(cudaMemcpyAsync(r->tdmaps.p, mc.data(), mc.size() * sizeof(CUtensorMap),
@@ -1415,6 +1476,17 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
         a.tmap_res = res; a.tmap_out = out; a.out = outf; a.cout = cout; a.relu = 0;
         return tc_conv3x3(a, st);
     };
+    // ng convs of one input in one launch over the map pairs dmc[mg ..]
+    auto convs = [&](int ng, int hh, int ww, const CUtensorMap* A, size_t mg, const CUtensorMap* wm, int w_row0,
+                     const float* bias, bool gbias, int m0, int m1, int m2, int m3, const __nv_bfloat16* mask) {
+        a.ng = ng; a.gmaps = dmc + mg; a.gbias = gbias; a.mask = mask;
+        a.gmode[0] = m0; a.gmode[1] = m1; a.gmode[2] = m2; a.gmode[3] = m3;
+        const mrs_status e = conv(hh, ww, A, -1, 1, wm, w_row0, bias, 64, m0, nullptr, nullptr);
+        a.ng = 0; a.gbias = 0; a.mask = nullptr;
+        return e;
+    };
+    // a second result of the next conv (TcConvArgs::op2)
+    auto second = [&](int op2, const __nv_bfloat16* x2, __nv_bfloat16* out2) { a.op2 = op2; a.x2 = x2; a.out2 = out2; };
     const WChunk* CH = r->ch.data();
     auto fmap = [&](int li, int j) { return &CH[r->first[li] + j].map; };       // single forward chunk
     auto frow = [&](int li) { return (int)(CH[r->first[li]].off / 64); };       // a layer's chunks in wmap_all
@@ -1434,24 +1506,27 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     for (int g = 0; g < kRDG; ++g) {
         for (int b = 0; b < kRDB; ++b) {
             const int k = kRDB * g + b;
+            // block output; + F_{g-1} after a group's last block; + F_0 at the end (Eq. F_DF)
+            const bool last = b == kRDB - 1;
             for (int c = 1; c <= kConv; ++c, ++li) {
                 const CUtensorMap* out = &mF[k][c - 1].o;        // F_1, F_2, F_3, ReLU(local fusion)
+                if (c == kConv && !last) second(2, X[k], X[k + 1]);
                 rc = c == 1 ? conv(h, w, &mX[k].a, -1, 1, fmap(li, 0), 0, fbias(li, 0), 64, TC_RELU_BF16, nullptr, out)
                             : conv(h, w, &mX[k].a, (long)mc_blk[k], c, &r->wmap_all, frow(li), fbias(li, 0), 64,
                                    TC_RELU_BF16, nullptr, out);
                 if (rc != MRS_OK) return rc;
             }
-            // block output; + F_{g-1} after a group's last block; + F_0 at the end (Eq. F_DF)
-            const bool last = b == kRDB - 1;
-            k_sum_bf16<<<grid_for(Pl * 64), 256, 0, st>>>(X[k + 1], X[k], Fk[k][3], last ? X[kRDB * g] : nullptr,
-                                                          k + 1 == nblk ? F0 : nullptr, nullptr, Pl * 64);
-            MRS_LAUNCHED(1);
+            second(0, nullptr, nullptr);
+            if (last) {
+                k_sum_bf16<<<grid_for(Pl * 8), 256, 0, st>>>(X[k + 1], X[k], Fk[k][3], X[kRDB * g],
+                                                             k + 1 == nblk ? F0 : nullptr, nullptr, Pl * 8);
+                MRS_LAUNCHED(1);
+            }
         }
     }
     for (int d = 0; d < D; ++d, ++li)
-        for (int q = 0; q < 4; ++q)
-            if ((rc = conv(hd[d], wd[d], &mU[d].a, -1, 1, fmap(li, q), 0, fbias(li, q), 64, TC_RELU_BF16,
-                           nullptr, &upO[d][q])) != MRS_OK) return rc;
+        if ((rc = convs(4, hd[d], wd[d], &mU[d].a, mg_up[d], &r->wmap_all, frow(li), fbias(li, 0), true, TC_RELU_BF16,
+                        TC_RELU_BF16, TC_RELU_BF16, TC_RELU_BF16, nullptr)) != MRS_OK) return rc;
     const int li_rec = li;
     if ((rc = conv(H, W, &mU[D].a, -1, 1, fmap(li_rec, 0), 0, fbias(li_rec, 0), CH[r->first[li_rec]].nout,
                    TC_PLAIN_F32, nullptr, nullptr, y, 3)) != MRS_OK) return rc;
@@ -1463,7 +1538,7 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
 
     // ---- backward
     auto mask = [&](const __nv_bfloat16* d, const __nv_bfloat16* act, size_t P, __nv_bfloat16* out) {
-        k_mask_copy_bf16<<<grid_for(P * 64), 256, 0, st>>>(d, act, P * 64, out);
+        k_mask_copy_bf16<<<grid_for(P * 8), 256, 0, st>>>(d, act, P * 8, out);
         MRS_LAUNCHED(1);
     };
     const CUtensorMap* WT = &r->wmapT_all;
@@ -1483,41 +1558,33 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
         MRS_CHECK(cudaMemcpyAsync(dSkip, G, Pl * 128, cudaMemcpyDeviceToDevice, st));
         for (int b = kRDB - 1; b >= 0; --b) {
             const int k = kRDB * g + b, lb = 3 + kConv * k;
-            // local fusion: dz4 = G masked by its ReLU output; part 0's gradient =
-            // G + conv^T, parts 1..3 start here
-            mask(G, Fk[k][3], Pl, dpb[k][0]);
-            if ((rc = conv(h, w, &mDp[k][0].a, -1, 1, WT, trow(lb + 3, 0), zero, 64, TC_RESID_BF16, &mG.o,
-                           &mG.o)) != MRS_OK) return rc;
-            for (int j = 1; j < 4; ++j)
-                if ((rc = conv(h, w, &mDp[k][0].a, -1, 1, WT, trow(lb + 3, j), zero, 64, TC_LIN_BF16, nullptr,
-                               &mDp[k][j].o)) != MRS_OK) return rc;
-            // dense convs 3, 2, 1: the gradient of F_c is complete once the later
-            // convs have added theirs; masked by F_c, then its input gradients
-            // added into parts 0 .. c - 1
-            for (int c = kConv - 1; c >= 1; --c) {
-                const int lc = lb + c - 1;
-                mask(dpb[k][c], Fk[k][c - 1], Pl, dpb[k][c]);
-                for (int j = 0; j < c; ++j) {
-                    const CUtensorMap* into = j ? &mDp[k][j].o : &mG.o;
-                    if ((rc = conv(h, w, &mDp[k][c].a, -1, 1, WT, trow(lc, j), zero, 64, TC_RESID_BF16, into,
-                                   into)) != MRS_OK) return rc;
-                }
-            }
+            // local fusion: dz4 = G masked by its ReLU output (written with G by the
+            // block before); part 0's gradient = G + conv^T, parts 1..3 start here
+            if (b == kRDB - 1) mask(G, Fk[k][3], Pl, dpb[k][0]);
+            if ((rc = convs(4, h, w, &mDp[k][0].a, mg_blk[k][0], WT, trow(lb + 3, 0), zero, false, TC_RESID_BF16,
+                            TC_LIN_BF16, TC_LIN_BF16, TC_MASK_BF16, nullptr)) != MRS_OK) return rc;
+            // dense convs 3, 2, 1: each one's input gradients are added into parts
+            // 0 .. c - 1; part c - 1 is then complete and masked by F_{c-1}
+            for (int c = kConv - 1; c >= 2; --c)
+                if ((rc = convs(c, h, w, &mDp[k][c].a, mg_blk[k][kConv - c], WT, trow(lb + c - 1, 0), zero, false,
+                                TC_RESID_BF16, TC_RESID_BF16, TC_RESID_BF16, TC_RESID_BF16, Fk[k][c - 2])) != MRS_OK)
+                    return rc;
+            if (b > 0) second(1, Fk[k - 1][3], dpb[k - 1][0]);
+            if ((rc = conv(h, w, &mDp[k][1].a, -1, 1, WT, trow(lb, 0), zero, 64, TC_RESID_BF16, &mG.o, &mG.o)) != MRS_OK)
+                return rc;
+            second(0, nullptr, nullptr);
         }
         // F_g = chain(F_{g-1}) + F_{g-1}
-        k_sum_bf16<<<grid_for(Pl * 64), 256, 0, st>>>(G, G, dSkip, nullptr, nullptr, nullptr, Pl * 64);
+        k_sum_bf16<<<grid_for(Pl * 8), 256, 0, st>>>(G, G, dSkip, nullptr, nullptr, nullptr, Pl * 8);
         MRS_LAUNCHED(1);
     }
     // fuse: dz = (dL/dF_DF + the chain's gradient) masked by F_0
-    k_sum_bf16<<<grid_for(Pl * 64), 256, 0, st>>>(dzf, gdf, G, nullptr, nullptr, F0, Pl * 64);
+    k_sum_bf16<<<grid_for(Pl * 8), 256, 0, st>>>(dzf, gdf, G, nullptr, nullptr, F0, Pl * 8);
     MRS_LAUNCHED(1);
     // its input gradients, masked by the encoders' ReLU outputs: chunk 0 into
     // F_LRHS's gradient, chunk q into deshuffle view q of F0_HRLS's
-    if ((rc = conv(h, w, &mDzf.a, -1, 1, WT, trow(2, 0), zero, 64, TC_MASK_BF16, &mFlr.o, &mDzlr.o)) != MRS_OK)
-        return rc;
-    for (int q = 1; q <= SS; ++q)
-        if ((rc = conv(h, w, &mDzf.a, -1, 1, WT, trow(2, q), zero, 64, TC_MASK_BF16, &dsfO[q - 1],
-                       &dz1O[q - 1])) != MRS_OK) return rc;
+    if ((rc = convs(1 + SS, h, w, &mDzf.a, mg_fuse, WT, trow(2, 0), zero, false, TC_MASK_BF16, TC_MASK_BF16,
+                    TC_MASK_BF16, TC_MASK_BF16, nullptr)) != MRS_OK) return rc;
     // the weight gradients of every layer in one launch, their sums in another
     // (178 launches each, with 38 to 152 partial sums apiece, were 55% of the
     // step's kernel time)
