@@ -50,7 +50,7 @@ constexpr size_t kParams12 = 599555;
 constexpr size_t kParams21 = 604739;
 constexpr int kCinMax = 21;
 
-inline int nout_of(int l) { return l == kLayers - 1 ? 16 : 64; }
+__host__ __device__ inline int nout_of(int l) { return l == kLayers - 1 ? 16 : 64; }
 
 // ---- input assembly ---------------------------------------------------------
 __device__ __forceinline__ void up_pixel(const float* __restrict__ lr, int h, int w, int s, int x,
@@ -442,15 +442,44 @@ mrs_status conv_simt(const float* x, int cin, const float* wp, const float* b, i
 
 // ---- weight packing ---------------------------------------------------------
 // packed[tap][o][c] (o < nout, c < 64), zero padded; layer l at l * 9*64*64
-__global__ void k_pack_bf16(const float* __restrict__ master, size_t woff, size_t boff, int cin,
-                            int cout, int nout, __nv_bfloat16* __restrict__ wp, float* __restrict__ bp)
+__device__ __forceinline__ void pack_one_bf16(const float* __restrict__ master, size_t woff, size_t boff, int cin,
+                                              int cout, int nout, __nv_bfloat16* __restrict__ wp,
+                                              float* __restrict__ bp, int i)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < 64) bp[i] = i < cout ? master[boff + i] : 0.0f;
     if (i >= 9 * nout * 64) return;
     int c = i % 64, o = (i / 64) % nout, t = i / (64 * nout);
     float v = (o < cout && c < cin) ? master[woff + ((size_t)o * 9 + t) * cin + c] : 0.0f;
     wp[i] = __float2bfloat16_rn(v);
+}
+__global__ void k_pack_bf16(const float* __restrict__ master, size_t woff, size_t boff, int cin,
+                            int cout, int nout, __nv_bfloat16* __restrict__ wp, float* __restrict__ bp)
+{
+    pack_one_bf16(master, woff, boff, cin, cout, nout, wp, bp, blockIdx.x * blockDim.x + threadIdx.x);
+}
+// a network's layers, for the kernels that pack them all in one launch (layer
+// blockIdx.y): a training step repacks every layer, and a launch each (35 with
+// the transposed ones) took 130 us of the fusion network's step, two take 6
+struct PackLayers {
+    long long woff[kLayers], boff[kLayers];
+    int cin[kLayers], cout[kLayers];
+};
+PackLayers pack_layers(int cin0)
+{
+    const auto& L = shapes(cin0);
+    PackLayers p;
+    for (int l = 0; l < kLayers; ++l) {
+        p.woff[l] = (long long)L[l].woff; p.boff[l] = (long long)L[l].boff;
+        p.cin[l] = L[l].cin; p.cout[l] = L[l].cout;
+    }
+    return p;
+}
+__global__ void k_pack_layers_bf16(const float* __restrict__ master, const PackLayers p,
+                                   __nv_bfloat16* __restrict__ wp, float* __restrict__ bp)
+{
+    const int l = blockIdx.y;
+    pack_one_bf16(master, p.woff[l], p.boff[l], p.cin[l], p.cout[l], nout_of(l), wp + (size_t)l * 9 * 64 * 64,
+                  bp + l * 64, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // fp8: per-output-channel scale = amax / 448 over that channel's weights
@@ -597,15 +626,29 @@ __global__ void k_pack_bf16_chunk(const float* __restrict__ w, int cin, int c0, 
     wp[i] = __float2bfloat16_rn(v);
 }
 
+// 8 channels a thread, stored at once: bound by the operand's bytes
 __global__ void k_to_operand(const float* x, size_t P, int cin, void* o, int fp8, float inv)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < P * 64;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < P * 8;
          i += (size_t)gridDim.x * blockDim.x) {
-        size_t p = i / 64;
-        int c = (int)(i % 64);
-        float v = c < cin ? x[p * cin + c] : 0.0f;
-        if (fp8) ((uint8_t*)o)[i] = (uint8_t)__nv_cvt_float_to_fp8(v * inv, __NV_SATFINITE, __NV_E4M3);
-        else ((__nv_bfloat16*)o)[i] = __float2bfloat16_rn(v);
+        const size_t p = i / 8;
+        const int c0 = (int)(i % 8) * 8;
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = c0 + k < cin ? x[p * cin + c0 + k] : 0.0f;
+        if (fp8) {
+            uint2 u;
+            uint8_t* b = (uint8_t*)&u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) b[k] = (uint8_t)__nv_cvt_float_to_fp8(v[k] * inv, __NV_SATFINITE, __NV_E4M3);
+            ((uint2*)o)[i] = u;
+        } else {
+            uint4 u;
+            __nv_bfloat16* b = (__nv_bfloat16*)&u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) b[k] = __float2bfloat16_rn(v[k]);
+            ((uint4*)o)[i] = u;
+        }
     }
 }
 
@@ -1041,21 +1084,26 @@ __global__ void k_gate_select(const float* __restrict__ fused, const float* __re
 // transposed, tap-flipped weights of layer (cin, cout) packed as the
 // tensor-core operand of dX = conv(dY): wp[t][c][o] = w[o][8 - t][c]
 // (rows c < cin of nout, columns o < cout of 64, zero padded)
-__global__ void k_pack_bf16_T(const float* __restrict__ master, size_t woff, int cin, int cout,
-                              int nout, __nv_bfloat16* __restrict__ wp)
+__device__ __forceinline__ void pack_one_bf16_T(const float* __restrict__ master, size_t woff, int cin, int cout,
+                                                int nout, __nv_bfloat16* __restrict__ wp, int i)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 9 * nout * 64) return;
     int o = i % 64, c = (i / 64) % nout, t = i / (64 * nout);
     float v = (c < cin && o < cout) ? master[woff + ((size_t)o * 9 + (8 - t)) * cin + c] : 0.0f;
     wp[i] = __float2bfloat16_rn(v);
 }
-
-// d[i] = act[i] > 0 ? d[i] : 0 over bf16 tensors
-__global__ void k_mask_bf16(__nv_bfloat16* __restrict__ d, const __nv_bfloat16* __restrict__ act, size_t n)
+__global__ void k_pack_bf16_T(const float* __restrict__ master, size_t woff, int cin, int cout,
+                              int nout, __nv_bfloat16* __restrict__ wp)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        if (!(__bfloat162float(act[i]) > 0.0f)) d[i] = __float2bfloat16_rn(0.0f);
+    pack_one_bf16_T(master, woff, cin, cout, nout, wp, blockIdx.x * blockDim.x + threadIdx.x);
+}
+// layers 1 .. of a network, one to a blockIdx.y
+__global__ void k_pack_layers_bf16_T(const float* __restrict__ master, const PackLayers p,
+                                     __nv_bfloat16* __restrict__ wp)
+{
+    const int l = 1 + blockIdx.y;
+    pack_one_bf16_T(master, p.woff[l], p.cin[l], p.cout[l], 64, wp + (size_t)l * 9 * 64 * 64,
+                    blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // out[p][c] = float(o[p][c]) for c < cin from bf16 [P][64] rows
@@ -1138,13 +1186,11 @@ namespace {
 mrs_status pack_bf16(mrs_net_s* net, cudaStream_t st)
 {
     if (net->bf_valid) return MRS_OK;
-    const auto& L = shapes(net->cin0);
+    k_pack_layers_bf16<<<dim3(9 * 64 * 64 / 256, kLayers), 256, 0, st>>>(net->master, pack_layers(net->cin0), net->wbf,
+                                                                         net->bias);
+    MRS_LAUNCHED(1);
     for (int l = 0; l < kLayers; ++l) {
         int nout = nout_of(l);
-        k_pack_bf16<<<(9 * nout * 64 + 255) / 256, 256, 0, st>>>(
-            net->master, L[l].woff, L[l].boff, L[l].cin, L[l].cout, nout,
-            net->wbf + (size_t)l * 9 * 64 * 64, net->bias + l * 64);
-        MRS_LAUNCHED(1);
         mrs_status s = tc_make_w_map(&net->wmap_bf[l], net->wbf + (size_t)l * 9 * 64 * 64, 9 * nout, nout, TC_BF16);
         if (s != MRS_OK) return s;
     }
@@ -1779,13 +1825,11 @@ mrs_status train_step_f32(mrs_net_s* net, const float* lrhs, const float* hrls, 
 mrs_status pack_bf16_T(mrs_net_s* net, cudaStream_t st)
 {
     if (net->bfT_valid) return MRS_OK;
-    const auto& L = shapes(net->cin0);
+    k_pack_layers_bf16_T<<<dim3(9 * 64 * 64 / 256, kLayers - 1), 256, 0, st>>>(net->master, pack_layers(net->cin0),
+                                                                               net->wbfT);
+    MRS_LAUNCHED(1);
     for (int l = 1; l < kLayers; ++l) {
-        __nv_bfloat16* wp = net->wbfT + (size_t)l * 9 * 64 * 64;
-        k_pack_bf16_T<<<(9 * 64 * 64 + 255) / 256, 256, 0, st>>>(net->master, L[l].woff, L[l].cin,
-                                                                 L[l].cout, 64, wp);
-        MRS_LAUNCHED(1);
-        mrs_status rc = tc_make_w_map(&net->wmap_bfT[l], wp, 9 * 64, 64, TC_BF16);
+        mrs_status rc = tc_make_w_map(&net->wmap_bfT[l], net->wbfT + (size_t)l * 9 * 64 * 64, 9 * 64, 64, TC_BF16);
         if (rc != MRS_OK) return rc;
     }
     net->bfT_valid = true;
@@ -1938,11 +1982,10 @@ mrs_status train_step_bf16(mrs_net_s* net, const float* lrhs, const float* hrls,
         int l2 = 2 + 2 * k, l1 = 1 + 2 * k;
         if ((rc = conv(&pl.dhA[k + 1], &net->wmap_bfT[l2], zero, TC_MASK_BF16, &pl.rO[k], &pl.daO[k], 64)) != MRS_OK)
             return rc;
+        a.mask = k == 0 ? hs : nullptr;            // the head's ReLU
         if ((rc = conv(&pl.daA[k], &net->wmap_bfT[l1], zero, TC_RESID_BF16, &pl.dhO[k + 1], &pl.dhO[k], 64)) != MRS_OK)
             return rc;
     }
-    k_mask_bf16<<<grid1d(F), 256, 0, st>>>(dhs, hs, F);
-    MRS_LAUNCHED(1);
     if ((rc = tc_conv3x3_wgrad(pl.wg, pl.blob.p, part, dbpart, net->err, st)) != MRS_OK) return rc;
     if ((rc = wg_reduce(pl.reds, pl.wg.ntiles, part, dbpart, net->grad, st)) != MRS_OK) return rc;
 

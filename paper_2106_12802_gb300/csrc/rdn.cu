@@ -410,15 +410,20 @@ __global__ void k_sum_bf16(__nv_bfloat16* out, const __nv_bfloat16* a, const __n
     }
 }
 
-// bf16 [P][64] rows from FP32 [P][cin] (channels past cin zero)
+// bf16 [P][64] rows from FP32 [P][cin] (channels past cin zero), 8 channels a
+// thread: bound by the rows' bytes, 16 x 192^2 pixels 35 -> 13 us
 __global__ void k_f32_to_bf16_rows(const float* __restrict__ x, size_t P, int cin,
                                    __nv_bfloat16* __restrict__ o)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < P * 64;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < P * 8;
          i += (size_t)gridDim.x * blockDim.x) {
-        const size_t p = i / 64;
-        const int c = (int)(i % 64);
-        o[i] = __float2bfloat16_rn(c < cin ? x[p * cin + c] : 0.0f);
+        const size_t p = i / 8;
+        const int c0 = (int)(i % 8) * 8;
+        uint4 u;
+        __nv_bfloat16* b = (__nv_bfloat16*)&u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) b[k] = __float2bfloat16_rn(c0 + k < cin ? x[p * cin + c0 + k] : 0.0f);
+        ((uint4*)o)[i] = u;
     }
 }
 
@@ -1219,7 +1224,7 @@ mrs_status repack_if_stale(mrs_rdn_s* r, cudaStream_t st)
 // fuse conv's 1 + s^2, an upsampling stage's 4) are one launch, and a mask or sum
 // that follows a conv is in its epilogue.  As 242 conv launches and 81
 // elementwise ones a step of 16 crops of 48 x 48 (x 4) took 5.37 ms of device
-// time, as 130 and 12 3.96 ms.
+// time, as 130 and 10 3.92 ms.
 mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, const float* alb,
                           const float* nrm, const float* extra, const float* tgt, int N, int H, int W,
                           int kind, float beta, float lr, float* yout, double* loss_out,
@@ -1533,7 +1538,7 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
 
     // ---- loss and dL/dI_SR
     if ((rc = loss_grad_f32(y, sTgt, Ph * 3, kTrainClip, kind, beta, dy, lparts, lsum, st)) != MRS_OK) return rc;
-    k_f32_to_bf16_rows<<<grid_for(Ph * 64), 256, 0, st>>>(dy, Ph, 3, dyb);
+    k_f32_to_bf16_rows<<<grid_for(Ph * 8), 256, 0, st>>>(dy, Ph, 3, dyb);
     MRS_LAUNCHED(1);
 
     // ---- backward
@@ -1542,16 +1547,13 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
         MRS_LAUNCHED(1);
     };
     const CUtensorMap* WT = &r->wmapT_all;
-    // H_Rec
-    if ((rc = conv(H, W, &mDyb.a, -1, 1, WT, trow(li_rec, 0), zero, 64, TC_LIN_BF16, nullptr, &mDUl[D].o)) != MRS_OK)
-        return rc;
-    // upsampling stages in reverse: the level-(d + 1) gradient masked by U[d + 1] > 0
-    for (int d = D - 1; d >= 0; --d) {
-        const int lu = 3 + kConv * nblk + d;
-        mask(dUl[d + 1], U[d + 1], Pd[d + 1], dUl[d + 1]);
-        if ((rc = conv(hd[d], wd[d], &dupA[d][0], (long)mc_up[d], 4, WT, trow(lu, 0), zero, 64, TC_LIN_BF16,
-                       nullptr, &mDUl[d].o)) != MRS_OK) return rc;
-    }
+    // H_Rec; a level's gradient is masked by that upsampling stage's ReLU output
+    if ((rc = conv(H, W, &mDyb.a, -1, 1, WT, trow(li_rec, 0), zero, 64, D ? TC_MASK_BF16 : TC_LIN_BF16,
+                   D ? &mU[D].o : nullptr, &mDUl[D].o)) != MRS_OK) return rc;
+    // upsampling stages in reverse
+    for (int d = D - 1; d >= 0; --d)
+        if ((rc = conv(hd[d], wd[d], &dupA[d][0], (long)mc_up[d], 4, WT, trow(3 + kConv * nblk + d, 0), zero, 64,
+                       d ? TC_MASK_BF16 : TC_LIN_BF16, d ? &mU[d].o : nullptr, &mDUl[d].o)) != MRS_OK) return rc;
     __nv_bfloat16* gdf = dUl[0];                  // dL/dF_DF: to F_G (the chain) and to F_0
     MRS_CHECK(cudaMemcpyAsync(G, gdf, Pl * 128, cudaMemcpyDeviceToDevice, st));
     for (int g = kRDG - 1; g >= 0; --g) {
