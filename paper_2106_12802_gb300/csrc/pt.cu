@@ -431,6 +431,33 @@ __device__ __forceinline__ int pixel_of(const JobView& J, int q)
     return (J.win_y0 + lp / J.win_w) * J.W + (J.win_x0 + lp % J.win_w);
 }
 
+// direction of path p's camera ray
+__device__ __forceinline__ V3 camera_dir(const JobView& J, int p)
+{
+    const int q = p - J.path_off;
+    int pix = pixel_of(J, q);
+    int sample = J.s0 + q % J.kk;
+    int px = pix % J.W, py = pix / J.W;
+    float4 g1 = draws((uint32_t)pix, (uint32_t)sample, 0u, 1u, J.key);
+    const float* cam = J.cam;
+    // grid g > 1: only the centre sub-pixel (g px + g/2, g py + g/2) of the
+    // pixel's g x g block is sampled (nearest-neighbour downsampling of a
+    // g-times finer image: the low-resolution renders of Sec. 3); g = 1 is
+    // the whole pixel footprint, the same operations as without a grid
+    const int g = J.grid;
+    float sx = ((float)(px * g + g / 2) + g1.z) / (float)(J.W * g);
+    float sy = ((float)(py * g + g / 2) + g1.w) / (float)(J.H * g);
+    float a = 2.0f * sx - 1.0f, bq = 1.0f - 2.0f * sy;
+    return normalize(mk(cam[3] + cam[6] * a + cam[9] * bq, cam[4] + cam[7] * a + cam[10] * bq,
+                        cam[5] + cam[8] * a + cam[11] * bq));
+}
+
+// The whole state of fresh paths, for a wave whose tail starts at bounce 0.
+// Other waves keep a fresh path's state out of memory (k_trace and k_shade
+// with kFirst): origin, throughput, radiance, pdfs and first-hit layers are
+// the same for all.  Writing the 84 bytes a path and reading them back was bound
+// by memory: 16.8 M paths, generation, first trace and first shading 235 + 1032 +
+// 581 us, now 1065 + 535
 template <class Jobs>
 __device__ __forceinline__ void raygen_body(const WaveParams& w, const Jobs& jobs)
 {
@@ -438,22 +465,8 @@ __device__ __forceinline__ void raygen_body(const WaveParams& w, const Jobs& job
     if (blockIdx.x == 0 && threadIdx.x == 0) w.cnt[0] = (uint32_t)w.n_paths;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < w.n_paths; p += gridDim.x * blockDim.x) {
         const JobView& J = jobs(p);
-        const int q = p - J.path_off;
-        int pix = pixel_of(J, q);
-        int sample = J.s0 + q % J.kk;
-        int px = pix % J.W, py = pix / J.W;
-        float4 g1 = draws((uint32_t)pix, (uint32_t)sample, 0u, 1u, J.key);
+        const V3 d = camera_dir(J, p);
         const float* cam = J.cam;
-        // grid g > 1: only the centre sub-pixel (g px + g/2, g py + g/2) of the
-        // pixel's g x g block is sampled (nearest-neighbour downsampling of a
-        // g-times finer image: the low-resolution renders of Sec. 3); g = 1 is
-        // the whole pixel footprint, the same operations as without a grid
-        const int g = J.grid;
-        float sx = ((float)(px * g + g / 2) + g1.z) / (float)(J.W * g);
-        float sy = ((float)(py * g + g / 2) + g1.w) / (float)(J.H * g);
-        float a = 2.0f * sx - 1.0f, bq = 1.0f - 2.0f * sy;
-        V3 d = normalize(mk(cam[3] + cam[6] * a + cam[9] * bq, cam[4] + cam[7] * a + cam[10] * bq,
-                            cam[5] + cam[8] * a + cam[11] * bq));
         P.ox[p] = cam[0]; P.oy[p] = cam[1]; P.oz[p] = cam[2];
         P.dx[p] = d.x; P.dy[p] = d.y; P.dz[p] = d.z;
         P.bx[p] = 1.0f; P.by[p] = 1.0f; P.bz[p] = 1.0f;
@@ -465,18 +478,29 @@ __device__ __forceinline__ void raygen_body(const WaveParams& w, const Jobs& job
     }
 }
 
-template <bool kCount, class Jobs>
+// kFirst: bounce 0, whose rays are made here
+template <bool kCount, bool kFirst, class Jobs>
 __device__ __forceinline__ void trace_body(const WaveParams& w, const Jobs& jobs, int b)
 {
     unsigned long long nv = 0, nt = 0;
     const PathSoA& P = w.P;
-    const int count = (int)*(volatile uint32_t*)&w.cnt[b];
+    if (kFirst && blockIdx.x == 0 && threadIdx.x == 0) w.cnt[0] = (uint32_t)w.n_paths;
+    const int count = kFirst ? w.n_paths : (int)*(volatile uint32_t*)&w.cnt[b];
     const int* q = (b & 1) ? P.q1 : P.q0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-        int p = b == 0 ? i : q[i];
-        V3 o = mk(P.ox[p], P.oy[p], P.oz[p]), d = mk(P.dx[p], P.dy[p], P.dz[p]);
+        int p = kFirst ? i : q[i];
+        const JobView& J = jobs(p);
+        V3 o, d;
+        if (kFirst) {
+            o = mk(J.cam[0], J.cam[1], J.cam[2]);
+            d = camera_dir(J, p);
+            P.dx[p] = d.x; P.dy[p] = d.y; P.dz[p] = d.z;
+        } else {
+            o = mk(P.ox[p], P.oy[p], P.oz[p]);
+            d = mk(P.dx[p], P.dy[p], P.dz[p]);
+        }
         float t = -1.0f;
-        int k = traverse<false, kCount>(jobs(p).S, o, d, T_INF, t, &nv, &nt);
+        int k = traverse<false, kCount>(J.S, o, d, T_INF, t, &nv, &nt);
         P.hit_t[p] = t;
         P.hit_id[p] = k;
     }
@@ -518,7 +542,9 @@ __device__ __forceinline__ ShadeConst shade_const(const JobView& J)
 // (shadow ray and its contribution left in P.sd* / P.sc*), BSDF sampling and
 // roulette.  cont: the path continues to bounce b + 1; shadow: a shadow ray
 // was set up.  Shared by the wavefront kernel and the tail kernel, so that a
-// path's arithmetic does not depend on which one shades it.
+// path's arithmetic does not depend on which one shades it.  kFirst: bounce 0 of
+// a path whose state is not in memory yet (see raygen_body).
+template <bool kFirst>
 __device__ __forceinline__ void shade_path(const WaveParams& w, const JobView& J,
                                            const ShadeConst& sc0, int b, int p, bool& cont,
                                            bool& shadow)
@@ -529,14 +555,30 @@ __device__ __forceinline__ void shade_path(const WaveParams& w, const JobView& J
     const bool env_on = sc0.env_on;
     const int n_choices = sc0.n_choices;
     const float pick = sc0.pick;
-    V3 o = mk(P.ox[p], P.oy[p], P.oz[p]), d = mk(P.dx[p], P.dy[p], P.dz[p]);
-    V3 beta = mk(P.bx[p], P.by[p], P.bz[p]);
-    V3 L = mk(P.Lx[p], P.Ly[p], P.Lz[p]);
-    float pdf_b = P.pdf_b[p], pdf_e = P.pdf_e[p];
+    V3 o, d = mk(P.dx[p], P.dy[p], P.dz[p]), beta, L;
+    float pdf_b, pdf_e;
+    if (kFirst) {
+        b = 0;
+        o = mk(J.cam[0], J.cam[1], J.cam[2]);
+        beta = mk(1.0f, 1.0f, 1.0f);
+        L = mk(0.0f, 0.0f, 0.0f);
+        pdf_b = pdf_e = 0.0f;
+    } else {
+        o = mk(P.ox[p], P.oy[p], P.oz[p]);
+        beta = mk(P.bx[p], P.by[p], P.bz[p]);
+        L = mk(P.Lx[p], P.Ly[p], P.Lz[p]);
+        pdf_b = P.pdf_b[p];
+        pdf_e = P.pdf_e[p];
+    }
     int k = P.hit_id[p];
     float t = P.hit_t[p];
     do {
         if (k < 0) {
+            if (kFirst) {
+                P.ax[p] = 0.0f; P.ay[p] = 0.0f; P.az[p] = 0.0f;
+                P.nx[p] = 0.0f; P.ny[p] = 0.0f; P.nz[p] = 0.0f; P.dep[p] = 0.0f;
+                if (w.layers) P.lobe[p] = 0;
+            }
             if (env_on) {
                 float wgt = 1.0f;
                 if (b > 0 && pdf_e > 0.0f)
@@ -658,7 +700,7 @@ __device__ __forceinline__ void shade_path(const WaveParams& w, const JobView& J
     P.Lx[p] = L.x; P.Ly[p] = L.y; P.Lz[p] = L.z;
 }
 
-template <class Jobs>
+template <bool kFirst, class Jobs>
 __device__ __forceinline__ void shade_body(const WaveParams& w, const Jobs& jobs, int b)
 {
     const PathSoA& P = w.P;
@@ -671,9 +713,9 @@ __device__ __forceinline__ void shade_body(const WaveParams& w, const Jobs& jobs
         bool cont = false, shadow = false;
         int p = 0;
         if (i < count) {
-            p = b == 0 ? i : q[i];
+            p = kFirst ? i : q[i];
             const JobView& J = jobs(p);
-            shade_path(w, J, shade_const(J), b, p, cont, shadow);
+            shade_path<kFirst>(w, J, shade_const(J), b, p, cont, shadow);
         }
         int slot = warp_append(cont, &w.cnt[b + 1]);
         if (cont) qn[slot] = p;
@@ -757,7 +799,7 @@ __device__ __forceinline__ void tail_body(const WaveParams& w, const Jobs& jobs,
         P.hit_t[p] = t;
         P.hit_id[p] = k;
         bool cont = false, shadow = false;
-        shade_path(w, J, shade_const(J), b, p, cont, shadow);
+        shade_path<false>(w, J, shade_const(J), b, p, cont, shadow);
         if (shadow) {
             atomicAdd(&s_scnt[b], 1u);
             V3 so = mk(P.ox[p], P.oy[p], P.oz[p]), sd = mk(P.sdx[p], P.sdy[p], P.sdz[p]);
@@ -794,24 +836,27 @@ __global__ void __launch_bounds__(kThreads)
 {
     raygen_body(w, ManyJobs{T});
 }
-template <bool kCount>
+template <bool kCount, bool kFirst>
 __global__ void __launch_bounds__(kThreads, 8) k_trace(const __grid_constant__ WaveParams w, int b)
 {
-    trace_body<kCount>(w, OneJob{w.J}, b);
+    trace_body<kCount, kFirst>(w, OneJob{w.J}, b);
 }
+template <bool kFirst>
 __global__ void __launch_bounds__(kThreads, 8)
     k_trace_b(const __grid_constant__ WaveParams w, const __grid_constant__ JobTable T, int b)
 {
-    trace_body<false>(w, ManyJobs{T}, b);
+    trace_body<false, kFirst>(w, ManyJobs{T}, b);
 }
+template <bool kFirst>
 __global__ void __launch_bounds__(kThreads) k_shade(const __grid_constant__ WaveParams w, int b)
 {
-    shade_body(w, OneJob{w.J}, b);
+    shade_body<kFirst>(w, OneJob{w.J}, b);
 }
+template <bool kFirst>
 __global__ void __launch_bounds__(kThreads)
     k_shade_b(const __grid_constant__ WaveParams w, const __grid_constant__ JobTable T, int b)
 {
-    shade_body(w, ManyJobs{T}, b);
+    shade_body<kFirst>(w, ManyJobs{T}, b);
 }
 template <bool kCount>
 __global__ void __launch_bounds__(kThreads, 8) k_shadow(const __grid_constant__ WaveParams w, int b)
@@ -839,8 +884,10 @@ __global__ void __launch_bounds__(kThreads, kBlocks)
 // Path p of a wave is sample p % kk of pixel p / kk: a pixel's samples are
 // consecutive paths, so a warp's camera rays leave through one or a few
 // pixels (coherent bounce-0 traversal and shading).  The accumulation reads
-// each pixel's kk consecutive samples, V at a time (one 16-byte load per
-// field when kk is a multiple of 4: a warp's loads are then contiguous).
+// each pixel's kk consecutive samples, V at a time: whole 32-byte sectors when
+// kk is a multiple of 8 (lanes are kk values apart, so 16-byte loads fetched each
+// sector twice: 16.8 M paths, kk = 16, 338 -> 153 us; three blocks an SM let all
+// ten fields' loads be in flight), 16 bytes when it is one of 4.
 template <int V> struct Vec;
 template <> struct Vec<1> {
     float v[1];
@@ -862,9 +909,20 @@ template <> struct Vec<4> {
     }
 };
 
+template <> struct Vec<8> {
+    float v[8];
+    __device__ __forceinline__ void load(const float* p)
+    {
+        asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+            : "l"(p) : "memory");
+    }
+    __device__ __forceinline__ void load_int(const int* p) { load(reinterpret_cast<const float*>(p)); }
+};
+
 // per pixel: add this wave's samples in sample order (Kahan for radiance)
 template <int V>
-__global__ void __launch_bounds__(kThreads) k_accumulate(const __grid_constant__ WaveParams w,
+__global__ void __launch_bounds__(kThreads, V == 8 ? 3 : 1) k_accumulate(const __grid_constant__ WaveParams w,
                                                           float* acc, int kk)
 {
     const PathSoA& P = w.P;
@@ -1038,6 +1096,13 @@ template <class K> int persistent_grid(K kernel)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0);
     return sm_count() * (per_sm < 1 ? 1 : per_sm);
 }
+void launch_trace(bool count, const WaveParams& w, int b, int g, cudaStream_t st)
+{
+    if (count && b == 0) k_trace<true, true><<<g, kThreads, 0, st>>>(w, b);
+    else if (count) k_trace<true, false><<<g, kThreads, 0, st>>>(w, b);
+    else if (b == 0) k_trace<false, true><<<g, kThreads, 0, st>>>(w, b);
+    else k_trace<false, false><<<g, kThreads, 0, st>>>(w, b);
+}
 template <bool kCount, int kBlocks> void launch_tail(const WaveParams& w, int b0, cudaStream_t st)
 {
     static const int g = persistent_grid(k_tail<kCount, kBlocks>);
@@ -1058,6 +1123,28 @@ inline int grid_for(int64_t n)
     int64_t cap = (int64_t)sm_count() * 8;
     if (g > cap) g = cap;
     return (int)(g < 1 ? 1 : g);
+}
+
+// samples loaded at a time (Vec): every pixel's run of kk samples has to start
+// on the load's boundary (the arrays are 256-byte aligned)
+inline int accumulate_width(const WaveParams& w, int kk)
+{
+    const int64_t off = w.J.path_off;
+    return kk % 8 == 0 && off % 8 == 0 ? 8 : kk % 4 == 0 && off % 4 == 0 ? 4 : 1;
+}
+void launch_accumulate(const WaveParams& w, float* acc, int kk, cudaStream_t st)
+{
+    const int v = accumulate_width(w, kk), g = grid_for(w.wh);
+    if (v == 8) k_accumulate<8><<<g, kThreads, 0, st>>>(w, acc, kk);
+    else if (v == 4) k_accumulate<4><<<g, kThreads, 0, st>>>(w, acc, kk);
+    else k_accumulate<1><<<g, kThreads, 0, st>>>(w, acc, kk);
+}
+void launch_accumulate_layers(const WaveParams& w, float* acc2, int kk, cudaStream_t st)
+{
+    const int v = accumulate_width(w, kk), g = grid_for(w.wh);
+    if (v == 8) k_accumulate_layers<8><<<g, kThreads, 0, st>>>(w, acc2, kk);
+    else if (v == 4) k_accumulate_layers<4><<<g, kThreads, 0, st>>>(w, acc2, kk);
+    else k_accumulate_layers<1><<<g, kThreads, 0, st>>>(w, acc2, kk);
 }
 
 }  // namespace
@@ -1155,15 +1242,17 @@ static mrs_status render_impl(mrs_scene S, Buf& arena, int64_t wave_paths, int32
         w.n_paths = w.J.n_paths;
         MRS_CHECK(cudaMemsetAsync(cnt, 0, 4 * 2 * 64, st));
         int g = grid_for(w.n_paths);
-        MRS_TIMED(PK_RAYGEN, st, k_raygen<<<g, kThreads, 0, st>>>(w));
-        MRS_LAUNCHED(1);
         const TailPlan plan = tail_plan(w.n_paths, tail);
         const int b_tail = plan.bounce;
-        for (int b = 0; b <= max_depth && b < b_tail; ++b) {
-            if (stats) MRS_TIMED(PK_TRACE, st, k_trace<true><<<g, kThreads, 0, st>>>(w, b));
-            else MRS_TIMED(PK_TRACE, st, k_trace<false><<<g, kThreads, 0, st>>>(w, b));
+        if (b_tail == 0) {
+            MRS_TIMED(PK_RAYGEN, st, k_raygen<<<g, kThreads, 0, st>>>(w));
             MRS_LAUNCHED(1);
-            MRS_TIMED(PK_SHADE, st, k_shade<<<g, kThreads, 0, st>>>(w, b));
+        }
+        for (int b = 0; b <= max_depth && b < b_tail; ++b) {
+            MRS_TIMED(PK_TRACE, st, launch_trace(stats != nullptr, w, b, g, st));
+            MRS_LAUNCHED(1);
+            if (b == 0) MRS_TIMED(PK_SHADE, st, k_shade<true><<<g, kThreads, 0, st>>>(w, b));
+            else MRS_TIMED(PK_SHADE, st, k_shade<false><<<g, kThreads, 0, st>>>(w, b));
             MRS_LAUNCHED(1);
             if (stats) MRS_TIMED(PK_SHADOW, st, k_shadow<true><<<g, kThreads, 0, st>>>(w, b));
             else MRS_TIMED(PK_SHADOW, st, k_shadow<false><<<g, kThreads, 0, st>>>(w, b));
@@ -1175,17 +1264,10 @@ static mrs_status render_impl(mrs_scene S, Buf& arena, int64_t wave_paths, int32
             else if (plan.blocks == 5) launch_tail<false, 5>(w, b_tail, st);
             else launch_tail<false, 4>(w, b_tail, st);
         }
-        // 16-byte sample loads when every pixel's run of kk samples starts on
-        // a 16-byte boundary (the arrays are 256-byte aligned)
-        const bool v4 = kk % 4 == 0;
-        if (v4) MRS_TIMED(PK_ACCUM, st, k_accumulate<4><<<grid_for(wh), kThreads, 0, st>>>(w, acc, kk));
-        else MRS_TIMED(PK_ACCUM, st, k_accumulate<1><<<grid_for(wh), kThreads, 0, st>>>(w, acc, kk));
+        MRS_TIMED(PK_ACCUM, st, launch_accumulate(w, acc, kk, st));
         MRS_LAUNCHED(1);
         if (acc2) {
-            if (v4)
-                MRS_TIMED(PK_ACCUM, st, k_accumulate_layers<4><<<grid_for(wh), kThreads, 0, st>>>(w, acc2, kk));
-            else
-                MRS_TIMED(PK_ACCUM, st, k_accumulate_layers<1><<<grid_for(wh), kThreads, 0, st>>>(w, acc2, kk));
+            MRS_TIMED(PK_ACCUM, st, launch_accumulate_layers(w, acc2, kk, st));
             MRS_LAUNCHED(1);
         }
         if (counts || shadow_counts) {
@@ -1422,11 +1504,18 @@ mrs_status render_batch_impl(mrs_ctx ctx, const mrs_render_job* jobs, int32_t n_
         const TailPlan plan = tail_plan(off, ctx->tail_bounce);
         const int b_tail = plan.bounce;
         const int g = grid_for(off);
-        MRS_TIMED(PK_RAYGEN, st, k_raygen_b<<<g, kThreads, 0, st>>>(w, T));
-        MRS_LAUNCHED(1);
+        if (b_tail == 0) {
+            MRS_TIMED(PK_RAYGEN, st, k_raygen_b<<<g, kThreads, 0, st>>>(w, T));
+            MRS_LAUNCHED(1);
+        }
         for (int b = 0; b <= maxd && b < b_tail; ++b) {
-            MRS_TIMED(PK_TRACE, st, k_trace_b<<<g, kThreads, 0, st>>>(w, T, b));
-            MRS_TIMED(PK_SHADE, st, k_shade_b<<<g, kThreads, 0, st>>>(w, T, b));
+            if (b == 0) {
+                MRS_TIMED(PK_TRACE, st, k_trace_b<true><<<g, kThreads, 0, st>>>(w, T, b));
+                MRS_TIMED(PK_SHADE, st, k_shade_b<true><<<g, kThreads, 0, st>>>(w, T, b));
+            } else {
+                MRS_TIMED(PK_TRACE, st, k_trace_b<false><<<g, kThreads, 0, st>>>(w, T, b));
+                MRS_TIMED(PK_SHADE, st, k_shade_b<false><<<g, kThreads, 0, st>>>(w, T, b));
+            }
             MRS_TIMED(PK_SHADOW, st, k_shadow_b<<<g, kThreads, 0, st>>>(w, T, b));
             MRS_LAUNCHED(3);
         }
@@ -1442,9 +1531,7 @@ mrs_status render_batch_impl(mrs_ctx ctx, const mrs_render_job* jobs, int32_t n_
             wc.J = T.J[c - wv.first];
             wc.wh = (int64_t)jobs[ch.job].W * jobs[ch.job].H;
             float* a = acc + acc_off[ch.job] * 13;
-            const bool v4 = ch.kk % 4 == 0 && wc.J.path_off % 4 == 0;
-            if (v4) MRS_TIMED(PK_ACCUM, st, k_accumulate<4><<<grid_for(wc.wh), kThreads, 0, st>>>(wc, a, ch.kk));
-            else MRS_TIMED(PK_ACCUM, st, k_accumulate<1><<<grid_for(wc.wh), kThreads, 0, st>>>(wc, a, ch.kk));
+            MRS_TIMED(PK_ACCUM, st, launch_accumulate(wc, a, ch.kk, st));
             MRS_LAUNCHED(1);
         }
     }
