@@ -309,9 +309,11 @@ template <int NOUT, int OPER> size_t fold_smem_bytes(int stages)
 __device__ __forceinline__ const TcConvArgs& more_of(const TcConvArgs& a) { return a; }
 __device__ __forceinline__ TcConvArgs more_of(const TcConvBase&) { return TcConvArgs{}; }
 
-// kMore: groups, masked sums and second results (TcConvArgs::ng, mask, op2);
-// tested for at run time in every conv they cost the inference layers 1 to 2%
-template <int NOUT, int OPER, bool kMore>
+// kImages: several images a tile (tc_images).  kMore: also groups, masked sums
+// and second results (TcConvArgs::ng, mask, op2).  Variants, because the tests
+// for them cost a layer that has neither: 3% on an image of 256 x 128 (fusion
+// network 171 against 166 us in BF16, 165 against 159 in FP8), 2% on a large one.
+template <int NOUT, int OPER, bool kImages, bool kMore>
 __global__ void __launch_bounds__(kThreads, 1)
     k_conv_fold(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                 const __grid_constant__ CUtensorMap tmap_res,
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int XB = (a.W + kFoldTile - 1) / kFoldTile;
-    const int im = tc_images(a.N, a.W), pitch = a.W + 2;      // images per tile, their rows apart
+    const int im = kImages ? tc_images(a.N, a.W) : 1, pitch = a.W + 2;      // images per tile, their rows apart
     const long long T = (long long)((a.N + im - 1) / im) * XB * a.H;
     // the CTA's group (of ng convolutions of the same input) and its place in it
     const int ng = kMore && more.ng > 1 ? more.ng : 1, group = kMore ? (int)blockIdx.x * ng / (int)gridDim.x : 0;
@@ -799,14 +801,14 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 // input-row ring depth of the conv (0: the most that fits shared memory)
 std::atomic<int> g_fold_ring{0};
 
-template <int NOUT, int OPER, bool kMore>
+template <int NOUT, int OPER, bool kImages, bool kMore>
 mrs_status launch_fold(const TcConvArgs& a, cudaStream_t st)
 {
     int smax = 4;
     while (fold_smem_bytes<NOUT, OPER>(smax + 1) <= 227 * 1024 && smax < 12) ++smax;
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_fold<NOUT, OPER, kMore>,
+        cudaError_t e = cudaFuncSetAttribute(k_conv_fold<NOUT, OPER, kImages, kMore>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)fold_smem_bytes<NOUT, OPER>(smax));
         if (e != cudaSuccess) return cuda_status(e, "conv smem attribute");
@@ -835,7 +837,7 @@ mrs_status launch_fold(const TcConvArgs& a, cudaStream_t st)
     cfg.attrs = la;
     cfg.numAttrs = 1;
     cudaError_t le = cudaSuccess;
-    MRS_TIMED(PK_CONV_TC, st, (le = cudaLaunchKernelEx(&cfg, k_conv_fold<NOUT, OPER, kMore>, *a.tmap_x, *a.tmap_w, *res, *out, b, stages)));
+    MRS_TIMED(PK_CONV_TC, st, (le = cudaLaunchKernelEx(&cfg, k_conv_fold<NOUT, OPER, kImages, kMore>, *a.tmap_x, *a.tmap_w, *res, *out, b, stages)));
     MRS_LAUNCHED(1);
     if (le != cudaSuccess) return cuda_status(le, "conv launch");
     return cuda_status(cudaGetLastError(), "conv launch");
@@ -960,16 +962,21 @@ mrs_status tc_conv3x3(const TcConvArgs& a, cudaStream_t st)
         return MRS_ERR_ARG;
     }
     if (a.ng > 1 || a.mask || a.op2) {
-        if (a.nout == 64 && a.operand == TC_BF16) return launch_fold<64, TC_BF16, true>(a, st);
+        if (a.nout == 64 && a.operand == TC_BF16) return launch_fold<64, TC_BF16, true, true>(a, st);
         set_error("tc_conv3x3: groups, masks and second results need 64 BF16 channels");
         return MRS_ERR_ARG;
     }
-    if (a.nout == 64)
-        return a.operand == TC_BF16 ? launch_fold<64, TC_BF16, false>(a, st) : launch_fold<64, TC_FP8, false>(a, st);
-    if (a.nout == 16)
-        return a.operand == TC_BF16 ? launch_fold<16, TC_BF16, false>(a, st) : launch_fold<16, TC_FP8, false>(a, st);
-    set_error("tc_conv3x3: nout must be 64 or 16");
-    return MRS_ERR_ARG;
+    if (a.nout != 64 && a.nout != 16) {
+        set_error("tc_conv3x3: nout must be 64 or 16");
+        return MRS_ERR_ARG;
+    }
+    const bool wide = a.nout == 64, bf = a.operand == TC_BF16;
+    if (tc_images(a.N, a.W) > 1) {
+        if (wide) return bf ? launch_fold<64, TC_BF16, true, false>(a, st) : launch_fold<64, TC_FP8, true, false>(a, st);
+        return bf ? launch_fold<16, TC_BF16, true, false>(a, st) : launch_fold<16, TC_FP8, true, false>(a, st);
+    }
+    if (wide) return bf ? launch_fold<64, TC_BF16, false, false>(a, st) : launch_fold<64, TC_FP8, false, false>(a, st);
+    return bf ? launch_fold<16, TC_BF16, false, false>(a, st) : launch_fold<16, TC_FP8, false, false>(a, st);
 }
 
 
