@@ -114,21 +114,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
     return mbar_wait_limit(bar, parity, err, kTimeoutCycles, 1000000u);
 }
 
-// every lane polls; the answer is the same for the whole warp
+// every lane polls; the answer is the same for the whole warp.  (Lane 0 polling
+// for the warp, a shuffle and a second look by all lanes took some 500 cycles
+// more a wait; polling without the suspending wait takes issue slots and made
+// the convolutions 4 to 10% slower.)
 __device__ __forceinline__ bool mbar_wait_all(uint64_t* bar, uint32_t parity, int* err)
 {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
-}
-
-// warp-wide wait: lane 0 polls, then every lane observes the completed phase
-// once (acquiring the data the phase guards)
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err)
-{
-    bool ok = true;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, err);
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    if (ok) (void)mbar_try_wait(bar, parity);
-    return ok;
 }
 
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int c0, int c1,
@@ -625,9 +617,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 u2[0] = *(const uint4*)(aux + p * 64 + grp * 16);
                 u2[1] = *(const uint4*)(aux + p * 64 + grp * 16 + 8);
             }
-            if (!mbar_wait_warp(&tfull[sl], use & 1, a.err)) { stop = true; break; }
+            // the staging slot first: it is usually free, and off the row's critical path
+            if (!mbar_wait_all(&rfull[slot], suse & 1, a.err)) { stop = true; break; }
+            if (!mbar_wait_all(&tfull[sl], use & 1, a.err)) { stop = true; break; }
             tc_fence_after();
-            if (!mbar_wait_warp(&rfull[slot], suse & 1, a.err)) { stop = true; break; }
             uint8_t* srow = sS + slot * SBYTES;
             if (active) {
                 const int c0 = grp * 16;
@@ -1204,7 +1197,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
 #pragma unroll
             for (int i = 0; i < 96; ++i) acc[i] = 0.0f;
             for (int g = w; g < runs; g += classes, ++k) {
-                if (!mbar_wait_warp(done, k & 1, err)) { ok = false; break; }
+                if (!mbar_wait_all(done, k & 1, err)) { ok = false; break; }
                 tc_fence_after();
 #pragma unroll
                 for (int h = 0; h < 12; ++h) {
