@@ -20,7 +20,7 @@
 //           residual / mask / FP32 partial sum / bilinear skip, BF16 results
 //           written into the staging slot (swizzled) and sent out by one TMA
 //           store per tile, or FP32 results stored directly
-//   warp 18: residual prefetch into one of three staging slots
+//   warp 18: residual prefetch into one of three or four staging slots
 //   warp 19: output TMA stores from the staging slots
 // Every wait is bounded (no hardware barrier inside the role loops): on
 // timeout the kernel sets *err, all roles unwind, TMEM is freed, and the host
@@ -45,7 +45,10 @@ constexpr int kEpiWarps = 16;                  // 4 per TMEM lane quarter
 constexpr int kResWarp = 2 + kEpiWarps;        // residual-prefetch warp
 constexpr int kStoreWarp = kResWarp + 1;       // output-store warp
 constexpr int kThreads = 32 * (kStoreWarp + 1);  // A-TMA, MMA, epilogue, residual, store warps
-constexpr int kSlots = 3;                      // residual / output staging slots
+// residual / output staging slots; epilogue warps of one row.  kAlt: the warps
+// form two groups that take alternate rows (each slot then belongs to one group)
+constexpr int fold_slots(bool alt) { return alt ? 4 : 3; }
+constexpr int fold_row_warps(bool alt) { return alt ? kEpiWarps / 2 : kEpiWarps; }
 constexpr long long kTimeoutCycles = 4000000000LL;   // ~2 s at 2 GHz
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -292,8 +295,9 @@ constexpr int kFoldMaxRows = 6;              // output rows per sub-piece of a m
 constexpr int fold_rowb(int oper) { return oper == TC_BF16 ? 128 : 64; }
 constexpr int fold_aslot(int oper) { return ((kFoldABox * fold_rowb(oper) + 1023) / 1024) * 1024; }
 
-template <int NOUT, int OPER> size_t fold_smem_bytes(int stages)
+template <int NOUT, int OPER, bool kAlt> size_t fold_smem_bytes(int stages)
 {
+    constexpr int kSlots = fold_slots(kAlt);
     return 1024 + ((9 * NOUT * fold_rowb(OPER) + 1023) & ~1023) + (size_t)stages * fold_aslot(OPER) +
            (size_t)kSlots * kFoldTile * 128 + 2 * 64 * 4 + 8 * (2 * stages + 2 + 2 * (512 / NOUT) + 3 * kSlots) + 16;
 }
@@ -305,7 +309,10 @@ __device__ __forceinline__ TcConvArgs more_of(const TcConvBase&) { return TcConv
 // and second results (TcConvArgs::ng, mask, op2).  Variants, because the tests
 // for them cost a layer that has neither: 3% on an image of 256 x 128 (fusion
 // network 171 against 166 us in BF16, 165 against 159 in FP8), 2% on a large one.
-template <int NOUT, int OPER, bool kImages, bool kMore>
+// kAlt: the epilogue's two groups have two rows' time for one row's latency, but
+// each row takes twice as long (a warp has 32 of its 64 channels): for CTAs with
+// rows enough (see tc_conv3x3).
+template <int NOUT, int OPER, bool kImages, bool kMore, bool kAlt>
 __global__ void __launch_bounds__(kThreads, 1)
     k_conv_fold(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                 const __grid_constant__ CUtensorMap tmap_res,
@@ -313,6 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const std::conditional_t<kMore, TcConvArgs, TcConvBase> a, int stages)
 {
     const auto& more = more_of(a);
+    constexpr int kSlots = fold_slots(kAlt), kRowWarps = fold_row_warps(kAlt);
     constexpr int NS = 512 / NOUT;                            // TMEM accumulator slots
     constexpr int ROWB = fold_rowb(OPER);                     // bytes per operand row
     constexpr int ASLOT = fold_aslot(OPER);
@@ -368,12 +376,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(wempty, 1);
         for (int i = 0; i < NS; ++i) {
             mbar_init(&tfull[i], 1);
-            mbar_init(&sfree[i], kEpiWarps);
+            mbar_init(&sfree[i], kRowWarps);
         }
         for (int i = 0; i < kSlots; ++i) {
             mbar_init(&rfull[i], 1);
             mbar_init(&rempty[i], 1);
-            mbar_init(&edone[i], kEpiWarps);
+            mbar_init(&edone[i], kRowWarps);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -592,13 +600,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else {
         // epilogue: warp w reads TMEM lanes 32 q .. 32 q + 31 (output pixels
-        // x0 + 32 q + lane) and channels [16 grp, 16 grp + 16) of the finished
+        // x0 + 32 q + lane) and channels [ch0, ch0 + 16 kBlk) of the finished
         // output row's slot, then zeroes them.  (FP8: the factors come from shared
         // memory and values are converted in pairs; loading a factor and converting
         // value by value bound the row: the network at 512 x 288 0.255 -> 0.233 ms)
         const int q = warp & 3, grp = (warp - 2) >> 2;
+        constexpr int kBlk = kAlt && NOUT >= 64 ? 2 : 1;       // 16-channel blocks of a warp
+        const int ch0 = (kAlt ? grp >> 1 : grp) * 16 * kBlk;
         const int j = q * 32 + lane;
-        const bool active = grp * 16 < NOUT;
+        const bool active = ch0 < NOUT;
         // the lane's image in its tile and pixel in the strip
         const bool masked = kMore && more.mask && group == ng - 1 && mode == TC_RESID_BF16;
         const __nv_bfloat16* aux = (const __nv_bfloat16*)(masked ? more.mask : kMore && more.op2 ? more.x2 : nullptr);
@@ -609,6 +619,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           int xb, n, y0, y1;
           piece_rows(f, f1, XB, a.H, xb, n, y0, y1);
           for (int y = y0; y < y1; ++y, ++lt) {
+            if (kAlt && (int)(lt & 1) != (grp & 1)) continue;
             const int sl = (int)((NS - (int)(lt % NS)) % NS);
             const uint32_t use = lt / NS;
             const uint32_t slot = lt % kSlots, suse = lt / kSlots;
@@ -616,22 +627,27 @@ __global__ void __launch_bounds__(kThreads, 1)
             const bool valid = x < a.W && ji < im && img < a.N;
             const size_t p = valid ? ((size_t)img * a.H + y) * a.W + x : 0;
             // the mask's or second result's operand, read while the row is computed
-            uint4 u2[2];
-            if (kMore && aux && active && valid) {
-                u2[0] = *(const uint4*)(aux + p * 64 + grp * 16);
-                u2[1] = *(const uint4*)(aux + p * 64 + grp * 16 + 8);
-            }
+            uint4 ux[2 * kBlk];
+            if (kMore && aux && active && valid)
+#pragma unroll
+                for (int e = 0; e < 2 * kBlk; ++e) ux[e] = *(const uint4*)(aux + p * 64 + ch0 + 8 * e);
             // the staging slot first: it is usually free, and off the row's critical path
             if (!mbar_wait_all(&rfull[slot], suse & 1, a.err)) { stop = true; break; }
             if (!mbar_wait_all(&tfull[sl], use & 1, a.err)) { stop = true; break; }
             tc_fence_after();
             uint8_t* srow = sS + slot * SBYTES;
             if (active) {
-                const int c0 = grp * 16;
-                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(sl * NOUT + c0);
-                uint32_t r0[16];
-                tmem_ld16(taddr, r0);
-                tmem_wait_ld();
+              const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(sl * NOUT);
+              uint32_t rr[kBlk][16];
+#pragma unroll
+              for (int blk = 0; blk < kBlk; ++blk) tmem_ld16(trow + ch0 + 16 * blk, rr[blk]);
+              tmem_wait_ld();
+#pragma unroll
+              for (int blk = 0; blk < kBlk; ++blk) {
+                const int c0 = ch0 + 16 * blk;
+                const uint32_t taddr = trow + c0;
+                const uint4* u2 = ux + 2 * blk;
+                const uint32_t (&r0)[16] = rr[blk];
                 uint32_t z[16];
 #pragma unroll
                 for (int e = 0; e < 16; ++e) z[e] = 0u;
@@ -761,7 +777,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                     }
                 }
-                tmem_wait_st();
+              }
+              tmem_wait_st();
             }
             // the slot is read and zeroed; the staging slot goes to the store warp
             tc_fence_before();
@@ -799,22 +816,22 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 // input-row ring depth of the conv (0: the most that fits shared memory)
 std::atomic<int> g_fold_ring{0};
 
-template <int NOUT, int OPER, bool kImages, bool kMore>
+template <int NOUT, int OPER, bool kImages, bool kMore, bool kAlt>
 mrs_status launch_fold(const TcConvArgs& a, cudaStream_t st)
 {
     int smax = 4;
-    while (fold_smem_bytes<NOUT, OPER>(smax + 1) <= 227 * 1024 && smax < 12) ++smax;
+    while (fold_smem_bytes<NOUT, OPER, kAlt>(smax + 1) <= 227 * 1024 && smax < 12) ++smax;
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_fold<NOUT, OPER, kImages, kMore>,
+        cudaError_t e = cudaFuncSetAttribute(k_conv_fold<NOUT, OPER, kImages, kMore, kAlt>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)fold_smem_bytes<NOUT, OPER>(smax));
+                                             (int)fold_smem_bytes<NOUT, OPER, kAlt>(smax));
         if (e != cudaSuccess) return cuda_status(e, "conv smem attribute");
         attr = true;
     }
     const int want = g_fold_ring.load(std::memory_order_relaxed);
     const int stages = want >= 3 ? (want < smax ? want : smax) : smax;
-    size_t smem = fold_smem_bytes<NOUT, OPER>(stages);
+    size_t smem = fold_smem_bytes<NOUT, OPER, kAlt>(stages);
     const std::conditional_t<kMore, TcConvArgs, TcConvBase> b = a;
     const int im = tc_images(a.N, a.W);
     const long long T = (long long)((a.N + im - 1) / im) * ((a.W + kFoldTile - 1) / kFoldTile) * a.H;
@@ -835,7 +852,7 @@ mrs_status launch_fold(const TcConvArgs& a, cudaStream_t st)
     cfg.attrs = la;
     cfg.numAttrs = 1;
     cudaError_t le = cudaSuccess;
-    MRS_TIMED(PK_CONV_TC, st, (le = cudaLaunchKernelEx(&cfg, k_conv_fold<NOUT, OPER, kImages, kMore>, *a.tmap_x, *a.tmap_w, *res, *out, b, stages)));
+    MRS_TIMED(PK_CONV_TC, st, (le = cudaLaunchKernelEx(&cfg, k_conv_fold<NOUT, OPER, kImages, kMore, kAlt>, *a.tmap_x, *a.tmap_w, *res, *out, b, stages)));
     MRS_LAUNCHED(1);
     if (le != cudaSuccess) return cuda_status(le, "conv launch");
     return cuda_status(cudaGetLastError(), "conv launch");
@@ -960,7 +977,7 @@ mrs_status tc_conv3x3(const TcConvArgs& a, cudaStream_t st)
         return MRS_ERR_ARG;
     }
     if (a.ng > 1 || a.mask || a.op2) {
-        if (a.nout == 64 && a.operand == TC_BF16) return launch_fold<64, TC_BF16, true, true>(a, st);
+        if (a.nout == 64 && a.operand == TC_BF16) return launch_fold<64, TC_BF16, true, true, false>(a, st);
         set_error("tc_conv3x3: groups, masks and second results need 64 BF16 channels");
         return MRS_ERR_ARG;
     }
@@ -970,11 +987,22 @@ mrs_status tc_conv3x3(const TcConvArgs& a, cudaStream_t st)
     }
     const bool wide = a.nout == 64, bf = a.operand == TC_BF16;
     if (tc_images(a.N, a.W) > 1) {
-        if (wide) return bf ? launch_fold<64, TC_BF16, true, false>(a, st) : launch_fold<64, TC_FP8, true, false>(a, st);
-        return bf ? launch_fold<16, TC_BF16, true, false>(a, st) : launch_fold<16, TC_FP8, true, false>(a, st);
+        if (wide) return bf ? launch_fold<64, TC_BF16, true, false, false>(a, st) : launch_fold<64, TC_FP8, true, false, false>(a, st);
+        return bf ? launch_fold<16, TC_BF16, true, false, false>(a, st) : launch_fold<16, TC_FP8, true, false, false>(a, st);
     }
-    if (wide) return bf ? launch_fold<64, TC_BF16, false, false>(a, st) : launch_fold<64, TC_FP8, false, false>(a, st);
-    return bf ? launch_fold<16, TC_BF16, false, false>(a, st) : launch_fold<16, TC_FP8, false, false>(a, st);
+    // alternating epilogue groups from 3 rows a CTA.  The fusion network in BF16
+    // at 1024^2 (54 rows) 1.212 -> 1.183 ms, 512 x 288 (7.6) 0.265 -> 0.262, in
+    // FP8 512 x 288 0.246 -> 0.240, 384 x 216 (4.3) 0.195 -> 0.193, 256 x 128 (1.7)
+    // 0.147 -> 0.151; the two-encoder network at 256^2 (3.4) 1.576 -> 1.568
+    const long long tiles = (long long)a.N * ((a.W + kFoldTile - 1) / kFoldTile) * a.H;
+    if (tiles >= 3LL * sm_count()) {
+        if (wide)
+            return bf ? launch_fold<64, TC_BF16, false, false, true>(a, st) : launch_fold<64, TC_FP8, false, false, true>(a, st);
+        return bf ? launch_fold<16, TC_BF16, false, false, true>(a, st) : launch_fold<16, TC_FP8, false, false, true>(a, st);
+    }
+    if (wide)
+        return bf ? launch_fold<64, TC_BF16, false, false, false>(a, st) : launch_fold<64, TC_FP8, false, false, false>(a, st);
+    return bf ? launch_fold<16, TC_BF16, false, false, false>(a, st) : launch_fold<16, TC_FP8, false, false, false>(a, st);
 }
 
 

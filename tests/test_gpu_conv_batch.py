@@ -44,3 +44,21 @@ def test_dgrad_of_a_batch_is_each_images(N, H, W, mode):
         one = mrs.conv3x3_dgrad(dy[n:n + 1].contiguous(), w, mode,
                                 None if mode == "linear" else aux[n:n + 1].contiguous(), "bf16")
         assert torch.equal(got[n:n + 1], one)
+
+
+@pytest.mark.parametrize("H", [1, 2, 455, 456, 457, 608, 1300])
+@pytest.mark.parametrize("precision,cin,cout", [("bf16", 64, 64), ("bf16", 130, 64), ("fp8", 64, 64), ("bf16", 9, 3)])
+def test_rows_do_not_depend_on_the_image_around_them(H, precision, cin, cout):
+    # images of one strip, from one row to many a CTA (the epilogue's two
+    # arrangements, odd and even counts): a row is that of the three-row image
+    # around it
+    rng = np.random.default_rng(H)
+    x = _images(5, 1, H, 70, cin)
+    x[:, :, 0, 0] = 7.0                                   # one FP8 scale for all
+    w = rng.normal(size=(cout, 3, 3, cin)).astype(np.float32)
+    b = rng.normal(size=cout).astype(np.float32)
+    got = mrs.conv3x3(x, w, b, precision=precision)
+    for y in sorted({0, 1 % H, H // 2, max(H - 2, 0), H - 1}):
+        lo, hi = max(y - 1, 0), min(y + 2, H)
+        one = mrs.conv3x3(x[:, lo:hi].contiguous(), w, b, precision=precision)
+        assert torch.equal(got[:, y], one[:, y - lo])
