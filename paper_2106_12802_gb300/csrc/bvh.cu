@@ -979,39 +979,49 @@ __device__ void hcluster_merge(const HClusterArgs& a, int L, int R, int p, HWarp
     const int target = root ? 1 : kHKeep;
     int m = 0;   // merges so far
     if (c > target) {
-        // all pairs (i, i + d), d = 1 .. 16, each evaluated once
+        // all pairs (i, i + d), d = 1 .. 16, each evaluated once, 8 at a time
         sc.D[lane][lane] = INFINITY;
-        for (int d = 1; d <= 16; ++d) {
-            const int j = (lane + d) & 31;
-            const float4 o0 = shfl4(b0, j);
-            const float o1x = __shfl_sync(0xffffffffu, b1.x, j), o1y = __shfl_sync(0xffffffffu, b1.y, j);
-            const float u = mine && ((alive >> j) & 1u)
-                                ? pair_area(b0, b1, o0, make_float4(o1x, o1y, 0.0f, 0.0f))
-                                : INFINITY;
-            sc.D[lane][j] = u;
-            sc.D[j][lane] = u;
+        sc.kb[2 * lane] = b0;
+        sc.kb[2 * lane + 1] = b1;
+        __syncwarp();
+#pragma unroll
+        for (int d0 = 1; d0 <= 16; d0 += 8) {
+            float u[8];
+#pragma unroll
+            for (int d = 0; d < 8; ++d) {
+                const int j = (lane + d0 + d) & 31;
+                u[d] = pair_area(b0, b1, sc.kb[2 * j], sc.kb[2 * j + 1]);
+            }
+#pragma unroll
+            for (int d = 0; d < 8; ++d) {
+                const int j = (lane + d0 + d) & 31;
+                const float x = mine && ((alive >> j) & 1u) ? u[d] : INFINITY;
+                sc.D[lane][j] = x;
+                sc.D[j][lane] = x;
+            }
         }
         __syncwarp();
     }
     for (int round = 0; c > target && round < 2 * kHKeep; ++round) {
         // nearest neighbour: smallest area, then pair hash, then position (the
         // hashes only where a row has a tie for its smallest area)
-        float best = INFINITY;
         int bj = -1;
-        bool tie = false;
-        if (mine) {
+        {
+            float v[32];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const float v = sc.D[lane][j];
-                tie = v == best ? true : (v < best ? false : tie);
-                bj = v < best ? j : bj;
-                best = fminf(best, v);
-            }
-        }
-        if (__any_sync(0xffffffffu, tie && best != INFINITY)) {
-            if (tie && best != INFINITY) {
-                for (int j = bj + 1; j < 32; ++j)
-                    if (sc.D[lane][j] == best && pair_key(lane, j) < pair_key(lane, bj)) bj = j;
+            for (int j = 0; j < 32; ++j) v[j] = sc.D[lane][j];
+            float m4[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+#pragma unroll
+            for (int j = 0; j < 32; ++j) m4[j & 3] = fminf(m4[j & 3], v[j]);
+            const float best = fminf(fminf(m4[0], m4[1]), fminf(m4[2], m4[3]));
+            unsigned at[4] = {0u, 0u, 0u, 0u};            // where the row has its smallest area
+#pragma unroll
+            for (int j = 0; j < 32; ++j) at[j & 3] |= v[j] == best ? 1u << j : 0u;
+            const unsigned eq = mine && best < INFINITY ? at[0] | at[1] | at[2] | at[3] : 0u;
+            bj = __ffs(eq) - 1;
+            for (unsigned e = eq & (eq - 1); e; e &= e - 1) {
+                const int j = __ffs(e) - 1;
+                if (pair_key(lane, j) < pair_key(lane, bj)) bj = j;
             }
         }
         const int back = __shfl_sync(0xffffffffu, bj, bj >= 0 ? bj : lane);
@@ -1043,13 +1053,29 @@ __device__ void hcluster_merge(const HClusterArgs& a, int L, int R, int p, HWarp
         }
         sc.kp[lane] = bj;
         __syncwarp();
-        for (unsigned mm = lm; mm; mm &= mm - 1) {
-            const int k = __ffs(mm) - 1;
-            const float u = mine && lane != k ? pair_area(sc.kb[2 * k], sc.kb[2 * k + 1], b0, b1)
-                                              : INFINITY;
-            sc.D[k][lane] = u;
-            sc.D[lane][k] = u;
-            sc.D[lane][sc.kp[k]] = INFINITY;
+        for (unsigned mm = lm; mm;) {
+            // four merges at a time (the last group's spare places repeat its first)
+            int k[4], kp[4];
+            float u[4];
+            k[0] = __ffs(mm) - 1;
+            mm &= mm - 1;
+#pragma unroll
+            for (int t = 1; t < 4; ++t) {
+                k[t] = mm ? __ffs(mm) - 1 : k[0];
+                mm &= mm - 1;
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                kp[t] = sc.kp[k[t]];
+                u[t] = pair_area(sc.kb[2 * k[t]], sc.kb[2 * k[t] + 1], b0, b1);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const float x = mine && lane != k[t] ? u[t] : INFINITY;
+                sc.D[k[t]][lane] = x;
+                sc.D[lane][k[t]] = x;
+                sc.D[lane][kp[t]] = INFINITY;
+            }
         }
         __syncwarp();
     }
