@@ -66,8 +66,12 @@ void prof_push(int k, cudaEvent_t a, cudaEvent_t b)
 namespace {
 
 constexpr int kBlock = 256;
-constexpr int kSortItems = 8;                 // keys per thread per sort tile
-constexpr int kTile = kBlock * kSortItems;    // 2048 keys per tile
+// keys per sort tile: 4 a thread up to kSmallSort keys, which would leave half of
+// the SMs without a tile of 8 (a radix tree's whole build for 153,600 keys 145 us
+// with 8, 136 with 4; 403,202: 229, 237; 977,202: 401, 543)
+constexpr int kSmallSort = 256 * 1024;
+constexpr int sort_items(int n) { return n <= kSmallSort ? 4 : 8; }
+constexpr int sort_tiles(int n) { return (n + kBlock * sort_items(n) - 1) / (kBlock * sort_items(n)); }
 
 __device__ __forceinline__ float centroid(const float* V, int i, int a)
 {
@@ -151,19 +155,27 @@ __global__ void k_morton(const float* __restrict__ V, int n, const float* __rest
 }
 
 // ---- stable LSD radix sort, 8-bit digits ---------------------------------
+// counts of each tile's digits: [digit][tile] for k_sort_scan, or [tile][digit]
+// (by_tile) where the scatter kernel adds them up itself.
+// A pass is bound by latency, and its scan, one block, was 7 of 18 us for 153,600
+// keys.  Up to kSumTiles tiles every scatter block reads all counts (a kilobyte a
+// tile, coalesced, from L2) and needs no scan kernel: the build 159 -> 145 us,
+// for 1,996,002 keys (975 tiles) 888 -> 789; the reads grow with the square.
+constexpr int kSumTiles = 1024;
+template <int kItems>
 __global__ void k_sort_hist(const uint32_t* __restrict__ keys, int n, int shift,
-                            uint32_t* __restrict__ counts, int ntiles)
+                            uint32_t* __restrict__ counts, int ntiles, bool by_tile)
 {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
-    int base = blockIdx.x * kTile;
-    for (int k = 0; k < kSortItems; ++k) {
+    int base = blockIdx.x * kBlock * kItems;
+    for (int k = 0; k < kItems; ++k) {
         int i = base + k * kBlock + threadIdx.x;
         if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1u);
     }
     __syncthreads();
-    counts[threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+    counts[by_tile ? blockIdx.x * 256 + threadIdx.x : threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
 // exclusive scan of counts[0..m) in place, one block of 1024 threads: warp w
@@ -216,16 +228,40 @@ __global__ void __launch_bounds__(1024) k_sort_scan(uint32_t* __restrict__ count
 
 // scatter: rank of each key among equal digits = tile offset + keys before it
 // in the tile (round-major, then warp, then lane order == index order)
+template <int kItems>
 __global__ void k_sort_scatter(const uint32_t* __restrict__ kin, const int* __restrict__ vin,
                                uint32_t* __restrict__ kout, int* __restrict__ vout, int n,
-                               int shift, const uint32_t* __restrict__ offs, int ntiles)
+                               int shift, const uint32_t* __restrict__ offs, int ntiles, bool by_tile)
 {
     __shared__ uint32_t run[256];
     __shared__ uint32_t wc[kBlock / 32][256];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    run[threadIdx.x] = offs[threadIdx.x * ntiles + blockIdx.x];
-    int base = blockIdx.x * kTile;
-    for (int k = 0; k < kSortItems; ++k) {
+    if (by_tile) {
+        // this thread's digit: its keys in the tiles before, and in all; then the
+        // smaller digits' keys by a scan over the block
+        __shared__ uint32_t wsum[kBlock / 32];
+        uint32_t before = 0, total = 0;
+#pragma unroll 8
+        for (int t = 0; t < ntiles; ++t) {
+            const uint32_t c = offs[t * 256 + threadIdx.x];
+            before += t < (int)blockIdx.x ? c : 0u;
+            total += c;
+        }
+        uint32_t x = total;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += t;
+        }
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) x += wsum[w];
+        run[threadIdx.x] = x - total + before;
+    } else {
+        run[threadIdx.x] = offs[threadIdx.x * ntiles + blockIdx.x];
+    }
+    int base = blockIdx.x * kBlock * kItems;
+    for (int k = 0; k < kItems; ++k) {
         for (int w = 0; w < kBlock / 32; ++w) wc[w][threadIdx.x] = 0;
         __syncthreads();
         int i = base + k * kBlock + threadIdx.x;
@@ -257,6 +293,21 @@ __global__ void k_sort_scatter(const uint32_t* __restrict__ kin, const int* __re
         }
         __syncthreads();
     }
+}
+
+// one pass over the digit at `shift`; counts: 256 words a tile (sort_tiles(n));
+// returns the kernels enqueued
+int sort_pass(const uint32_t* kin, const int* vin, uint32_t* kout, int* vout, int n, int shift, uint32_t* counts,
+              cudaStream_t st)
+{
+    const int ntiles = sort_tiles(n);
+    const bool by_tile = ntiles <= kSumTiles, small = sort_items(n) == 4;
+    if (small) k_sort_hist<4><<<ntiles, kBlock, 0, st>>>(kin, n, shift, counts, ntiles, by_tile);
+    else k_sort_hist<8><<<ntiles, kBlock, 0, st>>>(kin, n, shift, counts, ntiles, by_tile);
+    if (!by_tile) k_sort_scan<<<1, 1024, 0, st>>>(counts, 256 * ntiles);
+    if (small) k_sort_scatter<4><<<ntiles, kBlock, 0, st>>>(kin, vin, kout, vout, n, shift, counts, ntiles, by_tile);
+    else k_sort_scatter<8><<<ntiles, kBlock, 0, st>>>(kin, vin, kout, vout, n, shift, counts, ntiles, by_tile);
+    return by_tile ? 2 : 3;
 }
 
 // ---- Karras radix tree ------------------------------------------------------
@@ -1226,7 +1277,7 @@ mrs_status build_lbvh(mrs_scene_s* S, cudaStream_t st)
     S->tree_built = S->tree;     // without internal nodes either kind is the same tree
     if (n <= 0) return MRS_OK;
     int nparts = 2 * sm_count();
-    int ntiles = blocks_for(ns > 0 ? ns : 1, kTile);
+    int ntiles = sort_tiles(ns > 0 ? ns : 1);
     size_t need = sizeof(float) * 6 * nparts + sizeof(uint32_t) * 256 * (size_t)ntiles +
                   (sizeof(uint32_t) + sizeof(int)) * 2 * (size_t)(ns > 0 ? ns : 1) + 256;
     mrs_status s = S->sort_tmp.ensure(need);
@@ -1260,10 +1311,7 @@ mrs_status build_lbvh(mrs_scene_s* S, cudaStream_t st)
                 uint32_t* kout = (pass & 1) ? ka : kb;
                 int* vin = (pass & 1) ? vb : va;
                 int* vout = (pass & 1) ? va : vb;
-                k_sort_hist<<<ntiles, kBlock, 0, c>>>(kin, ns, shift, counts, ntiles);
-                k_sort_scan<<<1, 1024, 0, c>>>(counts, 256 * ntiles);
-                k_sort_scatter<<<ntiles, kBlock, 0, c>>>(kin, vin, kout, vout, ns, shift, counts, ntiles);
-                kernels += 3;
+                kernels += sort_pass(kin, vin, kout, vout, ns, shift, counts, c);
             }
             cudaMemcpyAsync(S->skeys, ka, sizeof(uint32_t) * ns, cudaMemcpyDeviceToDevice, c);
             cudaMemcpyAsync(S->order, va, sizeof(int) * ns, cudaMemcpyDeviceToDevice, c);
@@ -1467,7 +1515,8 @@ void free_scene(mrs_scene_s* S)
 //   centroid-bound partials | digit counts | keys a/b | values a/b | parent | visit
 constexpr int kStaticMaxTris = MRS_LBVH_STATIC_MAX_TRIS;
 constexpr int kStaticParts = 512;
-constexpr int kStaticTiles = (kStaticMaxTris + kTile - 1) / kTile;
+constexpr int kStaticTiles =      // the most that any n takes
+    std::max(sort_tiles(std::min(kStaticMaxTris, kSmallSort)), sort_tiles(kStaticMaxTris));
 constexpr size_t kStaticBytes = sizeof(float) * 6 * kStaticParts +
                                 sizeof(uint32_t) * 256 * kStaticTiles +
                                 sizeof(uint32_t) * 4 * (size_t)kStaticMaxTris +
@@ -1771,7 +1820,7 @@ extern "C" mrs_status mrs_scene_export_bvh(mrs_scene S, uint32_t* morton, int32_
     if (n == 0) return MRS_OK;
     // the LBVH over all n triangles, built by the same kernels
     const int nparts = 2 * sm_count();
-    const int ntiles = blocks_for(n, kTile);
+    const int ntiles = sort_tiles(n);
     size_t need = sizeof(float) * 6 * nparts + sizeof(uint32_t) * 256 * (size_t)ntiles +
                   sizeof(uint32_t) * 5 * (size_t)n + sizeof(int) * 7 * (size_t)n +
                   sizeof(float) * 6 * (2 * (size_t)n) + 1024;
@@ -1802,12 +1851,7 @@ extern "C" mrs_status mrs_scene_export_bvh(mrs_scene S, uint32_t* morton, int32_
         uint32_t* kout = (pass & 1) ? ka : kb;
         int* vin = (pass & 1) ? vb : va;
         int* vout = (pass & 1) ? va : vb;
-        k_sort_hist<<<ntiles, kBlock, 0, st>>>(kin, n, shift, counts, ntiles);
-        MRS_LAUNCHED(1);
-        k_sort_scan<<<1, 1024, 0, st>>>(counts, 256 * ntiles);
-        MRS_LAUNCHED(1);
-        k_sort_scatter<<<ntiles, kBlock, 0, st>>>(kin, vin, kout, vout, n, shift, counts, ntiles);
-        MRS_LAUNCHED(1);
+        MRS_LAUNCHED(sort_pass(kin, vin, kout, vout, n, shift, counts, st));
     }
     MRS_CHECK(cudaMemcpyAsync(ord, va, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice, st));
     if (n > 1) {
@@ -1863,7 +1907,6 @@ extern "C" mrs_status mrs_lbvh_build_static(const float* V, int32_t n, uint32_t*
     mrs_status s = static_scratch(&base);
     if (s != MRS_OK) return s;
     const int nparts = 2 * sm_count() < kStaticParts ? 2 * sm_count() : kStaticParts;
-    const int ntiles = blocks_for(n, kTile);
     unsigned char* p = base;
     float* part = (float*)p; p += sizeof(float) * 6 * kStaticParts;
     uint32_t* counts = (uint32_t*)p; p += sizeof(uint32_t) * 256 * kStaticTiles;
@@ -1885,12 +1928,7 @@ extern "C" mrs_status mrs_lbvh_build_static(const float* V, int32_t n, uint32_t*
         uint32_t* kout = (pass & 1) ? ka : kb;
         int* vin = (pass & 1) ? vb : va;
         int* vout = (pass & 1) ? va : vb;
-        k_sort_hist<<<ntiles, kBlock, 0, st>>>(kin, n, shift, counts, ntiles);
-        MRS_LAUNCHED(1);
-        k_sort_scan<<<1, 1024, 0, st>>>(counts, 256 * ntiles);
-        MRS_LAUNCHED(1);
-        k_sort_scatter<<<ntiles, kBlock, 0, st>>>(kin, vin, kout, vout, n, shift, counts, ntiles);
-        MRS_LAUNCHED(1);
+        MRS_LAUNCHED(sort_pass(kin, vin, kout, vout, n, shift, counts, st));
     }
     MRS_CHECK(cudaMemcpyAsync(order, va, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice, st));
     if (n > 1) {
