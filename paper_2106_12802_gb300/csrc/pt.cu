@@ -186,9 +186,9 @@ __device__ __forceinline__ bool in_leaf_box(const float* __restrict__ box, V3 o,
 }
 
 // closest hit (ties to the smaller triangle index) or any hit below tmax
-template <bool kAny, bool kCount = false>
-__device__ int traverse(const SceneView& S, V3 o, V3 d, float tmax, float& t_out,
-                        unsigned long long* nvisit = nullptr, unsigned long long* ntest = nullptr)
+template <bool kCount>
+__device__ __forceinline__ int traverse_as(const bool any, const SceneView& S, V3 o, V3 d, float tmax, float& t_out,
+                                           unsigned long long* nvisit = nullptr, unsigned long long* ntest = nullptr)
 {
     const int n = S.ns;
     int best = -1, best_prim = 0x7fffffff;
@@ -198,9 +198,9 @@ __device__ int traverse(const SceneView& S, V3 o, V3 d, float tmax, float& t_out
     for (int k = n; k < S.n; ++k) {
         int prim;
         if (kCount) ++*ntest;
-        float t = intersect(o, d, S.tris + 3 * k, kAny ? tmax : T_INF, prim);
+        float t = intersect(o, d, S.tris + 3 * k, any ? tmax : T_INF, prim);
         if (t > 0.0f) {
-            if (kAny) { t_out = t; return k; }
+            if (any) { t_out = t; return k; }
             if (t < bt || (t == bt && prim < best_prim)) { bt = t; best = k; best_prim = prim; }
         }
     }
@@ -211,9 +211,9 @@ __device__ int traverse(const SceneView& S, V3 o, V3 d, float tmax, float& t_out
     if (n == 1) {
         int prim;
         if (kCount) ++*ntest;
-        float t = intersect(o, d, S.tris, kAny ? tmax : T_INF, prim);
+        float t = intersect(o, d, S.tris, any ? tmax : T_INF, prim);
         if (t > 0.0f) {
-            if (kAny) { t_out = t; return 0; }
+            if (any) { t_out = t; return 0; }
             if (t < bt || (t == bt && prim < best_prim)) { bt = t; best = 0; best_prim = prim; }
         }
         if (best >= 0) t_out = bt;
@@ -245,10 +245,10 @@ __device__ int traverse(const SceneView& S, V3 o, V3 d, float tmax, float& t_out
         } else {
             int k = node - (n - 1), prim;
             if (kCount) ++*ntest;
-            float t = intersect(o, d, S.tris + 3 * k, kAny ? tmax : T_INF, prim);
-            if (t > 0.0f && (kAny || t < bt || (t == bt && prim < best_prim)) &&
-                in_leaf_box(S.leaf_box + 6 * (size_t)k, o, d, inv, kAny ? tmax : T_INF)) {
-                if (kAny) { t_out = t; return k; }
+            float t = intersect(o, d, S.tris + 3 * k, any ? tmax : T_INF, prim);
+            if (t > 0.0f && (any || t < bt || (t == bt && prim < best_prim)) &&
+                in_leaf_box(S.leaf_box + 6 * (size_t)k, o, d, inv, any ? tmax : T_INF)) {
+                if (any) { t_out = t; return k; }
                 bt = t;
                 best = k;
                 best_prim = prim;
@@ -259,6 +259,12 @@ __device__ int traverse(const SceneView& S, V3 o, V3 d, float tmax, float& t_out
     }
     if (best >= 0) t_out = bt;
     return best;
+}
+template <bool kAny, bool kCount = false>
+__device__ int traverse(const SceneView& S, V3 o, V3 d, float tmax, float& t_out,
+                        unsigned long long* nvisit = nullptr, unsigned long long* ntest = nullptr)
+{
+    return traverse_as<kCount>(kAny, S, o, d, tmax, t_out, nvisit, ntest);
 }
 
 // ---- materials --------------------------------------------------------------
@@ -763,7 +769,8 @@ __device__ __forceinline__ void shadow_body(const WaveParams& w, const Jobs& job
 // one), because lanes on different paths wait for one another at every
 // divergent step and a small wave is bound by that latency, not by issue slots
 // (48 x 48 @ 1 spp: 0.230 -> 0.128 ms on the Cornell box, 0.323 -> 0.159 ms on
-// the 200k-triangle scene; 160 x 120 @ 1: 0.274 -> 0.197, 0.337 -> 0.206).
+// the 200k-triangle scene; 160 x 120 @ 1: 0.274 -> 0.197, 0.337 -> 0.206; from
+// bounce 0 such waves now run in pairs of lanes, below).
 constexpr int kWorkSlot = 63;
 constexpr int64_t kTailSmall = 640 * 1024, kTailMedium = 2 * 1024 * 1024;   // see tail_plan
 template <bool kCount, class Jobs>
@@ -833,6 +840,90 @@ __device__ __forceinline__ void tail_body(const WaveParams& w, const Jobs& jobs,
     }
 }
 
+// The tail from bounce 0 of a small wave, in pairs of lanes: lane 2 i follows a
+// path, lane 2 i + 1 traces its shadow rays, while lane 2 i already traces the next
+// bounce's ray (which does not depend on them; the contribution is added before
+// that bounce is shaded, as in tail_body).  Such a wave is bound by its longest
+// path's chain of rays, which this cuts by up to half; it gives up half of a warp's
+// paths, so it pays up to kPairPaths paths for each warp of the grid (311 k in
+// all).  us, one lane a path -> pairs, Cornell box and 200k-triangle scene: 2.3 k
+// paths 134 -> 124, 121 -> 119; 38 k 229 -> 200, 258 -> 225; 130 k 327 -> 282, 443
+// -> 347; 307 k 480 -> 484, 502 -> 401; 420 k 558 -> 610, 537 -> 460.
+constexpr int kPairWidth = 16, kPairPaths = 64;
+template <class Jobs>
+__device__ __forceinline__ void tail_pair_body(const WaveParams& w, const Jobs& jobs, int max_depth)
+{
+    __shared__ uint32_t s_cnt[64], s_scnt[64];
+    for (int j = threadIdx.x; j < 64; j += blockDim.x) { s_cnt[j] = 0u; s_scnt[j] = 0u; }
+    __syncthreads();
+    const PathSoA& P = w.P;
+    const int count = (int)*(volatile uint32_t*)&w.cnt[0];
+    const int lane = threadIdx.x & 31, own = lane & ~1;
+    const bool helper = lane & 1;
+    const int warps = (int)(gridDim.x * (blockDim.x / 32));
+    const int width = min(kPairWidth, (count + warps - 1) / warps);
+    int p = -1, b = 0;
+    bool pending = false, ended = false;   // a shadow ray is to be traced; there is no next bounce
+    bool drained = false;                  // warp-uniform: the queue has been handed out
+    for (;;) {
+        const bool want = !helper && p < 0 && (lane >> 1) < width;
+        const unsigned m = __ballot_sync(0xffffffffu, want);
+        if (m && !drained) {
+            const int leader = __ffs(m) - 1;
+            uint32_t base = 0;
+            if (lane == leader) base = atomicAdd(&w.cnt[kWorkSlot], (uint32_t)__popc(m));
+            base = __shfl_sync(0xffffffffu, base, leader);
+            drained = base + (uint32_t)__popc(m) >= (uint32_t)count;
+            if (want) {
+                const uint32_t i = base + (uint32_t)__popc(m & ((1u << lane) - 1u));
+                if (i < (uint32_t)count) { p = (int)i; b = 0; pending = ended = false; }
+            }
+        }
+        // what this lane traces now: its path's next ray, or its neighbour's shadow ray
+        const int path = __shfl_sync(0xffffffffu, p, own);
+        const bool sh = __shfl_sync(0xffffffffu, (int)pending, own) != 0;
+        if (!__any_sync(0xffffffffu, path >= 0)) break;
+        __syncwarp();                      // the path lane's stores are seen by its helper
+        float t = -1.0f;
+        int k = -1;
+        if (path >= 0 && (helper ? sh : !ended)) {
+            V3 o = mk(P.ox[path], P.oy[path], P.oz[path]), d;
+            float tmax = T_INF;
+            if (helper) {
+                d = mk(P.sdx[path], P.sdy[path], P.sdz[path]);
+                tmax = P.stmax[path];
+            } else {
+                d = mk(P.dx[path], P.dy[path], P.dz[path]);
+            }
+            k = traverse_as<false>(helper, jobs(path).S, o, d, tmax, t);
+        }
+        __syncwarp();
+        const bool lit = __shfl_sync(0xffffffffu, k, own | 1) < 0;
+        if (helper || p < 0) continue;
+        if (pending && lit) {
+            P.Lx[p] = P.Lx[p] + P.scx[p];
+            P.Ly[p] = P.Ly[p] + P.scy[p];
+            P.Lz[p] = P.Lz[p] + P.scz[p];
+        }
+        pending = false;
+        if (ended) { p = -1; continue; }
+        const JobView& J = jobs(p);
+        P.hit_t[p] = t;
+        P.hit_id[p] = k;
+        bool cont = false;
+        shade_path<false>(w, J, shade_const(J), b, p, cont, pending);
+        if (pending) atomicAdd(&s_scnt[b], 1u);
+        if (cont) { atomicAdd(&s_cnt[b + 1], 1u); ++b; }
+        else if (pending) ended = true;
+        else p = -1;
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j <= max_depth + 1; j += blockDim.x) {
+        if (j > 0 && s_cnt[j]) atomicAdd(&w.cnt[j], s_cnt[j]);
+        if (j <= max_depth && s_scnt[j]) atomicAdd(&w.scnt[j], s_scnt[j]);
+    }
+}
+
 // The kernels: a one-job wave (a render) and a batched wave (a table of jobs)
 __global__ void __launch_bounds__(kThreads) k_raygen(const __grid_constant__ WaveParams w)
 {
@@ -879,6 +970,15 @@ template <bool kCount, int kBlocks>
 __global__ void __launch_bounds__(kThreads, kBlocks) k_tail(const __grid_constant__ WaveParams w, int b0)
 {
     tail_body<kCount>(w, OneJob{w.J}, b0, w.J.max_depth);
+}
+__global__ void __launch_bounds__(kThreads, 4) k_tail_pair(const __grid_constant__ WaveParams w)
+{
+    tail_pair_body(w, OneJob{w.J}, w.J.max_depth);
+}
+__global__ void __launch_bounds__(kThreads, 4)
+    k_tail_pair_b(const __grid_constant__ WaveParams w, const __grid_constant__ JobTable T, int max_depth)
+{
+    tail_pair_body(w, ManyJobs{T}, max_depth);
 }
 template <int kBlocks>
 __global__ void __launch_bounds__(kThreads, kBlocks)
@@ -1137,6 +1237,14 @@ void launch_trace(bool count, const WaveParams& w, int b, int g, cudaStream_t st
 }
 template <bool kCount, int kBlocks> void launch_tail(const WaveParams& w, int b0, cudaStream_t st)
 {
+    if (!kCount && kBlocks == 4 && b0 == 0) {
+        static const int gp = persistent_grid(k_tail_pair);
+        if (w.n_paths <= kPairPaths * gp * (kThreads / 32)) {
+            MRS_TIMED(PK_TAIL, st, (k_tail_pair<<<gp, kThreads, 0, st>>>(w)));
+            MRS_LAUNCHED(1);
+            return;
+        }
+    }
     static const int g = persistent_grid(k_tail<kCount, kBlocks>);
     MRS_TIMED(PK_TAIL, st, (k_tail<kCount, kBlocks><<<g, kThreads, 0, st>>>(w, b0)));
     MRS_LAUNCHED(1);
@@ -1144,6 +1252,14 @@ template <bool kCount, int kBlocks> void launch_tail(const WaveParams& w, int b0
 template <int kBlocks>
 void launch_tail_b(const WaveParams& w, const JobTable& T, int b0, int max_depth, cudaStream_t st)
 {
+    if (kBlocks == 4 && b0 == 0) {
+        static const int gp = persistent_grid(k_tail_pair_b);
+        if (w.n_paths <= kPairPaths * gp * (kThreads / 32)) {
+            MRS_TIMED(PK_TAIL, st, (k_tail_pair_b<<<gp, kThreads, 0, st>>>(w, T, max_depth)));
+            MRS_LAUNCHED(1);
+            return;
+        }
+    }
     static const int g = persistent_grid(k_tail_b<kBlocks>);
     MRS_TIMED(PK_TAIL, st, (k_tail_b<kBlocks><<<g, kThreads, 0, st>>>(w, T, b0, max_depth)));
     MRS_LAUNCHED(1);

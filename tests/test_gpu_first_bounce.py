@@ -33,6 +33,19 @@ def test_render_does_not_depend_on_where_the_tail_starts(scenes, spp, depth):
         assert all(torch.equal(out[0][k], o[k]) for k in out[0])
 
 
+@pytest.mark.parametrize("W,H,spp", [(1, 1, 1), (69, 71, 1), (278, 280, 1), (411, 379, 1), (556, 560, 1), (300, 277, 4)])
+def test_pairs_of_lanes(scenes, W, H, spp):
+    # a path a pair of lanes (tail from bounce 0): a warp part filled, filled, and
+    # refilled from the queue; past the rule's end (the last) a path a lane
+    for sc in scenes:
+        sc.set_tail(0)
+        a = mrs.render(sc, W, H, spp, 6, 3, 4)
+        sc.set_tail(40)
+        b = mrs.render(sc, W, H, spp, 6, 3, 4)
+        sc.set_tail(-1)
+        assert all(torch.equal(a[k], b[k]) for k in a)
+
+
 @pytest.mark.parametrize("spp", [6, 8])
 def test_layers_of_a_window(scenes, spp):
     res = []
