@@ -3,7 +3,8 @@
 // tree of Karras (HPG 2012) with a bottom-up box refit, or locally-ordered
 // clustering over the sorted leaves (in grid-wide rounds, or inside the radix
 // tree's subtrees in one launch); every tree is written in the same traversal
-// node layout (both child boxes + child ids in one 64-byte node).
+// node layout (both child boxes, as centres and half extents, + child ids in one
+// 64-byte node).
 //
 // Compiled with --fmad=false: the Morton quantisation must round exactly like
 // the oracle's ((v0 + v1) + v2) * (1/3), (c - lo) * (1024 / extent).

@@ -137,7 +137,7 @@ struct mrs_scene_s {
     int* parent = nullptr;       // [2n-1]
     int* visit = nullptr;        // [n-1]
     float* box = nullptr;        // [2n-1][6]
-    float4* nodes = nullptr;     // [n-1][4]: child boxes + child ids
+    float4* nodes = nullptr;     // [n-1][4]: child boxes (centres, half extents) + child ids
     float4* tris = nullptr;      // [n][3]: (v0, prim bits), (e1, 0), (e2, 0) in sorted order
     int2* tri_ml = nullptr;      // [n]: material, light in sorted order
     mrs::Buf sort_tmp;           // radix-sort scratch

@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // x0 + 32 q + lane) and channels [ch0, ch0 + 16 kBlk) of the finished
         // output row's slot, then zeroes them.  (FP8: the factors come from shared
         // memory and values are converted in pairs; loading a factor and converting
-        // value by value bound the row: the network at 512 x 288 0.255 -> 0.233 ms)
+        // value by value bound the row: the network at 512 x 288 0.255 -> 0.238 ms)
         const int q = warp & 3, grp = (warp - 2) >> 2;
         constexpr int kBlk = kAlt && NOUT >= 64 ? 2 : 1;       // 16-channel blocks of a warp
         const int ch0 = (kAlt ? grp >> 1 : grp) * 16 * kBlk;

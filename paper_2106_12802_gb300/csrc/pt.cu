@@ -1,10 +1,10 @@
 // Wavefront Monte Carlo path tracer: produces the LRHS / HRLS radiance and
 // the albedo / normal / depth render layers of the multi-resolution sampling
 // method (Sec. 1, Sec. 3.2-3.3).  Per wave of paths:
-//   raygen -> for each bounce: traverse (closest hit) -> shade (emission, NEE
-//   shadow-ray setup, BSDF sampling, roulette, warp-ballot compaction) ->
-//   traverse_shadow (any hit, adds the unoccluded NEE term) -> accumulate
-//   (per-pixel Kahan sums in sample order).
+//   camera rays (raygen, or the first traversal) -> for each bounce: traverse
+//   (closest hit) -> shade (emission, NEE shadow-ray setup, BSDF sampling,
+//   roulette, warp-ballot compaction) -> traverse_shadow (any hit, adds the
+//   unoccluded NEE term) -> accumulate (per-pixel Kahan sums in sample order).
 //
 // Compiled with --fmad=false and IEEE div/sqrt: every float operation is a
 // single correctly rounded binary32 operation in the order written, which is
@@ -138,7 +138,8 @@ __device__ __forceinline__ float intersect(V3 o, V3 d, const float4* tri, float 
 // (1 + 8 u) holds whenever the exact interval is not empty.  Replacing the
 // lo / hi form took 1024^2 @ 4 spp on the 200k-triangle scene from 3.47 to
 // 3.21 ms and 256^2 @ 64 spp from 3.30 to 3.07 ms (issue slots, not memory,
-// bound the traversal: 69% used, ALU pipe 49%).
+// bound the traversal: 69% used, ALU pipe 49%); with in_leaf_box on every hit,
+// which these slightly larger boxes need, the former 3.46 to 3.33.
 __device__ __forceinline__ bool slab(float cx, float cy, float cz, float hx, float hy, float hz,
                                      V3 o, V3 inv, float tmax, float& tn)
 {
