@@ -443,7 +443,11 @@ mrs_status mrs_net_get_params(mrs_net net, float* params);
  * albedo, normal device [N][H][W][3] with H = scale*h, W = scale*w;
  * out device [N][H][W][3].  scale in {1, 2, 4, 8}; precision one of
  * MRS_PREC_*.  Activation workspace lives in the net handle (grown on
- * demand).  Limits: N*H*W <= 2^27 pixels. */
+ * demand; make the first call of a size before any stream capture).  A call
+ * recorded in a CUDA graph: an FP32 replay uses the weights as they are when it
+ * runs; BF16 and FP8 replays use the packed weights, which the first direct
+ * call after a change of the weights packs again.
+ * Limits: N*H*W <= 2^27 pixels. */
 mrs_status mrs_fuse(mrs_net net, const float* lrhs, const float* hrls, const float* albedo,
                     const float* normal, int32_t N, int32_t H, int32_t W, int32_t scale,
                     int32_t precision, float* out, void* stream);
@@ -668,7 +672,7 @@ mrs_status mrs_rdn_free(mrs_rdn rdn);
  * reference precision) or MRS_PREC_BF16 (tensor cores: BF16 activations and
  * weights, FP32 accumulation, a conv over more than 64 input channels
  * accumulates its 64-channel chunks in FP32).  Workspace lives in the handle
- * (grown on demand).  Limit: N*H*W <= 2^26. */
+ * (grown on demand).  Recorded calls: as mrs_fuse.  Limit: N*H*W <= 2^26. */
 mrs_status mrs_rdn_fuse(mrs_rdn rdn, const float* lrhs, const float* hrls, const float* albedo,
                         const float* normal, const float* extra, int32_t N, int32_t H, int32_t W,
                         int32_t precision, float* out, void* stream);

@@ -211,8 +211,8 @@ __device__ __forceinline__ void f2_get(f2_t a, float& x, float& y)
 // packed weights wp[c][t][o] (c < ceil4(cin), o < cop, zero beyond cin / cout) of
 // w [cout][9][cin], or, transposed, of the gradient conv's flipped taps: its
 // inputs are w's outputs, wp[o][t][c] = w[o][8 - t][c]
-__global__ void k_pack_simt(const float* __restrict__ w, int cin, int cout, int transposed, int cop,
-                            float* __restrict__ wp)
+__device__ __forceinline__ void pack_simt_body(const float* __restrict__ w, int cin, int cout, int transposed, int cop,
+                                               float* __restrict__ wp)
 {
     const int ci = transposed ? cout : cin, co = transposed ? cin : cout;
     const int n = ((ci + 3) & ~3) * 9 * cop;
@@ -223,6 +223,17 @@ __global__ void k_pack_simt(const float* __restrict__ w, int cin, int cout, int 
             v = transposed ? w[((size_t)c * 9 + (8 - t)) * cin + o] : w[((size_t)o * 9 + t) * cin + c];
         wp[i] = v;
     }
+}
+__global__ void k_pack_simt(const float* __restrict__ w, int cin, int cout, int transposed, int cop,
+                            float* __restrict__ wp)
+{
+    pack_simt_body(w, cin, cout, transposed, cop, wp);
+}
+// a network's layers, one to a blockIdx.y
+__global__ void k_pack_simt_layers(const __grid_constant__ SimtLayers p)
+{
+    const SimtLayers::Layer& l = p.layer[blockIdx.y];
+    pack_simt_body(l.w, l.cin, l.cout, 0, l.cop, l.wp);
 }
 
 // x [P][xs] (first cin channels read), out / res [P][os] / [P][rs] (first
@@ -408,6 +419,21 @@ mrs_status simt_pack(const float* w, int cin, int cout, int transposed, float* w
     const int cop = simt_cop(transposed ? cin : cout);
     const size_t n = transposed ? simt_pack_floats(cout, cin) : simt_pack_floats(cin, cout);
     k_pack_simt<<<(int)std::min<size_t>((n + 255) / 256, 2048), 256, 0, st>>>(w, cin, cout, transposed, cop, wp);
+    MRS_LAUNCHED(1);
+    return cuda_status(cudaGetLastError(), "simt pack");
+}
+
+bool SimtLayers::add(const float* w, int cin, int cout, float* wp)
+{
+    if (n == kMax) { set_error("simt_pack_layers: too many layers"); return false; }
+    layer[n++] = Layer{w, wp, cin, cout, simt_cop(cout)};
+    largest = std::max(largest, simt_pack_floats(cin, cout));
+    return true;
+}
+
+mrs_status simt_pack_layers(const SimtLayers& p, cudaStream_t st)
+{
+    k_pack_simt_layers<<<dim3((int)std::min<size_t>((p.largest + 255) / 256, 1024), p.n), 256, 0, st>>>(p);
     MRS_LAUNCHED(1);
     return cuda_status(cudaGetLastError(), "simt pack");
 }
@@ -1169,7 +1195,10 @@ struct mrs_net_s {
     __nv_bfloat16* wbfT = nullptr; // [18][9][64][64] transposed, tap-flipped (backward)
     bool bfT_valid = false;
     float* wsimt = nullptr;        // FP32 weights as the SIMT conv reads them, layer after layer
-    bool simt_valid = false;
+    // wsimt holds master's values.  A call that is being recorded packs whatever
+    // this says, so that its replays follow the weights; once a training step was
+    // recorded, whose replays change them unseen, every call packs
+    bool simt_valid = false, step_recorded = false;
     Buf act;                       // activation workspace
     Buf aux;                       // small device scratch
     Buf tact;                      // training activations
@@ -1220,12 +1249,14 @@ size_t simt_off(mrs_net_s* net, int l) { return l ? simt_pack_floats(net->cin0, 
 const float* wsimt(mrs_net_s* net, int l) { return net->wsimt + simt_off(net, l); }
 mrs_status pack_simt(mrs_net_s* net, cudaStream_t st)
 {
-    if (net->simt_valid) return MRS_OK;
+    const bool rec = recording(st);
+    if (net->simt_valid && !rec) return MRS_OK;
     const auto& L = shapes(net->cin0);
-    mrs_status rc = MRS_OK;
-    for (int l = 0; l < kLayers && rc == MRS_OK; ++l)
-        rc = simt_pack(net->master + L[l].woff, L[l].cin, L[l].cout, 0, net->wsimt + simt_off(net, l), st);
-    net->simt_valid = rc == MRS_OK && !recording(st);
+    SimtLayers p;
+    for (int l = 0; l < kLayers; ++l)
+        if (!p.add(net->master + L[l].woff, L[l].cin, L[l].cout, net->wsimt + simt_off(net, l))) return MRS_ERR_ARG;
+    const mrs_status rc = simt_pack_layers(p, st);
+    if (!rec) net->simt_valid = rc == MRS_OK && !net->step_recorded;
     return rc;
 }
 
@@ -1813,6 +1844,7 @@ mrs_status train_step_f32(mrs_net_s* net, const float* lrhs, const float* hrls, 
                                                         net->np, lr, (float)b1, (float)b2, 1e-8f, bc1, bc2));
     MRS_LAUNCHED(1);
     net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = net->simt_valid = false;
+    if (recording(st)) net->step_recorded = true;
     if (loss_out) {
         double h = 0;
         MRS_CHECK(cudaMemcpyAsync(&h, lres, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1998,6 +2030,7 @@ mrs_status train_step_bf16(mrs_net_s* net, const float* lrhs, const float* hrls,
                                                         net->np, lr, (float)b1, (float)b2, 1e-8f, bc1, bc2));
     MRS_LAUNCHED(1);
     net->bf_valid = net->f8_valid = net->xscale_valid = net->bfT_valid = net->simt_valid = false;
+    if (recording(st)) net->step_recorded = true;
     if (loss_out) {
         double h = 0;
         MRS_CHECK(cudaMemcpyAsync(&h, lres, sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -33,6 +33,16 @@ size_t simt_pack_floats(int cin, int cout);
 // w [cout][9][cin]; transposed: for the gradient with respect to the input
 // (inputs cout, outputs cin, taps flipped; simt_pack_floats(cout, cin) floats)
 mrs_status simt_pack(const float* w, int cin, int cout, int transposed, float* wp, cudaStream_t st);
+// a network's layers in one launch (each w [cout][9][cin] into its wp): a
+// recorded call holds it, and replays it with the call
+struct SimtLayers {
+    static constexpr int kMax = 72;
+    struct Layer { const float* w; float* wp; int cin, cout, cop; } layer[kMax];
+    int n = 0;
+    size_t largest = 0;            // floats of the largest wp
+    bool add(const float* w, int cin, int cout, float* wp);
+};
+mrs_status simt_pack_layers(const SimtLayers& p, cudaStream_t st);
 mrs_status simt_conv3x3(const float* x, int cin, int xs, const float* wp, const float* b, int cout,
                         int mode, int relu, const float* res, int rs, float* out, int os,
                         const float* lrhs, int N, int H, int W, int s, cudaStream_t st);

@@ -488,7 +488,8 @@ struct mrs_rdn_s {
     Buf f32, bf;                   // activation workspaces
     Buf simt;                      // FP32 weights as the SIMT conv reads them
     std::vector<size_t> simt_off;  // ... of each layer (floats)
-    bool simt_valid = false;
+    // simt holds master's values; recorded calls and steps as for the fusion network
+    bool simt_valid = false, step_recorded = false;
     int* err = nullptr;
     // training state (allocated by the first training step)
     float* grad = nullptr;         // gradient of the last step (parameter layout)
@@ -588,7 +589,8 @@ mrs_status pack_chunks(mrs_rdn_s* r, const float* P)
 // every layer's packed FP32 weights (the 1x1 fuse conv as a centre tap)
 mrs_status pack_simt(mrs_rdn_s* r, cudaStream_t st)
 {
-    if (r->simt_valid) return MRS_OK;
+    const bool rec = recording(st);
+    if (r->simt_valid && !rec) return MRS_OK;
     size_t n = 0;
     r->simt_off.clear();
     for (const RLayer& l : r->L) {
@@ -599,11 +601,14 @@ mrs_status pack_simt(mrs_rdn_s* r, cudaStream_t st)
     if (rc != MRS_OK) return rc;
     k_centre_tap<<<grid_for((size_t)64 * 9 * r->L[2].cin), 256, 0, st>>>(r->master + r->L[2].woff, r->L[2].cin, r->w_fuse3);
     MRS_LAUNCHED(1);
-    for (size_t li = 0; li < r->L.size() && rc == MRS_OK; ++li) {
+    SimtLayers p;
+    for (size_t li = 0; li < r->L.size(); ++li) {
         const RLayer& l = r->L[li];
-        rc = simt_pack(li == 2 ? r->w_fuse3 : r->master + l.woff, l.cin, l.cout, 0, r->simt.as<float>() + r->simt_off[li], st);
+        if (!p.add(li == 2 ? r->w_fuse3 : r->master + l.woff, l.cin, l.cout, r->simt.as<float>() + r->simt_off[li]))
+            return MRS_ERR_ARG;
     }
-    r->simt_valid = rc == MRS_OK && !recording(st);
+    rc = simt_pack_layers(p, st);
+    if (!rec) r->simt_valid = rc == MRS_OK && !r->step_recorded;
     return rc;
 }
 
@@ -1107,6 +1112,7 @@ mrs_status rdn_train_f32(mrs_rdn_s* r, const float* lrhs, const float* hrls, con
         return rc;
     r->bf_stale = true;
     r->simt_valid = false;
+    if (recording(st)) r->step_recorded = true;
     if (loss_out) {
         double hsum = 0;
         MRS_CHECK(cudaMemcpyAsync(&hsum, lsum, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1626,6 +1632,7 @@ mrs_status rdn_train_bf16(mrs_rdn_s* r, const float* lrhs, const float* hrls, co
     if ((rc = adam_f32(r->master, r->grad, r->adam_m, r->adam_v, r->np, lr, r->step, st)) != MRS_OK) return rc;
     r->bf_stale = true;
     r->simt_valid = false;
+    if (recording(st)) r->step_recorded = true;
     if (loss_out) {
         double hsum = 0;
         int herr = 0;
