@@ -1361,6 +1361,12 @@ mrs_status tc_wgrad_plan(const std::vector<WgTile>& tiles, int classes, WgPlan& 
     return MRS_OK;
 }
 
+// a unit a (tile, class) pair, or its two halves; a first unit for each CTA and the end
+size_t tc_wgrad_blob_max(int ntiles, int classes)
+{
+    return ntiles * (sizeof(WgDesc) + 2 * (size_t)classes * sizeof(WgUnit)) + ((size_t)sm_count() + 1) * sizeof(int);
+}
+
 mrs_status tc_conv3x3_wgrad(const WgPlan& plan, const void* d_blob, float* part, float* dbpart, int* err,
                             cudaStream_t st)
 {

@@ -145,6 +145,8 @@ struct WgPlan {
     size_t dbpart_floats() const { return (size_t)ntiles * classes * 64; }
 };
 mrs_status tc_wgrad_plan(const std::vector<WgTile>& tiles, int classes, WgPlan& plan);
+// bytes of a plan's blob at most
+size_t tc_wgrad_blob_max(int ntiles, int classes);
 mrs_status tc_conv3x3_wgrad(const WgPlan& plan, const void* d_blob, float* part, float* dbpart,
                             int* err, cudaStream_t st);
 // Operand maps of a tile: [N][H][W][64] bf16 with the given strides (bytes)

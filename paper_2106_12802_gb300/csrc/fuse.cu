@@ -1160,14 +1160,22 @@ Scratch& scratch()
 namespace mrs {
 // What a BF16 training step of one shape needs besides its data: the tensor
 // maps of its activations (all inside the handle's workspace) and the
-// weight-gradient tiles.  Made again when the shape or the workspace changes.
+// weight-gradient tiles.  A handle keeps those of its last kStepPlans shapes
+// (batches of two shapes in turn then build, allocate and upload nothing), and
+// those that a recorded step reads, which are neither changed nor freed before
+// the handle is.
+constexpr int kStepPlans = 8;
 struct StepPlan {
     int N = -1, H = -1, W = -1;
     void* act = nullptr;
     CUtensorMap x0A, dybA, hA[9], hO[9], rA[8], rO[8], dhA[9], dhO[9], daA[8], daO[8];
     WgPlan wg;
-    Buf blob;                      // wg.blob, then the tiles' WgRed, on the device
+    std::vector<uint8_t> image;    // wg.blob, then the tiles' WgRed
+    Buf blob;                      // ... on the device
     const WgRed* reds = nullptr;
+    bool uploaded = false;         // by a step that ran (a recorded step's upload is recorded with it)
+    bool recorded = false;
+    uint64_t used = 0;             // the handle's plan_clock at its last step
     ~StepPlan() { blob.release(); }
 };
 }  // namespace mrs
@@ -1204,7 +1212,8 @@ struct mrs_net_s {
     Buf tact;                      // training activations
     Buf ttmp;                      // training scratch (transposed weights, dW partials, loss)
     int* err = nullptr;            // device error word
-    std::unique_ptr<mrs::StepPlan> plan;   // tensor maps and wgrad tiles of the last BF16 step's shape
+    std::vector<std::unique_ptr<mrs::StepPlan>> plans;   // of BF16 steps
+    uint64_t plan_clock = 0;
     int loss_kind = MRS_LOSS_L1LOG;
     float loss_beta = 0.1f;
 };
@@ -1868,13 +1877,32 @@ mrs_status pack_bf16_T(mrs_net_s* net, cudaStream_t st)
     return cuda_status(cudaGetLastError(), "pack bf16 T");
 }
 
-// The plan of a step of this shape over the workspace tensors (see StepPlan)
+// The plan of a step of this shape over the workspace tensors, on the device as
+// of `st` (see StepPlan).  The upload is ordered on st, not on the legacy stream,
+// which a non-blocking stream does not wait for.
 mrs_status step_plan(mrs_net_s* net, int N, int H, int W, __nv_bfloat16* x0, __nv_bfloat16* hs, __nv_bfloat16* rs,
-                     __nv_bfloat16* dyb, __nv_bfloat16* dhs, __nv_bfloat16* das)
+                     __nv_bfloat16* dyb, __nv_bfloat16* dhs, __nv_bfloat16* das, cudaStream_t st, StepPlan*& plan)
 {
-    if (net->plan && net->plan->N == N && net->plan->H == H && net->plan->W == W && net->plan->act == x0)
+    const bool rec = recording(st);
+    auto use = [&](StepPlan& p) -> mrs_status {
+        if (!p.uploaded) {
+            MRS_CHECK(cudaMemcpyAsync(p.blob.p, p.image.data(), p.image.size(), cudaMemcpyHostToDevice, st));
+            p.uploaded = !rec;
+        }
+        p.recorded = p.recorded || rec;
+        p.used = ++net->plan_clock;
+        plan = &p;
         return MRS_OK;
-    net->plan.reset();
+    };
+    // the shape's plan, and the place of the longest unused one that may go
+    size_t direct = 0, oldest = net->plans.size();
+    for (size_t i = 0; i < net->plans.size(); ++i) {
+        StepPlan& p = *net->plans[i];
+        if (p.N == N && p.H == H && p.W == W && p.act == x0) return use(p);
+        if (p.recorded) continue;
+        ++direct;
+        if (oldest == net->plans.size() || p.used < net->plans[oldest]->used) oldest = i;
+    }
     std::unique_ptr<StepPlan> pl(new StepPlan());
     const size_t F = (size_t)N * H * W * 64;
     const auto& L = shapes(net->cin0);
@@ -1919,14 +1947,25 @@ mrs_status step_plan(mrs_net_s* net, int N, int H, int W, __nv_bfloat16* x0, __n
     if (rc == MRS_OK) rc = tc_wgrad_plan(tiles, 8, pl->wg);
     if (rc != MRS_OK) return rc;
     for (size_t t = 0; t < reds.size(); ++t) reds[t].np = pl->wg.np[t];
-    const size_t off = (pl->wg.blob.size() + 15) & ~(size_t)15;
-    if ((rc = pl->blob.ensure(off + reds.size() * sizeof(WgRed))) != MRS_OK) return rc;
-    MRS_CHECK(cudaMemcpy(pl->blob.p, pl->wg.blob.data(), pl->wg.blob.size(), cudaMemcpyHostToDevice));
-    MRS_CHECK(cudaMemcpy((uint8_t*)pl->blob.p + off, reds.data(), reds.size() * sizeof(WgRed), cudaMemcpyHostToDevice));
+    const size_t off = (pl->wg.blob.size() + 15) & ~(size_t)15, red_bytes = reds.size() * sizeof(WgRed);
+    pl->image.resize(off + red_bytes);
+    memcpy(pl->image.data(), pl->wg.blob.data(), pl->wg.blob.size());
+    memcpy(pl->image.data() + off, reds.data(), red_bytes);
+    if (direct >= kStepPlans) {
+        // the device memory of the plan that goes (in stream order: steps of a
+        // handle share its workspace)
+        std::swap(pl->blob, net->plans[oldest]->blob);
+        net->plans.erase(net->plans.begin() + oldest);
+    }
+    {
+        RelaxedCapture relaxed;    // a step of a new shape may be recorded
+        rc = pl->blob.ensure(tc_wgrad_blob_max((int)tiles.size(), 8) + 16 + red_bytes);
+    }
+    if (rc != MRS_OK) return rc;
     pl->reds = (const WgRed*)((uint8_t*)pl->blob.p + off);
     pl->N = N; pl->H = H; pl->W = W; pl->act = x0;
-    net->plan = std::move(pl);
-    return MRS_OK;
+    net->plans.push_back(std::move(pl));
+    return use(*net->plans.back());
 }
 
 // BF16 training step: forward and transposed convolutions on the tensor-core
@@ -1952,8 +1991,9 @@ mrs_status train_step_bf16(mrs_net_s* net, const float* lrhs, const float* hrls,
     float* dy = y + P * 3;
     float* lrc = dy + P * 3;
     float* hrc = lrc + nlr;
-    if ((rc = step_plan(net, N, H, W, x0, hs, rs, dyb, dhs, das)) != MRS_OK) return rc;
-    StepPlan& pl = *net->plan;
+    StepPlan* plan = nullptr;
+    if ((rc = step_plan(net, N, H, W, x0, hs, rs, dyb, dhs, das, st, plan)) != MRS_OK) return rc;
+    const StepPlan& pl = *plan;
     size_t tneed = 64 * 4 + (pl.wg.part_floats() + pl.wg.dbpart_floats()) * 4 + (kRedBlocks + 8) * 8;
     if ((rc = net->ttmp.ensure(tneed)) != MRS_OK) return rc;
     if ((rc = pack_bf16(net, st)) != MRS_OK) return rc;

@@ -24,6 +24,13 @@ inline bool recording(cudaStream_t st)
     return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
 }
 
+// device memory may be allocated while a stream of this thread is being recorded
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // FP32 3x3 convolution with zero padding 1 on [N][H][W][.] tensors:
 // out[p][o] (o < cout, pixel stride os) from x[p][c] (c < cin, pixel stride
 // xs) with the weights that simt_pack packed (16-byte aligned,
