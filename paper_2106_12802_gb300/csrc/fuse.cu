@@ -254,10 +254,12 @@ __global__ void __launch_bounds__(128, 4)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gx = lane & 3, ty = ((lane & 15) >> 2) + (OG == 8 ? 0 : 4 * warp);
     const int og = (lane >> 4) + (OG == 8 ? 2 * warp : 0);
-    const int x0 = blockIdx.x * kSX, y0 = blockIdx.y * kRows;
+    // blocks along x, then y, in grid.x: grid.y would end at 65,535 rows of blocks
+    const unsigned nbx = (unsigned)(W + kSX - 1) / kSX;
+    const int x0 = (int)(blockIdx.x % nbx) * kSX, y0 = (int)(blockIdx.x / nbx) * kRows;
     const int ngrp = (cout + 8 * OG - 1) / (8 * OG);
-    const int n = blockIdx.z / ngrp;
-    const int o0 = (blockIdx.z % ngrp) * 8 * OG;
+    const int n = blockIdx.y / ngrp;
+    const int o0 = (blockIdx.y % ngrp) * 8 * OG;
     const float* xin = x + (size_t)n * H * W * xs;
     float4 xr[kNX];
     // input channels c0 .. c0 + 3 of this thread's pixels of the tile
@@ -444,7 +446,7 @@ mrs_status simt_conv3x3(const float* x, int cin, int xs, const float* wp, const 
 {
     const bool vec = (cin & 3) == 0 && (xs & 3) == 0 && ((uintptr_t)x & 15) == 0;
     const int cop = simt_cop(cout), og = cout > 16 ? 8 : 2, rows = 32 / og;
-    const dim3 grid((W + kSX - 1) / kSX, (H + rows - 1) / rows, N * ((cout + 8 * og - 1) / (8 * og)));
+    const dim3 grid((unsigned)((W + kSX - 1) / kSX) * (unsigned)((H + rows - 1) / rows), N * ((cout + 8 * og - 1) / (8 * og)));
     auto launch = [&](auto kernel) {
         kernel<<<grid, 128, 0, st>>>(x, cin, xs, wp, cop, b, cout, mode, relu, res, rs, out, os, lrhs, H, W, s);
     };
