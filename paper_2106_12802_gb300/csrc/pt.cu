@@ -150,19 +150,28 @@ __device__ __forceinline__ bool slab(float cx, float cy, float cz, float hx, flo
     return tn <= tf * 1.0000005f;
 }
 
-// 1 / d where some component of d is zero: its slab is 0 outside and
-// everything inside, so any large reciprocal serves that keeps every
-// (c - o) inv in the tree finite (an infinite one would make inf - inf, and
-// the axis would no longer cull): 1e36 over the farthest point of the root's boxes
-__device__ __noinline__ V3 reciprocal_zero(const float4* __restrict__ nodes, V3 o, V3 d, V3 inv)
+// A direction's components at least this large have reciprocals (at most 1e18)
+// with which the slab test of any box stays finite, for coordinates up to 1e20
+constexpr float kTinyDir = 1e-18f;
+__device__ __forceinline__ bool has_tiny(V3 d) { return fminf(fminf(fabsf(d.x), fabsf(d.y)), fabsf(d.z)) < kTinyDir; }
+__device__ __noinline__ V3 reciprocal(V3 d) { return mk(1.0f / d.x, 1.0f / d.y, 1.0f / d.z); }
+
+// inv = 1 / d for the slab test where some component of d is zero or so small that
+// (c - o) inv could be infinite in the tree: a centre's infinite distance less or
+// plus a finite half chord is infinite on both sides, and a box around the origin
+// would be culled.  Such a component's slab is next to 0 outside and everything
+// inside, so any large reciprocal serves that keeps (c - o) inv and h inv finite:
+// 1e38 over the farthest point of the root's boxes, which puts the far side of a
+// box beyond T_INF unless it is closer to o than 1e-8 of that
+__device__ __noinline__ V3 reciprocal_tiny(const float4* __restrict__ nodes, V3 o, V3 d, V3 inv)
 {
     const float4 a = __ldg(nodes), b = __ldg(nodes + 1), c = __ldg(nodes + 2);
-    const float mx = fmaxf(fabsf(a.x - o.x) + b.z, fabsf(a.y - o.x) + b.w);
-    const float my = fmaxf(fabsf(a.z - o.y) + c.x, fabsf(a.w - o.y) + c.y);
-    const float mz = fmaxf(fabsf(b.x - o.z) + c.z, fabsf(b.y - o.z) + c.w);
-    if (d.x == 0.0f) inv.x = copysignf(1e36f / fmaxf(mx, 1.0f), d.x);
-    if (d.y == 0.0f) inv.y = copysignf(1e36f / fmaxf(my, 1.0f), d.y);
-    if (d.z == 0.0f) inv.z = copysignf(1e36f / fmaxf(mz, 1.0f), d.z);
+    const float mx = 1e38f / fmaxf(fmaxf(fabsf(a.x - o.x) + b.z, fabsf(a.y - o.x) + b.w), 1.0f);
+    const float my = 1e38f / fmaxf(fmaxf(fabsf(a.z - o.y) + c.x, fabsf(a.w - o.y) + c.y), 1.0f);
+    const float mz = 1e38f / fmaxf(fmaxf(fabsf(b.x - o.z) + c.z, fabsf(b.y - o.z) + c.w), 1.0f);
+    if (fabsf(inv.x) > mx) inv.x = copysignf(mx, d.x);
+    if (fabsf(inv.y) > my) inv.y = copysignf(my, d.y);
+    if (fabsf(inv.z) > mz) inv.z = copysignf(mz, d.z);
     return inv;
 }
 
@@ -170,14 +179,12 @@ __device__ __noinline__ V3 reciprocal_zero(const float4* __restrict__ nodes, V3 
 // put a grazing hit just outside the triangle's box; such a hit does not count,
 // whatever the tree above the leaf lets through (the boxes tested there are
 // slightly larger).  Only a triangle that was hit gets here, about once per ray.
-// inv: the traversal's reciprocals (infinite here where d is zero).
+// inv: the traversal's reciprocals (not 1 / d where d has a tiny component).
 __device__ __forceinline__ bool in_leaf_box(const float* __restrict__ box, V3 o, V3 d, V3 inv, float tmax)
 {
     const float2* p = (const float2*)box;
     const float2 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);   // lo.xy | lo.z hi.x | hi.yz
-    if (d.x == 0.0f) inv.x = copysignf(INFINITY, d.x);
-    if (d.y == 0.0f) inv.y = copysignf(INFINITY, d.y);
-    if (d.z == 0.0f) inv.z = copysignf(INFINITY, d.z);
+    if (has_tiny(d)) inv = reciprocal(d);
     const float t0x = (a.x - o.x) * inv.x, t1x = (b.y - o.x) * inv.x;
     const float t0y = (a.y - o.y) * inv.y, t1y = (c.x - o.y) * inv.y;
     const float t0z = (b.x - o.z) * inv.z, t1z = (c.y - o.z) * inv.z;
@@ -221,7 +228,7 @@ __device__ __forceinline__ int traverse_as(const bool any, const SceneView& S, V
         return best;
     }
     V3 inv = mk(1.0f / d.x, 1.0f / d.y, 1.0f / d.z);
-    if (d.x == 0.0f || d.y == 0.0f || d.z == 0.0f) inv = reciprocal_zero(S.nodes, o, d, inv);
+    if (has_tiny(d)) inv = reciprocal_tiny(S.nodes, o, d, inv);
     int stack[kStack];
     int sp = 0;
     int node = 0;
