@@ -407,9 +407,8 @@ __device__ __forceinline__ int add_acquire(int* p, int v)
 }
 
 // One axis of a box as the traversal reads it: centre and half extent.  h
-// covers both sides exactly (rounded up), times 1 + 8 u (u = 2^-24): the slab
-// test (pt.cu) forms (c - o) inv -+ h |inv|, whose rounding is at most
-// 3 u |t| + 2 u h |inv| per side, so its interval holds the box's
+// covers both sides exactly (rounded up), times 1 + 8 u (u = 2^-24), which makes up
+// for the part of the slab test's rounding that grows with h (pt.cu, slab)
 __device__ __forceinline__ void centre_half(float lo, float hi, float& c, float& h)
 {
     c = 0.5f * lo + 0.5f * hi;

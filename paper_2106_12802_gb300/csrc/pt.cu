@@ -134,12 +134,22 @@ __device__ __forceinline__ float intersect(V3 o, V3 d, const float4* tri, float 
 // write_node in bvh.cu): per axis (c - o) inv is the box centre's distance and
 // h |inv| half its chord, so entry and exit are two FMAs, and only the maxima
 // and minima over the axes are left for the half-rate ALU pipe (5 min / max and
-// compare operations per box; the lo / hi form needs 6 more).  tn <= tf
-// (1 + 8 u) holds whenever the exact interval is not empty.  Replacing the
+// compare operations per box; the lo / hi form needs 6 more).  Replacing the
 // lo / hi form took 1024^2 @ 4 spp on the 200k-triangle scene from 3.47 to
 // 3.21 ms and 256^2 @ 64 spp from 3.30 to 3.07 ms (issue slots, not memory,
 // bound the traversal: 69% used, ALU pipe 49%); with in_leaf_box on every hit,
 // which these slightly larger boxes need, the former 3.46 to 3.33.
+// The factor: a box passes whenever a leaf box within it passes in_leaf_box
+// against the same tmax, whose rounding a grazing hit may rest on.  With the exact
+// interval [A, B] of the box and H its half chord (both with inv as rounded, which
+// either test uses; u = 2^-24, second orders left out), (c - o) inv is off by
+// 2 u (|A| + H) at most, the FMA by u |A|, and h is 8 u larger than H:
+//   tn <= A (1 + 3 u) - 6 u H,  tf >= B (1 - 3 u) + 6 u H.
+// The leaf's entry n and exit f, off by 2 u, lie in [A, B] and have
+// n <= f (1 + 8 u)(1 + u); hence tn <= tf (1 + 19 u), and one u for the product here.
+// 1 + 24 u it is.  (1 + 8 u culled 3 in a million hits near a side of a box
+// 150 and more times as far as it is wide.)
+constexpr float kSlabSlack = 1.0f + 12 * 0x1p-23f;
 __device__ __forceinline__ bool slab(float cx, float cy, float cz, float hx, float hy, float hz,
                                      V3 o, V3 inv, float tmax, float& tn)
 {
@@ -147,7 +157,7 @@ __device__ __forceinline__ bool slab(float cx, float cy, float cz, float hx, flo
     const float ix = fabsf(inv.x), iy = fabsf(inv.y), iz = fabsf(inv.z);
     tn = fmaxf(fmaxf(fmaxf(fmaf(-hx, ix, tx), fmaf(-hy, iy, ty)), fmaf(-hz, iz, tz)), 0.0f);
     const float tf = fminf(fminf(fminf(fmaf(hx, ix, tx), fmaf(hy, iy, ty)), fmaf(hz, iz, tz)), tmax);
-    return tn <= tf * 1.0000005f;
+    return tn <= tf * kSlabSlack;
 }
 
 // A direction's components at least this large have reciprocals (at most 1e18)
