@@ -1114,10 +1114,26 @@ __device__ __forceinline__ void wg_issue(uint32_t tmem, uint64_t a01, uint64_t a
     }
 }
 
+// kOne: a launch of one tile, described by its parameter instead of lists in device
+// memory; CTA c takes class c, or a half of class c / 2 (halves set: up to half as
+// many classes as SMs), and classes = runs.  Through the lists, which the host makes
+// and whose upload the kernel waits for, the call for a layer's gradient took 108 us
+// with 8 images of 30 x 30, so 84.
+struct WgNone {};
+template <bool kOne>
 __global__ void __launch_bounds__(kWgThreads, 1)
-    k_wgrad_tc(const WgDesc* __restrict__ tiles, const WgUnit* __restrict__ units, const int* __restrict__ first,
+    k_wgrad_tc(const __grid_constant__ std::conditional_t<kOne, WgDesc, WgNone> one, int halves,
+               const WgDesc* __restrict__ tiles, const WgUnit* __restrict__ units, const int* __restrict__ first,
                int classes, float* __restrict__ part, float* __restrict__ dbpart, int* err)
 {
+    auto unit = [&](int u) -> WgUnit {
+        if constexpr (kOne) return halves ? WgUnit{0, (int)blockIdx.x / 2, 1 + (int)blockIdx.x % 2} : WgUnit{0, (int)blockIdx.x, 0};
+        else return units[u];
+    };
+    auto desc = [&](const WgUnit& w) -> const WgDesc& {
+        if constexpr (kOne) return one;
+        else return tiles[w.tile];
+    };
     constexpr uint32_t kTmemCols = 512;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -1130,7 +1146,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     constexpr int kWgEpiWarps = 13;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int u0 = first[blockIdx.x], u1 = first[blockIdx.x + 1];
+    const int u0 = kOne ? 0 : first[blockIdx.x], u1 = kOne ? 1 : first[blockIdx.x + 1];
 
     for (int i = threadIdx.x; i < kWgOnes / 4; i += kWgThreads) ((uint32_t*)sOnes)[i] = 0x3F803F80u;  // bf16 1.0
     fence_async_smem();
@@ -1157,12 +1173,15 @@ __global__ void __launch_bounds__(kWgThreads, 1)
             int s = 0;
             bool ok = true;
             for (int u = u0; ok && u < u1; ++u) {
-                const WgDesc& d = tiles[units[u].tile];
-                // maps in global memory, written by the host before the launch
-                asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)&d.x) : "memory");
-                asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)&d.dy) : "memory");
+                const WgUnit un = unit(u);
+                const WgDesc& d = desc(un);
+                if constexpr (!kOne) {
+                    // maps in global memory, written by the host before the launch
+                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)&d.x) : "memory");
+                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)&d.dy) : "memory");
+                }
                 const int XS = d.XS, H = d.H;
-                for (int g = units[u].w; ok && g < d.runs; g += classes) {
+                for (int g = un.w; ok && g < d.runs; g += classes) {
                     const int je = wg_run(d, g + 1);
                     for (int j = wg_run(d, g); j < je;
                          ++j, ++it, s = (s + 1 == kWgStages ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
@@ -1187,10 +1206,11 @@ __global__ void __launch_bounds__(kWgThreads, 1)
             int s = 0;
             bool ok = true;
             for (int u = u0; ok && u < u1; ++u) {
-                const WgDesc& d = tiles[units[u].tile];
+                const WgUnit un = unit(u);
+                const WgDesc& d = desc(un);
                 const int XS = d.XS, W = d.W;
-                const int half = units[u].half;
-                for (int g = units[u].w; ok && g < d.runs; g += classes, ++k) {
+                const int half = un.half;
+                for (int g = un.w; ok && g < d.runs; g += classes, ++k) {
                     const int jb = wg_run(d, g), je = wg_run(d, g + 1);
                     // the previous run's accumulators have been read
                     if (k > 0 && !mbar_wait(tfree, (k - 1) & 1, err)) { ok = false; break; }
@@ -1223,8 +1243,9 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         uint32_t k = 0;
         bool ok = true;
         for (int u = u0; ok && u < u1; ++u) {
-            const WgDesc& d = tiles[units[u].tile];
-            const int w = units[u].w, half = units[u].half, runs = d.runs, cin = d.cin, cout = d.cout;
+            const WgUnit un = unit(u);
+            const WgDesc& d = desc(un);
+            const int w = un.w, half = un.half, runs = d.runs, cin = d.cin, cout = d.cout;
             const bool mine = half == 0 || (half == 1 ? col0 < 192 : col0 >= 192);
             float acc[96];
 #pragma unroll
@@ -1247,7 +1268,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
             }
             if (!ok) break;
             if (!mine) continue;
-            const size_t slot = (size_t)units[u].tile * classes + w;
+            const size_t slot = (size_t)un.tile * classes + w;
             float* P = part + slot * kWgPart;
             if (bias) {
                 if (lane == 0)
@@ -1289,6 +1310,22 @@ mrs_status tc_make_wg_dy_map(CUtensorMap* m, const void* ptr, int N, int H, int 
     return tc_make_view_map(m, ptr, N, H, W, px_stride, row_stride, img_stride, kWgKB);
 }
 
+static mrs_status wg_desc(const WgTile& w, WgDesc& e)
+{
+    if (w.cin < 1 || w.cin > 64 || w.cout < 1 || w.cout > 64 || w.runs < 1) {
+        set_error("tensor-core weight gradient: cin, cout must be in [1, 64], runs >= 1");
+        return MRS_ERR_ARG;
+    }
+    memset(&e, 0, sizeof(e));
+    e.x = w.x; e.dy = w.dy; e.H = w.H; e.W = w.W; e.cin = w.cin; e.cout = w.cout;
+    e.XS = (w.W + kWgKB - 1) / kWgKB;
+    const long long nj = (long long)w.N * w.H * e.XS;
+    if (nj > 0x7fffffff) { set_error("tensor-core weight gradient: too many jobs"); return MRS_ERR_CAPACITY; }
+    e.njobs = (int)nj;
+    e.runs = (int)std::min<long long>(nj, w.runs);
+    return MRS_OK;
+}
+
 mrs_status tc_wgrad_plan(const std::vector<WgTile>& tiles, int classes, WgPlan& plan)
 {
     const int nt = (int)tiles.size();
@@ -1301,18 +1338,10 @@ mrs_status tc_wgrad_plan(const std::vector<WgTile>& tiles, int classes, WgPlan& 
     plan.np.assign(nt, 0);
     for (int t = 0; t < nt; ++t) {
         const WgTile& w = tiles[t];
-        if (w.cin < 1 || w.cin > 64 || w.cout < 1 || w.cout > 64 || w.runs < 1) {
-            set_error("tc_wgrad_plan: cin, cout must be in [1, 64], runs >= 1");
-            return MRS_ERR_ARG;
-        }
         WgDesc& e = d[t];
-        memset(&e, 0, sizeof(e));
-        e.x = w.x; e.dy = w.dy; e.H = w.H; e.W = w.W; e.cin = w.cin; e.cout = w.cout;
-        e.XS = (w.W + kWgKB - 1) / kWgKB;
-        const long long nj = (long long)w.N * w.H * e.XS;
-        if (nj > 0x7fffffff) { set_error("tc_wgrad_plan: too many jobs"); return MRS_ERR_CAPACITY; }
-        e.njobs = (int)nj;
-        e.runs = (int)std::min<long long>(nj, w.runs);
+        const mrs_status rc = wg_desc(w, e);
+        if (rc != MRS_OK) return rc;
+        const long long nj = e.njobs;
         plan.np[t] = std::min(e.runs, classes);
         for (int c = 0; c < plan.np[t]; ++c) {
             long long cost = 0;
@@ -1367,22 +1396,40 @@ size_t tc_wgrad_blob_max(int ntiles, int classes)
     return ntiles * (sizeof(WgDesc) + 2 * (size_t)classes * sizeof(WgUnit)) + ((size_t)sm_count() + 1) * sizeof(int);
 }
 
+template <bool kOne>
+static mrs_status launch_wgrad(const std::conditional_t<kOne, WgDesc, WgNone>& one, int halves, int ctas, const WgDesc* d,
+                               const WgUnit* u, const int* first, int classes, float* part, float* dbpart, int* err,
+                               cudaStream_t st)
+{
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc<kOne>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
+        if (e != cudaSuccess) return cuda_status(e, "wgrad smem attribute");
+        attr = true;
+    }
+    MRS_TIMED(PK_WGRAD_TC, st, (k_wgrad_tc<kOne><<<ctas, kWgThreads, kWgSmem, st>>>(one, halves, d, u, first, classes, part, dbpart, err)));
+    MRS_LAUNCHED(1);
+    return cuda_status(cudaGetLastError(), "wgrad launch");
+}
+
 mrs_status tc_conv3x3_wgrad(const WgPlan& plan, const void* d_blob, float* part, float* dbpart, int* err,
                             cudaStream_t st)
 {
     if (plan.ctas < 1) return MRS_OK;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
-        if (e != cudaSuccess) return cuda_status(e, "wgrad smem attribute");
-        attr = true;
-    }
     const WgDesc* d = (const WgDesc*)d_blob;
     const WgUnit* u = (const WgUnit*)(d + plan.ntiles);
-    const int* first = (const int*)(u + plan.units);
-    MRS_TIMED(PK_WGRAD_TC, st, (k_wgrad_tc<<<plan.ctas, kWgThreads, kWgSmem, st>>>(d, u, first, plan.classes, part, dbpart, err)));
-    MRS_LAUNCHED(1);
-    return cuda_status(cudaGetLastError(), "wgrad launch");
+    return launch_wgrad<false>({}, 0, plan.ctas, d, u, (const int*)(u + plan.units), plan.classes, part, dbpart, err, st);
+}
+
+mrs_status tc_conv3x3_wgrad(const WgTile& tile, float* part, float* dbpart, int* np, int* err, cudaStream_t st)
+{
+    WgDesc d;
+    const mrs_status rc = wg_desc(tile, d);
+    if (rc != MRS_OK) return rc;
+    *np = d.runs;
+    if (d.runs < 1) return MRS_OK;
+    const int halves = 2 * d.runs <= sm_count();
+    return launch_wgrad<true>(d, halves, d.runs * (1 + halves), nullptr, nullptr, nullptr, d.runs, part, dbpart, err, st);
 }
 
 }  // namespace mrs

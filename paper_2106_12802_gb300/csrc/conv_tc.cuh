@@ -128,8 +128,8 @@ void tc_set_ring(int stages);
 // FP32 in that order and written as partial w of the tile's np = min(runs, C):
 //   part[(slot + w) * kWgPart + (tap * cout + o) * cin + c], dbpart[(slot + w) * 64 + o]
 // (slot: C times the tile's number).  The sums' order depends on the tiles alone.
-// C = 8 leaves few partials; a list of one tile takes C = runs, whose units of
-// work are enough for every SM.
+// C = 8 leaves few partials of a list; one tile alone takes C = runs, whose units
+// of work are enough for every SM.
 constexpr int kWgKB = 64;          // pixels per job
 constexpr int kWgPart = 9 * 64 * 64;
 struct WgTile {
@@ -149,6 +149,8 @@ mrs_status tc_wgrad_plan(const std::vector<WgTile>& tiles, int classes, WgPlan& 
 size_t tc_wgrad_blob_max(int ntiles, int classes);
 mrs_status tc_conv3x3_wgrad(const WgPlan& plan, const void* d_blob, float* part, float* dbpart,
                             int* err, cudaStream_t st);
+// One tile alone, without a plan: C = its runs, *np of them
+mrs_status tc_conv3x3_wgrad(const WgTile& tile, float* part, float* dbpart, int* np, int* err, cudaStream_t st);
 // Operand maps of a tile: [N][H][W][64] bf16 with the given strides (bytes)
 // between pixels, rows and images (as tc_make_view_map).
 mrs_status tc_make_wg_x_map(CUtensorMap* m, const void* ptr, int N, int H, int W, long long px_stride,

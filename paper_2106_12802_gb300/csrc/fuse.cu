@@ -2356,7 +2356,7 @@ extern "C" mrs_status mrs_conv3x3_wgrad(const float* x, const float* dy, int32_t
     const size_t maxp = (size_t)std::max(kDwSplits, sm_count());
     Scratch& S = scratch();
     std::lock_guard<std::mutex> g(S.mu);
-    size_t need = (nw + cout) * 4 + maxp * (9 * 64 * 64 + 64) * 4 + 8192 +
+    size_t need = (nw + cout) * 4 + maxp * (9 * 64 * 64 + 64) * 4 + 4096 +
                   (precision == MRS_PREC_BF16 ? 2 * P * 128 : 0);
     mrs_status rc = S.b.ensure(need);
     if (rc != MRS_OK) return rc;
@@ -2378,17 +2378,11 @@ extern "C" mrs_status mrs_conv3x3_wgrad(const float* x, const float* dy, int32_t
         MRS_LAUNCHED(1);
         k_to_operand<<<1024, 256, 0, st>>>(dy, P, cout, dq, 0, 1.0f);
         MRS_LAUNCHED(1);
-        std::vector<WgTile> tile(1);
-        WgTile& t = tile[0];
+        WgTile t;
         if ((rc = tc_make_wg_x_map(&t.x, xq, N, H, W, 128, 128LL * W, 128LL * W * H)) != MRS_OK) return rc;
         if ((rc = tc_make_wg_dy_map(&t.dy, dq, N, H, W, 128, 128LL * W, 128LL * W * H)) != MRS_OK) return rc;
         t.N = N; t.H = H; t.W = W; t.cin = cin; t.cout = cout; t.runs = sm_count();   // np partials at most
-        WgPlan plan;
-        if ((rc = tc_wgrad_plan(tile, t.runs, plan)) != MRS_OK) return rc;
-        void* blob = dq + P * 128;      // 1024-byte aligned or not, a multiple of 128
-        MRS_CHECK(cudaMemcpyAsync(blob, plan.blob.data(), plan.blob.size(), cudaMemcpyHostToDevice, st));
-        if ((rc = tc_conv3x3_wgrad(plan, blob, part, dbpart, err, st)) != MRS_OK) return rc;
-        np = plan.np[0];
+        if ((rc = tc_conv3x3_wgrad(t, part, dbpart, &np, err, st)) != MRS_OK) return rc;
     }
     const size_t gstride = precision == MRS_PREC_FP32 ? nw : (size_t)kWgPart;
     k_dw_reduce<<<(int)((nw + cout + 31) / 32), 256, 0, st>>>(part, dbpart, np, gstride,
