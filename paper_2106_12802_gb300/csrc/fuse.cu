@@ -177,8 +177,9 @@ __global__ void k_input_q(const float* lrhs, const float* hrls, const float* alb
 // was bound by shared-memory wavefronts (86%), a third of them bank conflicts:
 // the 21-channel network on 486 x 330 7.42 -> 3.80 ms (26 -> 51 TFLOP/s of the
 // 80.5 of 152 SMs x 128 lanes), the 35 convolutions of its training step at 6 x
-// 128^2 9.40 -> 5.13 ms.  Up to 16 outputs (the 3-channel heads) run as two
-// groups of 8 on four times the rows, so that the rest is not padding.
+// 128^2 9.40 -> 5.13 ms.  Up to 16 outputs (the 3-channel heads; up to 32 on large
+// images, see simt_conv3x3) run as two groups of 8 on four times the rows, so that the
+// rest is not padding.
 constexpr int kSC = 4;           // input channels per stage
 constexpr int kSX = 32;          // pixels of a block along x
 constexpr int kSPitch = 36;
@@ -445,7 +446,13 @@ mrs_status simt_conv3x3(const float* x, int cin, int xs, const float* wp, const 
                         const float* lrhs, int N, int H, int W, int s, cudaStream_t st)
 {
     const bool vec = (cin & 3) == 0 && (xs & 3) == 0 && ((uintptr_t)x & 15) == 0;
-    const int cop = simt_cop(cout), og = cout > 16 ? 8 : 2, rows = 32 / og;
+    // Groups of 16 outputs up to 16, and up to 32 where groups of 64, half of them
+    // padding, would take more than a block an SM (a block of either takes as long, but
+    // the higher tile's first stage takes longer): 64 -> 32 channels at 1024^2 1318 ->
+    // 813 us, 144^2 (180 blocks) 102 -> 91, 128^2 (128 blocks) 79 as 64 and 91 as 16
+    const int cop = simt_cop(cout);
+    const long long blocks = (long long)((W + kSX - 1) / kSX) * ((H + 3) / 4) * N;
+    const int og = cout > 32 || (cout > 16 && (blocks <= sm_count() || N > 32767)) ? 8 : 2, rows = 32 / og;   // grid.y
     const dim3 grid((unsigned)((W + kSX - 1) / kSX) * (unsigned)((H + rows - 1) / rows), N * ((cout + 8 * og - 1) / (8 * og)));
     auto launch = [&](auto kernel) {
         kernel<<<grid, 128, 0, st>>>(x, cin, xs, wp, cop, b, cout, mode, relu, res, rs, out, os, lrhs, H, W, s);
