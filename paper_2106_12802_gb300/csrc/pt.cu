@@ -164,7 +164,15 @@ __device__ __forceinline__ bool slab(float cx, float cy, float cz, float hx, flo
 // with which the slab test of any box stays finite, for coordinates up to 1e20
 constexpr float kTinyDir = 1e-18f;
 __device__ __forceinline__ bool has_tiny(V3 d) { return fminf(fminf(fabsf(d.x), fabsf(d.y)), fabsf(d.z)) < kTinyDir; }
-__device__ __noinline__ V3 reciprocal(V3 d) { return mk(1.0f / d.x, 1.0f / d.y, 1.0f / d.z); }
+// 1 / d, given the reciprocals of the components that are not tiny
+__device__ __forceinline__ float reciprocal(float d, float inv)
+{
+    return d == 0.0f ? copysignf(INFINITY, d) : fabsf(d) < kTinyDir ? 1.0f / d : inv;
+}
+__device__ __noinline__ V3 reciprocal(V3 d, V3 inv)
+{
+    return mk(reciprocal(d.x, inv.x), reciprocal(d.y, inv.y), reciprocal(d.z, inv.z));
+}
 
 // inv = 1 / d for the slab test where some component of d is zero or so small that
 // (c - o) inv could be infinite in the tree: a centre's infinite distance less or
@@ -176,12 +184,13 @@ __device__ __noinline__ V3 reciprocal(V3 d) { return mk(1.0f / d.x, 1.0f / d.y, 
 __device__ __noinline__ V3 reciprocal_tiny(const float4* __restrict__ nodes, V3 o, V3 d, V3 inv)
 {
     const float4 a = __ldg(nodes), b = __ldg(nodes + 1), c = __ldg(nodes + 2);
-    const float mx = 1e38f / fmaxf(fmaxf(fabsf(a.x - o.x) + b.z, fabsf(a.y - o.x) + b.w), 1.0f);
-    const float my = 1e38f / fmaxf(fmaxf(fabsf(a.z - o.y) + c.x, fabsf(a.w - o.y) + c.y), 1.0f);
-    const float mz = 1e38f / fmaxf(fmaxf(fabsf(b.x - o.z) + c.z, fabsf(b.y - o.z) + c.w), 1.0f);
-    if (fabsf(inv.x) > mx) inv.x = copysignf(mx, d.x);
-    if (fabsf(inv.y) > my) inv.y = copysignf(my, d.y);
-    if (fabsf(inv.z) > mz) inv.z = copysignf(mz, d.z);
+    const float mx = fmaxf(fabsf(a.x - o.x) + b.z, fabsf(a.y - o.x) + b.w);
+    const float my = fmaxf(fabsf(a.z - o.y) + c.x, fabsf(a.w - o.y) + c.y);
+    const float mz = fmaxf(fabsf(b.x - o.z) + c.z, fabsf(b.y - o.z) + c.w);
+    const float most = 1e38f / fmaxf(fmaxf(mx, my), fmaxf(mz, 1.0f));
+    if (fabsf(inv.x) > most) inv.x = copysignf(most, d.x);
+    if (fabsf(inv.y) > most) inv.y = copysignf(most, d.y);
+    if (fabsf(inv.z) > most) inv.z = copysignf(most, d.z);
     return inv;
 }
 
@@ -194,7 +203,7 @@ __device__ __forceinline__ bool in_leaf_box(const float* __restrict__ box, V3 o,
 {
     const float2* p = (const float2*)box;
     const float2 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);   // lo.xy | lo.z hi.x | hi.yz
-    if (has_tiny(d)) inv = reciprocal(d);
+    if (has_tiny(d)) inv = reciprocal(d, inv);
     const float t0x = (a.x - o.x) * inv.x, t1x = (b.y - o.x) * inv.x;
     const float t0y = (a.y - o.y) * inv.y, t1y = (c.x - o.y) * inv.y;
     const float t0z = (b.x - o.z) * inv.z, t1z = (c.y - o.z) * inv.z;
