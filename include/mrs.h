@@ -477,6 +477,11 @@ mrs_status mrs_fuse_extra(mrs_net net, const float* lrhs, const float* hrls, con
  * the tensor cores with BF16 activations and activation gradients, FP32
  * accumulation, FP32 dW / db reductions and FP32 master weights.  loss_out (HOST, may be NULL) receives
  * the loss before the update; when non-NULL the call synchronises `stream`.
+ * The workspace (FP32: about 4.9 KB per pixel plus 10 MB; BF16, which keeps every
+ * layer's gradient for its weight gradients: about 4.7 KB per pixel plus 22 MB) lives
+ * in the net handle.  A step without loss_out can be recorded in a CUDA graph
+ * once a step of its size has run; its replays update the weights with the bias
+ * correction of the step that was recorded.
  * Limit: N*H*W <= 2^22 pixels. */
 mrs_status mrs_train_step(mrs_net net, const float* lrhs, const float* hrls, const float* albedo,
                           const float* normal, const float* target, int32_t N, int32_t H,
@@ -707,8 +712,9 @@ mrs_status mrs_rdn_check(mrs_rdn rdn);
  * MRS_ERR_TIMEOUT if a BF16 step's tensor-core wait gave up).  The first step
  * allocates the gradient and Adam moments (3 x n_params floats, moments
  * zero); the workspace (FP32: about 20 KB per LR pixel plus 1.3 KB per HR
- * pixel; BF16: about 19 KB per LR pixel plus 1 KB per HR pixel) lives in
- * the handle.  A later MRS_PREC_BF16 mrs_rdn_fuse repacks its BF16 weights
+ * pixel; BF16: about 19 KB per LR pixel plus 1 KB per HR pixel, and 1.2 MB of
+ * partial sums for each 64 x 64 tile of the weight gradients: 191, 210 and 272
+ * MB at scale 2, 4 and 8 whatever the batch) lives in the handle.  A later MRS_PREC_BF16 mrs_rdn_fuse repacks its BF16 weights
  * from the updated FP32 ones.  A BF16 step copies the batch into the
  * handle's staging buffers; the first step of a shape (N, H, W, loss, beta)
  * runs its launches directly and records them as a CUDA graph that later

@@ -175,9 +175,9 @@ __global__ void k_input_q(const float* lrhs, const float* hrls, const float* alb
 // it is the FMA pipe (a packed FMA holds it two cycles).  The form before (4
 // pixels x 16 channels, scalar FMAs, 4-byte copies with the channel fastest)
 // was bound by shared-memory wavefronts (86%), a third of them bank conflicts:
-// the 21-channel network on 486 x 330 7.42 -> 3.80 ms (26 -> 51 TFLOP/s of the
+// the 21-channel network on 486 x 330 7.42 -> 3.75 ms (26 -> 52 TFLOP/s of the
 // 80.5 of 152 SMs x 128 lanes), the 35 convolutions of its training step at 6 x
-// 128^2 9.40 -> 5.13 ms.  Up to 16 outputs (the 3-channel heads; up to 32 on large
+// 128^2 9.40 -> 5.05 ms.  Up to 16 outputs (the 3-channel heads; up to 32 on large
 // images, see simt_conv3x3) run as two groups of 8 on four times the rows, so that the
 // rest is not padding.
 constexpr int kSC = 4;           // input channels per stage

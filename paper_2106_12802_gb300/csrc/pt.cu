@@ -1236,6 +1236,8 @@ SceneView view(const mrs_scene_s* S)
 // -> 0.55, 1.26 -> 0.97, 1.88 -> 1.60.  4 against 5 blocks: 434k paths 0.562 /
 // 0.600, 1.0M 1.003 / 0.991, 2.1M 1.791 / 1.716; 5 against 8: 2.1M 1.716 /
 // 1.690, 4.2M 3.22 / 3.10.  Bounce 0 against 1 at 4.2M: Cornell 3.92 / 3.81.
+// (The blocks' line belongs between 1.0M and 2.1M, the bounce's between 2.1M and 4.2M;
+// one line at the 2.1M serves both within 2%.)
 struct TailPlan {
     int bounce;   // first bounce in the tail kernel
     int blocks;   // blocks per SM of the instantiation
